@@ -22,8 +22,8 @@
 //
 // preprocess_bwd (Sec. 3.3): one thread per point; per view it chains the
 // screen-space adjoint {dpx, dpy, dq, do, dr, dg, db} (q = 1/s^2; the
-// compositing kernels leave dpx = q t0, dpy = q t1 and dq = -t2 / 2 to this
-// stage, which applies the factors once per point-view) through the
+// compositing kernels leave dpx = o q t0, dpy = o q t1 and dq = -o t2 / 2 to
+// this stage, which applies the factors once per point-view) through the
 // kernel width, the projection, the direction normalisation and the SH basis
 // back to the point position, SH coefficients and opacity.  Views are
 // visited in a fixed order, so the result does not depend on scheduling.
@@ -291,7 +291,7 @@ __device__ void pre_bwd_point(const Batch &b, const DevOpts &o, const DevScene &
     for (int j = 0; j < K * 3; ++j) dh[j] = 0.0f;
     const float P0 = __ldg(sc.pos + 3 * i), P1 = __ldg(sc.pos + 3 * i + 1),
                 P2 = __ldg(sc.pos + 3 * i + 2);
-    const float r = __ldg(sc.radius + i);
+    const float r = __ldg(sc.radius + i), op = __ldg(sc.opacity + i);
     float dP0 = 0.f, dP1 = 0.f, dP2 = 0.f, dop = 0.f;
 
     const int nv = sc.view_count;
@@ -323,7 +323,10 @@ __device__ void pre_bwd_point(const Batch &b, const DevOpts &o, const DevScene &
         const float s = o.radius_mode == 0 ? V.fx * r * iz : r * (float)min(V.W, V.H) * 0.5f;
         float q; // 1/s^2, approximate as well
         asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(q) : "f"(s * s));
-        const float gpx = ga.x * q, gpy = ga.y * q, gq = -0.5f * ga.z;
+        // the geometry terms lack the amplitude; a term of 0 stays 0 whatever it is
+        const float gpx = ga.x == 0.f ? 0.f : ga.x * op * q;
+        const float gpy = ga.y == 0.f ? 0.f : ga.y * op * q;
+        const float gq = ga.z == 0.f ? 0.f : -0.5f * op * ga.z;
         float dX0 = 0.f, dX1 = 0.f, dX2 = 0.f;
         // p = (fx X0/z + cx, fy X1/z + cy)
         dX0 += gpx * V.fx * iz;

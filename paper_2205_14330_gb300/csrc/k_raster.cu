@@ -14,12 +14,11 @@
 // behind the point, so
 //   dL/dc     = alpha T g
 //   dL/dalpha = T (c.g) - S / (1 - alpha)
-// and, below the alpha_max clamp,
-//   dL/do = dL/dalpha G,  dL/dp = dL/dalpha alpha q (u - p),
-//   dL/dq = -dL/dalpha alpha d2 / 2          (q = 1/s^2).
-// The kernels sum {ca (u - p), ca d2} with ca = dL/dalpha alpha, without
-// the per-point factors q and -1/2, which the point stage applies once per
-// point-view: the terms are {ca dx, ca dy, ca d2, do, dr, dg, db}.
+// and, below the alpha_max clamp, with dG = dL/dalpha G,
+//   dL/do = dG,  dL/dp = o dG q (u - p),  dL/dq = -o dG d2 / 2   (q = 1/s^2).
+// The kernels sum {dG (u - p), dG d2}, without the per-point factors o, q and
+// -1/2, which the point stage applies once per point-view: the terms are
+// {dG dx, dG dy, dG d2, do, dr, dg, db}.
 // The 7 per-point terms of a warp go to the per-(view, point) buffer with
 // 16-byte atomics: straight from each contributing lane when few lanes
 // contribute, else summed first with a transposed shuffle reduction (two
@@ -30,20 +29,37 @@
 // entries of its own block, and it skips those whose cutoff disc misses its
 // still active pixels.  Three schedules:
 //   - warp-streamed (batch depth 0, default): a block covers one TW x TH
-//     screen tile, each warp an 8 x 4 sub-block of it; every warp walks its
-//     entries by itself, 32 per step, culls them with one ballot and stops
-//     as soon as its own pixels have saturated.  No block barriers.
-//   - persistent (batch depth 0, persistent): one launch; warps take (tile,
-//     8 x 8 block) items longest list first from an atomic counter; a lane
-//     owns two pixels of a column, four rows apart, and their arithmetic
-//     runs packed (fp32x2).  The forward steps through each chunk's hits in
-//     lockstep; the backward forms the adjoint at both pixels per hit.
+//     screen tile, each warp an 8 x 8 block of it; a lane owns two pixels of
+//     a column, four rows apart.  Every warp walks its entries by itself, 32
+//     per step, culls them with one ballot, steps through the hits in
+//     lockstep and stops as soon as its own pixels have saturated.  No block
+//     barriers.
+//   - persistent (batch depth 0, persistent): the same walk in one launch;
+//     warps take (tile, 8 x 8 block) items longest list first from an atomic
+//     counter.
 //   - block-staged (batch depth > 0): the block stages `depth` records in
 //     shared memory and each warp culls the batch into its own list; block
 //     barriers between batches, per-block shared-memory gradient sums.
+// What bounds the walks: 92 M (8 x 8 block, hit) steps on the 1M-point,
+// 64-view batch, of whose 64 pixels 44 are still active and 17 include the
+// point.  The forward is bound by instruction issue (about 45 a step; one
+// pixel's weight, three colour sums and T are 6 of them), the backward by
+// issue (85 a step, 71% of the slots) and the L1 data path (82%) together: a
+// shared-memory read of 16 bytes a lane takes four cycles of that path even
+// when every lane reads the same address, and so do the atomics' operands.
+// So hits are staged compacted, the loops over them carry no bit scans and
+// are unrolled with the loads first, a point's own scalars stay scalar
+// operands (a packed operation would need them duplicated), the blend is
+// predicated per pixel instead of masked, and a chunk whose amplitudes are
+// all below the clamp skips the clamp.  Measured against lockstep loops over
+// hit masks (8 x 4 one-pixel warps in the streamed schedule), 1M points, 64
+// views, 16 x 32 tiles, persistent: forward 5.31 -> 4.09 ms, backward 9.34 ->
+// 8.84 ms; 500k points, 4 views of 800 x 800, 16 x 16 tiles, streamed: forward
+// 257 -> 188 us, backward 423 -> 363 us, in store mode 333 -> 304 us and 569 ->
+// 528 us; one 1920 x 1080 view of 1M points: forward 216 -> 151 us.
 // Store mode (STORE): the forward also keeps T before each of a pixel's
 // first store_depth composited points, and the backward reads it there
-// instead of dividing.
+// instead of dividing, each value one composited point ahead of its use.
 #include "pbr_internal.cuh"
 
 namespace pbr {
@@ -126,41 +142,10 @@ __device__ __forceinline__ bool disc_meets_rect(const float4 a, const PixelGeom 
     return __fadd_rn(__fmul_rn(ex, ex), __fmul_rn(ey, ey)) <= a.z;
 }
 
-// Whether the cutoff disc of a record holds every pixel centre of the
-// rectangle: the per-pixel fp32 test applied to the centre farthest from the
-// splat centre (per axis the edge with the larger rounded offset), which by
-// monotone rounding has the largest fp32 squared distance.
-__device__ __forceinline__ bool disc_covers_rect(const float4 a, const PixelGeom &g)
-{
-    const float lx = __fsub_rn(g.xl, a.x), hx = __fsub_rn(g.xh, a.x);
-    const float ly = __fsub_rn(g.yl, a.y), hy = __fsub_rn(g.yh, a.y);
-    const float ex = fabsf(lx) > fabsf(hx) ? lx : hx;
-    const float ey = fabsf(ly) > fabsf(hy) ? ly : hy;
-    return __fadd_rn(__fmul_rn(ex, ex), __fmul_rn(ey, ey)) <= a.z;
-}
-
-// The rectangle of pixel centres of the warp's lanes that are still
-// active (g's own rectangle when every lane is).  Warp-wide reductions: all
-// 32 lanes must call it together, outside any lane-dependent branch or
-// short-circuit.
-__device__ __forceinline__ PixelGeom active_rect(const PixelGeom &g, bool active)
-{
-    PixelGeom r = g;
-    const uint32_t x = (uint32_t)g.x, y = (uint32_t)g.y;
-    const uint32_t x0 = __reduce_min_sync(0xffffffffu, active ? x : 0xffffffffu);
-    const uint32_t x1 = __reduce_max_sync(0xffffffffu, active ? x : 0u);
-    const uint32_t y0 = __reduce_min_sync(0xffffffffu, active ? y : 0xffffffffu);
-    const uint32_t y1 = __reduce_max_sync(0xffffffffu, active ? y : 0u);
-    r.xl = (float)x0 + 0.5f;
-    r.xh = (float)x1 + 0.5f;
-    r.yl = (float)y0 + 0.5f;
-    r.yh = (float)y1 + 0.5f;
-    return r;
-}
-
-// active_rect for a warp that owns P pixels per lane, one column, rows 4
-// apart (g[q] below g[q-1]): the rectangle of the centres of its still
-// active pixels.  The same calling rule holds.
+// The rectangle of the centres of the still active pixels of a warp that
+// owns P pixels per lane, one column, rows 4 apart (g[q] below g[q-1]).
+// Warp-wide reductions: all 32 lanes must call it together, outside any
+// lane-dependent branch or short-circuit.
 template <int P>
 __device__ __forceinline__ PixelGeom active_rect_rows(const PixelGeom (&g)[P], const bool (&act)[P])
 {
@@ -344,7 +329,7 @@ __device__ __forceinline__ int queue_take(WarpQueue &q, int &qn, uint32_t &qh, i
 // it the exact cutoff decision).
 __device__ __forceinline__ float unfused1(float v)
 {
-    asm volatile("" : "+f"(v));
+    asm("" : "+f"(v));
     return v;
 }
 
@@ -372,40 +357,8 @@ __device__ __forceinline__ float rcp_approx(float x)
     return y;
 }
 
-// Branch-free adjoint for a warp-uniform loop: `take` (0 or 1) says whether
-// the point was composited at this pixel; with take = 0 every term is 0 and
-// T, S are unchanged.
-// With has_tb, tb is the stored transmittance before the point (store mode)
-// instead of the one recovered by division.
-__device__ __forceinline__ void pixel_adjoint_masked(float take, float d2, float dx, float dy,
-                                                     const float4 a, const float4 c, float amax,
-                                                     float g0, float g1, float g2, float &T,
-                                                     float &S, float v[8], bool has_tb = false,
-                                                     float tb = 0.0f)
-{
-    const float G = ex2_approx(d2 * a.w);
-    const float raw = c.x * G;
-    const float alpha = fminf(amax, raw) * take;
-    const float rom = rcp_approx(1.0f - alpha);
-    const float Tb = has_tb ? tb : T * rom;
-    const float wgt = alpha * Tb;
-    const float cg = c.y * g0 + c.z * g1 + c.w * g2;
-    v[4] = wgt * g0;
-    v[5] = wgt * g1;
-    v[6] = wgt * g2;
-    const float dalpha = (Tb * cg - S * rom) * take;
-    S = fmaf(wgt, cg, S);
-    T = Tb;
-    const float ca = raw < amax ? dalpha * alpha : 0.0f; // clamped: no geometry terms
-    v[0] = ca * dx;
-    v[1] = ca * dy;
-    v[2] = ca * d2;
-    v[3] = raw < amax ? dalpha * G : 0.0f;
-    v[7] = 0.0f;
-}
-
 // Per-pixel adjoint of one composited point (see the file comment).  On
-// return v[0..6] = {ca dx, ca dy, ca d2, do, dr, dg, db}; T and S are
+// return v[0..6] = {dG dx, dG dy, dG d2, do, dr, dg, db}; T and S are
 // updated.
 __device__ __forceinline__ void pixel_adjoint(float d2, float dx, float dy, const float4 a,
                                               const float4 c, float amax, float g0, float g1,
@@ -425,11 +378,11 @@ __device__ __forceinline__ void pixel_adjoint(float d2, float dx, float dy, cons
     S = fmaf(wgt, cg, S);
     T = Tb;
     if (raw < amax) {
-        const float ca = dalpha * alpha;
-        v[0] = ca * dx;
-        v[1] = ca * dy;
-        v[2] = ca * d2;
-        v[3] = dalpha * G;
+        const float dG = dalpha * G;
+        v[0] = dG * dx;
+        v[1] = dG * dy;
+        v[2] = dG * d2;
+        v[3] = dG;
     }
 }
 
@@ -450,7 +403,36 @@ __device__ __forceinline__ int64_t pixel_index(const PixelGeom &g)
 // Store mode: T before the cnt-th composited point of pixel pix.
 __device__ __forceinline__ void store_T(const StoreBuf &sto, int64_t pix, uint32_t cnt, float T)
 {
-    if (sto.T && cnt < (uint32_t)sto.depth) sto.T[pix * sto.depth + cnt] = T;
+    if (cnt < (uint32_t)sto.depth) sto.T[pix * sto.depth + cnt] = T;
+}
+
+// Store mode, backward: one pixel's list read back to front, each value
+// fetched one composited point ahead of its use.
+struct StoreRow {
+    const float *p;
+    uint32_t k, depth; // composited points not yet visited
+    float nxt;         // T before point k - 1 (when k - 1 < depth)
+};
+
+__device__ __forceinline__ StoreRow store_row(const StoreBuf &sto, int64_t pix, bool inside)
+{
+    StoreRow r;
+    r.p = sto.T + pix * sto.depth;
+    r.depth = (uint32_t)sto.depth;
+    r.k = inside ? sto.n[pix] : 0u;
+    r.nxt = r.k > 0 && r.k <= r.depth ? r.p[r.k - 1] : 0.0f;
+    return r;
+}
+
+// Visits the pixel's next composited point if `take`: whether its T was
+// stored, and T.
+__device__ __forceinline__ bool row_next(StoreRow &r, bool take, float &T)
+{
+    const bool has = take && r.k <= r.depth;
+    T = r.nxt;
+    r.k -= take;
+    if (take && r.k - 1u < r.depth) r.nxt = r.p[r.k - 1u];
+    return has;
 }
 
 __device__ __forceinline__ void write_pixel(const PixelGeom &g, const DevOpts &o, float T,
@@ -480,88 +462,6 @@ __device__ __forceinline__ void add_stats(unsigned long long *stats, uint32_t a,
     }
 }
 
-// ======================================================= warp-streamed
-// One warp composites its 8 x 4 sub-block of a tile.  Each step takes 32
-// entries of the warp's 8 x 8 block from its queue, culls them against the
-// warp's rectangle with one ballot and stages the hits in the warp's shared
-// buffer; then
-//   phase 1 (warp-uniform): for every hit, every lane runs its exact fp32
-//            cutoff test and records the hit in its own bitmask;
-//   phase 2 (per lane): each lane walks only its own included entries.
-// wbuf: this warp's 64 float4 (a-parts, then b-parts of the chunk).
-// g: the lane's pixel and the warp's rectangle; [s, e): the tile's list.
-template <bool STATS, bool STORE>
-__device__ __forceinline__ void fwd_stream_item(const PixelGeom &g, uint32_t s, uint32_t e,
-                                                uint32_t bit, const DevOpts &o, int lane,
-                                                const uint32_t *__restrict__ keys,
-                                                const uint32_t *__restrict__ pv_list,
-                                                const float4 *__restrict__ rec,
-                                                float *__restrict__ out_rgb,
-                                                float *__restrict__ T_final,
-                                                uint32_t *__restrict__ n_contrib,
-                                                uint32_t &examined_acc, uint32_t &composited_acc,
-                                                float4 *wbuf, uint32_t *wpos, WarpQueue &q,
-                                                const StoreBuf &sto)
-{
-    float T = 1.0f, C0 = 0.f, C1 = 0.f, C2 = 0.f;
-    uint32_t cnt = 0, last = 0, examined = 0;
-    bool done = !g.inside;
-    const int64_t pix = STORE && g.inside ? pixel_index(g) : 0;
-    uint32_t p = s;
-    int qn = 0;
-    uint32_t qh = 0;
-    while (!__all_sync(0xffffffffu, done)) {
-        queue_fill_front(keys, pv_list, s, e, bit, p, qn, qh, q, lane);
-        if (qn == 0) break;
-        uint32_t rel = 0, pv = 0;
-        const int take = queue_take(q, qn, qh, lane, rel, pv);
-        const bool valid = lane < take;
-        float4 a = make_float4(0.f, 0.f, -1.f, 0.f);
-        if (valid) a = __ldg(rec + 2 * (size_t)pv);
-        // every lane takes part in the reductions, whatever its entry
-        const PixelGeom ar = active_rect(g, !done);
-        const bool hit = valid && disc_meets_rect(a, ar);
-        const bool covers = hit && disc_covers_rect(a, ar);
-        uint32_t m = __ballot_sync(0xffffffffu, hit);
-        // entries whose disc holds every active pixel need no per-pixel test
-        uint32_t mine = __ballot_sync(0xffffffffu, covers);
-        if (hit) {
-            wbuf[lane] = a;
-            wbuf[32 + lane] = __ldg(rec + 2 * (size_t)pv + 1);
-            wpos[lane] = rel;
-        }
-        __syncwarp();
-        if (STATS && !done) examined += (uint32_t)__popc(m);
-        m &= ~mine;
-        while (m) {
-            const int j = __ffs(m) - 1;
-            m &= m - 1;
-            const float4 aj = wbuf[j];
-            float dx, dy;
-            if (pixel_d2(g.ux, g.uy, aj.x, aj.y, dx, dy) <= aj.z) mine |= 1u << j;
-        }
-        if (done) mine = 0;
-        while (mine) {
-            const int j = __ffs(mine) - 1;
-            mine &= mine - 1;
-            const float4 aj = wbuf[j];
-            float dx, dy;
-            const float d2 = pixel_d2(g.ux, g.uy, aj.x, aj.y, dx, dy);
-            last = wpos[j] + 1;
-            if (STORE) store_T(sto, pix, cnt, T);
-            if (pixel_blend(d2, aj, wbuf[32 + j], o, T, C0, C1, C2, cnt)) {
-                done = true;
-                break;
-            }
-        }
-        __syncwarp(); // chunk consumed before the buffers are refilled
-    }
-    examined_acc += examined;
-    composited_acc += cnt;
-    if (STORE && g.inside) sto.n[pix] = cnt;
-    write_pixel(g, o, T, C0, C1, C2, last, out_rgb, T_final, n_contrib);
-}
-
 // ------------------------------------------------- packed two-pixel math
 // A lane of the 8 x 8-pixel warps owns two pixels of one column, rows 4
 // apart (A above B); their per-point arithmetic runs in packed fp32x2
@@ -571,42 +471,44 @@ __device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a
 __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 
-// Keeps the compiler from fusing the product that produced v into a later
-// packed add (it merges a product feeding a packed add into one packed FMA,
-// even across __fmul_rn, which changes the rounding of a distance and with it
-// the exact cutoff decision).
-__device__ __forceinline__ float2 unfused(float2 v)
-{
-    unsigned long long r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(v.x), "f"(v.y));
-    asm volatile("" : "+l"(r));
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(v.x), "=f"(v.y) : "l"(r));
-    return v;
-}
-
 // Squared fp32 distances from the lane's two pixel centres (ux, uy.x) and
-// (ux, uy.y) to the splat centre, with the rounding of pixel_d2: dx =
-// ux - px (shared), dy = uy - py, d2 = dx dx + dy dy, each operation rounded
-// to nearest (no contraction).
+// (ux, uy.y) to the splat centre: dx = ux - px (shared), dy = uy - py, d2 =
+// dx dx + dy dy.  FUSED 0 (streamed): each operation rounded to nearest, as
+// in pixel_d2.  FUSED 1 (persistent): dy dy + dx dx rounded once.  Each
+// schedule keeps its own rounding, forward and backward alike: whether a
+// pixel on the edge of a disc includes the point can turn on the last bit.
+template <bool FUSED>
 __device__ __forceinline__ float2 pair_d2(float ux, float2 uy, float px, float py, float &dx,
                                           float2 &dy)
 {
     dx = __fsub_rn(ux, px);
-    dy = add2(uy, f2(-py));
+    dy = make_float2(__fsub_rn(uy.x, py), __fsub_rn(uy.y, py));
     const float dx2 = __fmul_rn(dx, dx);
-    return add2(unfused(f2(dx2)), unfused(mul2(dy, dy)));
+    if (FUSED) return make_float2(__fmaf_rn(dy.x, dy.x, dx2), __fmaf_rn(dy.y, dy.y, dx2));
+    const float2 dy2 = mul2(dy, dy); // the sums are scalar: no packed add to fuse it into
+    return make_float2(__fadd_rn(dx2, dy2.x), __fadd_rn(dx2, dy2.y));
 }
 
-// Forward of one 8 x 8 block by one warp, for the persistent schedule:
-// lane l owns the pixels (l & 7, l >> 3) and (l & 7, 4 + (l >> 3)), gA and
-// gB.  The warp takes the tile list's entries with its block's bit (`bit`)
-// 32 at a time from its queue, culls them against the rectangle of its
-// active pixels and stages the hits; then it steps through the hits in list
-// order, every lane testing and blending the point at both of its pixels at
-// once (packed fp32x2, .x pixel A, .y pixel B), with the blend of a pixel
-// the point does not include (or that has stopped) masked to zero weight.
-// Each pixel's blend sequence and roundings are the one-pixel walk's.
-template <bool STATS, bool STORE>
+// One warp's shared memory of the forward.
+struct FwdWarp {
+    float4 a[32], c[32]; // the chunk's hits: record halves
+    uint32_t pos[32];    // and their list positions
+    WarpQueue q;
+};
+
+// Forward of one 8 x 8 block by one warp: lane l owns the pixels (l & 7, l >>
+// 3) and (l & 7, 4 + (l >> 3)), gA and gB.  The warp takes the tile list's
+// entries with its block's bit (`bit`) 32 at a time from its queue, culls
+// them against the rectangle of its active pixels and stages the hits in list
+// order; then it steps through them, every lane testing and blending the
+// point at both of its pixels; the blend of a pixel the point does not
+// include (or that has stopped) is predicated off.  Each pixel's blend
+// sequence and roundings are the one-pixel walk's.
+// A pixel is active while its T is at least t_eps (-1 outside the image).
+// COUNT: the points composited per pixel are counted (pair counts, store
+// mode, the count cap).
+// FUSED: the rounding of the squared distance (pair_d2).
+template <bool COUNT, bool STORE, bool FUSED>
 __device__ __forceinline__ void fwd_pair_item(const PixelGeom &gA, const PixelGeom &gB,
                                               uint32_t s, uint32_t e, uint32_t bit,
                                               const DevOpts &o, int lane,
@@ -617,92 +519,96 @@ __device__ __forceinline__ void fwd_pair_item(const PixelGeom &gA, const PixelGe
                                               float *__restrict__ T_final,
                                               uint32_t *__restrict__ n_contrib,
                                               uint32_t &examined_acc, uint32_t &composited_acc,
-                                              float4 *wbuf, uint32_t *wpos, WarpQueue &q,
-                                              const StoreBuf &sto)
+                                              FwdWarp &m, const StoreBuf &sto)
 {
     const int64_t pixA = STORE && gA.inside ? pixel_index(gA) : 0;
     const int64_t pixB = STORE && gB.inside ? pixel_index(gB) : 0;
-    float2 T = f2(1.0f), C0 = f2(0.0f), C1 = f2(0.0f), C2 = f2(0.0f);
+    float2 T = make_float2(gA.inside ? 1.0f : -1.0f, gB.inside ? 1.0f : -1.0f);
+    float2 C0 = f2(0.0f), C1 = f2(0.0f), C2 = f2(0.0f);
     uint32_t cntA = 0, cntB = 0, lastA = 0, lastB = 0, examined = 0;
-    bool doneA = !gA.inside, doneB = !gB.inside;
     const PixelGeom g2[2] = {gA, gB};
-    const float2 uy2 = make_float2(gA.uy, gB.uy);
-    const uint32_t cmax = (uint32_t)o.max_per_pixel;
+    const float ux = gA.ux;
+    const float2 uy = make_float2(gA.uy, gB.uy);
+    const float eps = o.t_eps, amax = o.alpha_max;
+    // pixels that reached the count cap
+    const uint32_t cmax = COUNT && o.max_per_pixel ? (uint32_t)o.max_per_pixel : 0xffffffffu;
+    const uint32_t lt = lanemask_lt_r();
     uint32_t p = s;
     int qn = 0;
     uint32_t qh = 0;
-    while (!__all_sync(0xffffffffu, doneA && doneB)) {
-        queue_fill_front(keys, pv_list, s, e, bit, p, qn, qh, q, lane);
+    while (true) {
+        const bool act[2] = {T.x >= eps && cntA < cmax, T.y >= eps && cntB < cmax};
+        if (!__any_sync(0xffffffffu, act[0] || act[1])) break;
+        queue_fill_front(keys, pv_list, s, e, bit, p, qn, qh, m.q, lane);
         if (qn == 0) break;
         uint32_t rel = 0, pv = 0;
-        const int take = queue_take(q, qn, qh, lane, rel, pv);
+        const int take = queue_take(m.q, qn, qh, lane, rel, pv);
         const bool valid = lane < take;
-        float4 a = make_float4(0.f, 0.f, -1.f, 0.f);
-        if (valid) a = __ldg(rec + 2 * (size_t)pv);
+        float4 a = make_float4(0.f, 0.f, -1.f, 0.f), c = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (valid) {
+            a = __ldg(rec + 2 * (size_t)pv);
+            c = __ldg(rec + 2 * (size_t)pv + 1);
+        }
         // every lane takes part in the reductions, whatever its entry
-        const bool act[2] = {!doneA, !doneB};
         const PixelGeom ar = active_rect_rows<2>(g2, act);
         const bool hit = valid && disc_meets_rect(a, ar);
-        uint32_t m = __ballot_sync(0xffffffffu, hit);
-        if (hit) {
-            wbuf[lane] = a;
-            wbuf[32 + lane] = __ldg(rec + 2 * (size_t)pv + 1);
-            wpos[lane] = rel;
-        }
+        const uint32_t hm = __ballot_sync(0xffffffffu, hit);
+        const int nh = __popc(hm);
+        // the slots behind the hits are filled with points no pixel includes
+        const int slot = hit ? __popc(hm & lt) : nh + __popc(~hm & lt);
+        m.a[slot] = hit ? a : make_float4(0.f, 0.f, -1.f, 0.f);
+        m.c[slot] = hit ? c : make_float4(0.f, 0.f, 0.f, 0.f);
+        m.pos[slot] = rel;
         __syncwarp();
-        if (STATS) examined += (uint32_t)__popc(m) * ((uint32_t)!doneA + (uint32_t)!doneB);
-        // the chunk's composited entries of each pixel, as bits of the chunk
-        // (counts and the last position follow after the chunk)
-        uint32_t incA = 0u, incB = 0u;
-        while (m) {
-            const int j = __ffs(m) - 1;
-            m &= m - 1;
-            const float4 aj = wbuf[j];
-            float dx;
-            float2 dy;
-            const float2 d2 = pair_d2(gA.ux, uy2, aj.x, aj.y, dx, dy);
-            const bool inA = !doneA && d2.x <= aj.z, inB = !doneB && d2.y <= aj.z;
-            if (!__any_sync(0xffffffffu, inA || inB)) continue;
-            const float4 cj = wbuf[32 + j];
-            const float2 ea = mul2(d2, f2(aj.w));
-            const float2 raw = mul2(f2(cj.x), make_float2(ex2_approx(ea.x), ex2_approx(ea.y)));
-            const float2 alpha = make_float2(inA ? fminf(o.alpha_max, raw.x) : 0.0f,
-                                             inB ? fminf(o.alpha_max, raw.y) : 0.0f);
-            if (STORE) {
-                if (inA) store_T(sto, pixA, cntA + __popc(incA), T.x);
-                if (inB) store_T(sto, pixB, cntB + __popc(incB), T.y);
-            }
-            const float2 wgt = mul2(alpha, T);
-            C0 = fma2(wgt, f2(cj.y), C0);
-            C1 = fma2(wgt, f2(cj.z), C1);
-            C2 = fma2(wgt, f2(cj.w), C2);
-            T = add2(T, make_float2(-wgt.x, -wgt.y));
-            const uint32_t bit_j = 1u << j;
-            if (inA) {
-                incA |= bit_j;
-                doneA = T.x < o.t_eps;
-            }
-            if (inB) {
-                incB |= bit_j;
-                doneB = T.y < o.t_eps;
-            }
-            if (cmax) { // count cap (warp-uniform branch)
-                doneA = doneA || (inA && cntA + __popc(incA) == cmax);
-                doneB = doneB || (inB && cntB + __popc(incB) == cmax);
+        if (COUNT) examined += (uint32_t)nh * ((uint32_t)act[0] + (uint32_t)act[1]);
+        // the chunk's last composited hit of each pixel
+        int jA = -1, jB = -1;
+        constexpr int FWD_UNROLL = STORE ? 2 : 4;
+        for (int j0 = 0; j0 < nh; j0 += FWD_UNROLL) {
+#pragma unroll
+            for (int u = 0; u < FWD_UNROLL; ++u) {
+                const float4 aj = m.a[j0 + u], cj = m.c[j0 + u];
+                float dx;
+                float2 dy;
+                const float2 d2 = pair_d2<FUSED>(ux, uy, aj.x, aj.y, dx, dy);
+                bool inA = d2.x <= aj.z && T.x >= eps, inB = d2.y <= aj.z && T.y >= eps;
+                if (COUNT) {
+                    inA = inA && cntA < cmax;
+                    inB = inB && cntB < cmax;
+                }
+                const float rawA = __fmul_rn(cj.x, ex2_approx(__fmul_rn(d2.x, aj.w)));
+                const float rawB = __fmul_rn(cj.x, ex2_approx(__fmul_rn(d2.y, aj.w)));
+                if (STORE) {
+                    if (inA) store_T(sto, pixA, cntA, T.x);
+                    if (inB) store_T(sto, pixB, cntB, T.y);
+                }
+                const float2 wgt = mul2(make_float2(fminf(amax, rawA), fminf(amax, rawB)), T);
+                if (inA) {
+                    C0.x = fmaf(wgt.x, cj.y, C0.x);
+                    C1.x = fmaf(wgt.x, cj.z, C1.x);
+                    C2.x = fmaf(wgt.x, cj.w, C2.x);
+                    T.x = __fsub_rn(T.x, wgt.x);
+                    jA = j0 + u;
+                    if (COUNT) ++cntA;
+                }
+                if (inB) {
+                    C0.y = fmaf(wgt.y, cj.y, C0.y);
+                    C1.y = fmaf(wgt.y, cj.z, C1.y);
+                    C2.y = fmaf(wgt.y, cj.w, C2.y);
+                    T.y = __fsub_rn(T.y, wgt.y);
+                    jB = j0 + u;
+                    if (COUNT) ++cntB;
+                }
             }
         }
-        if (incA) {
-            cntA += __popc(incA);
-            lastA = wpos[31 - __clz(incA)] + 1;
-        }
-        if (incB) {
-            cntB += __popc(incB);
-            lastB = wpos[31 - __clz(incB)] + 1;
-        }
+        if (jA >= 0) lastA = m.pos[jA] + 1;
+        if (jB >= 0) lastB = m.pos[jB] + 1;
         __syncwarp(); // chunk consumed before the buffers are refilled
     }
-    examined_acc += examined;
-    composited_acc += cntA + cntB;
+    if (COUNT) {
+        examined_acc += examined;
+        composited_acc += cntA + cntB;
+    }
     if (STORE) {
         if (gA.inside) sto.n[pixA] = cntA;
         if (gB.inside) sto.n[pixB] = cntB;
@@ -711,114 +617,25 @@ __device__ __forceinline__ void fwd_pair_item(const PixelGeom &gA, const PixelGe
     write_pixel(gB, o, T.y, C0.y, C1.y, C2.y, lastB, out_rgb, T_final, n_contrib);
 }
 
-// Up to this many contributing pixels of a warp add their terms with their
-// own vector atomics; more go through the transposed warp reduction.  The
-// reduction costs some 35 instructions whatever the count, the atomics
-// cost L2 throughput per pixel; measured on the batched 1M-point
-// workload, the backward runs fastest between 12 and 16 (13.0 ms against
-// 14.8 ms with the reduction for 2 or more and 22 ms with atomics only).
-constexpr int BWD_DIRECT_MAX = 16;
-// The same for the two-pixels-per-lane backward, whose lanes add the terms
-// of both their pixels: fastest at 20-24 (11.1 ms; 11.4 ms at 16, 11.9 ms
-// at 8, 15.8 ms with atomics only on the same workload; re-measured on a
-// later version: 10.13 ms at 24, 10.14 at 20, 10.61 at 28 and 11.39 with
-// the reduction for every point).
-constexpr int BWD_PAIR_DIRECT_MAX = 24;
-// The persistent backward runs 8 x 8-pixel warps (two pixels per lane):
-// 8 x 16 (four pixels per lane) examined 41% more pairs through the coarser
-// cull and needed 80 registers (13.4 ms against 11.1).
+// ------------------------------------------------------------- backward
+// Up to this many lanes with a contributing pixel add their terms (the sums
+// over both their pixels) with their own vector atomics; more go through the
+// transposed warp reduction, which costs some 35 instructions whatever the
+// count, where the atomics cost L1 and L2 throughput per lane.  On the
+// 1M-point, 64-view batch an earlier form of the loop took 10.13 ms at 24,
+// 10.14 at 20, 10.61 at 28, 11.39 with the reduction for every point.
+// Summing a batch of 8 or 16 hits at once instead (recursion terms to shared
+// memory, then one lane per hit and column group) needed two atomics a hit
+// and no reduction, but its shared-memory traffic made the L1 path the bound:
+// 8.84-9.3 ms against 8.87.
+constexpr int BWD_DIRECT_MAX = 24;
 
-// One warp back-propagates through sub-block `sub` of tile `tile`, taking
-// the entries of its 8 x 8 block (`bit`) from its queue, back to front.
-template <int TW, int TH, bool STORE>
-__device__ __forceinline__ void bwd_stream_item(const Batch &b, const DevOpts &o, uint32_t tile,
-                                                int sub, uint32_t bit, int lane,
-                                                const uint2 *__restrict__ ranges,
-                                                const uint32_t *__restrict__ keys,
-                                                const uint32_t *__restrict__ pv_list,
-                                                const float4 *__restrict__ rec,
-                                                const float *__restrict__ T_final,
-                                                const uint32_t *__restrict__ n_contrib,
-                                                const float *__restrict__ grad_rgb,
-                                                float *__restrict__ g2d, uint32_t &examined,
-                                                uint32_t &used, float4 *wbuf, uint32_t *wpv,
-                                                uint32_t *wpos, WarpQueue &q, const StoreBuf &sto)
-{
-    const PixelGeom g = pixel_geom<TW, TH>(b, tile, sub, lane);
-    const uint32_t s = ranges[tile].x;
-    float T = 1.0f, g0 = 0.f, g1 = 0.f, g2 = 0.f;
-    uint32_t L = 0, k = 0; // k: composited points not yet visited (store mode)
-    int64_t pix = 0;
-    if (g.inside) {
-        pix = g.V->pix_base + (int64_t)g.y * g.V->W + g.x;
-        if (STORE) k = sto.n[pix];
-        T = T_final[pix];
-        L = n_contrib[pix];
-        g0 = grad_rgb[3 * pix];
-        g1 = grad_rgb[3 * pix + 1];
-        g2 = grad_rgb[3 * pix + 2];
-    }
-    float S = T * (o.bg[0] * g0 + o.bg[1] * g1 + o.bg[2] * g2);
-    const uint32_t wmax = __reduce_max_sync(0xffffffffu, L);
-    if (wmax == 0) return;
-    int64_t c = (int64_t)((wmax - 1) & ~31u);
-    int qn = 0;
-    uint32_t qh = 0;
-    while (true) {
-        queue_fill_back(keys, pv_list, s, wmax, bit, c, qn, qh, q, lane);
-        if (qn == 0) break;
-        uint32_t rel = 0, pv = 0;
-        const int take = queue_take(q, qn, qh, lane, rel, pv);
-        const bool valid = lane < take;
-        float4 a = make_float4(0.f, 0.f, -1.f, 0.f);
-        if (valid) a = __ldg(rec + 2 * (size_t)pv);
-        // lanes whose composited list reaches the chunk's nearest entry; every
-        // lane takes part in the reductions, whatever its entry
-        const uint32_t lowest = __shfl_sync(0xffffffffu, rel, take - 1);
-        const PixelGeom ar = active_rect(g, L > lowest);
-        const bool hit = valid && disc_meets_rect(a, ar);
-        uint32_t m = __ballot_sync(0xffffffffu, hit);
-        if (hit) {
-            wbuf[lane] = a;
-            wbuf[32 + lane] = __ldg(rec + 2 * (size_t)pv + 1);
-            wpv[lane] = pv;
-            wpos[lane] = rel;
-        }
-        __syncwarp();
-        while (m) {
-            const int j = __ffs(m) - 1; // back to front: queue order
-            m &= m - 1;
-            const float4 aj = wbuf[j];
-            const float4 cj = wbuf[32 + j];
-            const bool before = wpos[j] < L;
-            float dx, dy;
-            const float d2 = pixel_d2(g.ux, g.uy, aj.x, aj.y, dx, dy);
-            const bool contrib = before && d2 <= aj.z;
-            examined += before;
-            used += contrib;
-            const uint32_t cm = __ballot_sync(0xffffffffu, contrib);
-            if (cm) {
-                float v[8];
-                bool has_tb = false;
-                float tb = 0.0f;
-                if (STORE && contrib && --k < (uint32_t)sto.depth) {
-                    has_tb = true;
-                    tb = sto.T[pix * sto.depth + k];
-                }
-                pixel_adjoint_masked(contrib ? 1.0f : 0.0f, d2, dx, dy, aj, cj, o.alpha_max, g0,
-                                     g1, g2, T, S, v, has_tb, tb);
-                if (__popc(cm) > BWD_DIRECT_MAX) {
-                    warp_add_terms(v, lane, g2d, wpv[j]);
-                } else if (contrib) { // few pixels: each adds its own terms
-                    float4 *dst = reinterpret_cast<float4 *>(g2d) + 2 * (size_t)wpv[j];
-                    atomicAdd(dst, make_float4(v[0], v[1], v[2], v[3]));
-                    atomicAdd(dst + 1, make_float4(v[4], v[5], v[6], 0.f));
-                }
-            }
-        }
-        __syncwarp(); // chunk consumed before the buffers are refilled
-    }
-}
+// One warp's shared memory of the backward.
+struct BwdWarp {
+    float4 a[32], c[32]; // the chunk's hits: record halves
+    uint2 ip[32];        // their list positions and point-views
+    WarpQueue q;
+};
 
 // Adjoint state of one pixel: T after its last composited point, the colour
 // behind (S, starting from the background term), dL/dC and the list length.
@@ -851,60 +668,144 @@ struct BwdPair {
     uint32_t LA, LB;
 };
 
-// The adjoint of one composited point at both pixels of a lane (the
-// operations of pixel_adjoint_masked, packed): take.x / take.y (0 or 1) say
-// whether the point was composited at pixel A / B (0: its terms are 0 and
-// T, S stay).  Returns the sum over the two pixels of the terms {ca dx,
-// ca dy, ca d2, do, dr, dg, db} in v[0..6].
-// Bit 0 / 1 of has_tb: tb.x / .y is the stored transmittance before the
-// point at pixel A / B (store mode) instead of the one recovered by
-// division.
-__device__ __forceinline__ void pair_adjoint(float2 take, float2 d2, float dx, float2 dy,
-                                             const float4 a, const float4 c, float amax,
-                                             BwdPair &p, float v[8], uint32_t has_tb = 0u,
-                                             float2 tb = {0.0f, 0.0f})
+// What a point contributes to the recursions of a lane's two pixels before T
+// and S enter: alpha, G and 1 / (1 - alpha) (0, 0 and 1 where the point was
+// not composited; G 0 also where alpha is clamped, which has no geometry
+// terms), and c.g.
+struct PairAlpha {
+    float2 alpha, G, rom, cg;
+};
+
+// tA, tB: whether the point was composited at the lane's pixels; d2: its
+// squared distances.  CLAMP 0: the point's amplitude is below the clamp, so
+// alpha is too.  Operands that are the point's own stay scalar (a packed
+// operation would need them duplicated).
+template <bool CLAMP>
+__device__ __forceinline__ PairAlpha pair_alpha(bool tA, bool tB, float2 d2, const float4 a,
+                                                const float4 c, float amax, const BwdPair &p)
 {
-    const float2 e = mul2(d2, f2(a.w));
-    const float2 G = make_float2(ex2_approx(e.x), ex2_approx(e.y));
-    const float2 raw = mul2(f2(c.x), G);
-    const float2 alpha = mul2(make_float2(fminf(amax, raw.x), fminf(amax, raw.y)), take);
-    const float2 om = fma2(alpha, f2(-1.0f), f2(1.0f));
-    const float2 rom = make_float2(rcp_approx(om.x), rcp_approx(om.y));
-    float2 Tb = mul2(p.T, rom);
-    if (has_tb & 1u) Tb.x = tb.x;
-    if (has_tb & 2u) Tb.y = tb.y;
-    const float2 wgt = mul2(alpha, Tb);
-    const float2 cg = fma2(f2(c.w), p.g2, fma2(f2(c.z), p.g1, mul2(f2(c.y), p.g0)));
-    const float2 t4 = mul2(wgt, p.g0), t5 = mul2(wgt, p.g1), t6 = mul2(wgt, p.g2);
+    PairAlpha r;
+    r.G.x = ex2_approx(__fmul_rn(d2.x, a.w));
+    r.G.y = ex2_approx(__fmul_rn(d2.y, a.w));
+    if (CLAMP) {
+        const float rawA = c.x * r.G.x, rawB = c.x * r.G.y;
+        r.alpha = make_float2(tA ? fminf(amax, rawA) : 0.0f, tB ? fminf(amax, rawB) : 0.0f);
+        r.G = make_float2(tA && rawA < amax ? r.G.x : 0.0f, tB && rawB < amax ? r.G.y : 0.0f);
+    } else {
+        r.G = make_float2(tA ? r.G.x : 0.0f, tB ? r.G.y : 0.0f);
+        r.alpha = make_float2(c.x * r.G.x, c.x * r.G.y);
+    }
+    const float2 om = fma2(r.alpha, f2(-1.0f), f2(1.0f));
+    r.rom = make_float2(rcp_approx(om.x), rcp_approx(om.y));
+    r.cg = make_float2(fmaf(c.w, p.g2.x, fmaf(c.z, p.g1.x, c.y * p.g0.x)),
+                       fmaf(c.w, p.g2.y, fmaf(c.z, p.g1.y, c.y * p.g0.y)));
+    return r;
+}
+
+// The recursions at one point and its terms summed over the lane's two
+// pixels: v = {t0, t1, t2, do, dr, dg, db, 0}; updates T and S.  hasA /
+// hasB: tb holds the stored transmittance before the point (store mode)
+// instead of the one recovered by division.
+__device__ __forceinline__ void pair_recur(const PairAlpha &r, float2 d2, float dx, float2 dy,
+                                           BwdPair &p, bool hasA, bool hasB, float2 tb, float v[8])
+{
+    float2 Tb = mul2(p.T, r.rom);
+    if (hasA) Tb.x = tb.x;
+    if (hasB) Tb.y = tb.y;
+    const float2 w = mul2(r.alpha, Tb);
+    const float2 sr = mul2(p.S, r.rom);
+    const float2 dalpha = fma2(Tb, r.cg, make_float2(-sr.x, -sr.y));
+    p.S = fma2(w, r.cg, p.S);
+    p.T = Tb;
+    const float2 dG = mul2(dalpha, r.G);
+    const float2 t1 = mul2(dG, dy), t2 = mul2(dG, d2);
+    const float2 t4 = mul2(w, p.g0), t5 = mul2(w, p.g1), t6 = mul2(w, p.g2);
+    v[3] = dG.x + dG.y;
+    v[0] = v[3] * dx;
+    v[1] = t1.x + t1.y;
+    v[2] = t2.x + t2.y;
     v[4] = t4.x + t4.y;
     v[5] = t5.x + t5.y;
     v[6] = t6.x + t6.y;
-    const float2 dalpha = mul2(fma2(Tb, cg, mul2(p.S, mul2(rom, f2(-1.0f)))), take);
-    p.S = fma2(wgt, cg, p.S);
-    p.T = Tb;
-    // clamped alpha: no geometry terms
-    const float2 ca0 = mul2(dalpha, alpha), dg0 = mul2(dalpha, G);
-    const float2 ca = make_float2(raw.x < amax ? ca0.x : 0.0f, raw.y < amax ? ca0.y : 0.0f);
-    const float2 t1 = mul2(ca, dy), t2 = mul2(ca, d2);
-    v[0] = (ca.x + ca.y) * dx;
-    v[1] = t1.x + t1.y;
-    v[2] = t2.x + t2.y;
-    v[3] = (raw.x < amax ? dg0.x : 0.0f) + (raw.y < amax ? dg0.y : 0.0f);
     v[7] = 0.0f;
 }
 
-// Backward of one 8 x 8 block (blocks numbered row-major, TW/8 per row) by
-// one warp, for the persistent schedule: lane l owns the pixels A = (l & 7,
-// l >> 3) and B = (l & 7, 4 + (l >> 3)).  The warp takes the tile list's
-// entries with its block's bit (`bit`) from its queue, back to front.  Per
-// listed point the lane forms the adjoint at both pixels (packed fp32x2)
-// and adds the two term vectors, so the per-point warp work (staging, cull,
-// reduction or atomics) serves 64 pixels.  Each pixel's T and S recursions
-// are the one-pixel walk's operations.
-// V, (tx, ty): the tile's view and position; s: the start of its list.
-template <int TW, int TH, bool STATS, bool STORE>
-__device__ __forceinline__ void bwd_pair_item(const DevView *V, int tx, int ty, uint32_t s,
-                                              uint32_t bit, const DevOpts &o, int sub, int lane,
+// Adds one point's terms to its slot of the gradient buffer; cm: the lanes
+// with a contributing pixel.
+__device__ __forceinline__ void bwd_add(uint32_t cm, bool any, const float v[8], int lane,
+                                        float *__restrict__ g2d, uint32_t pv)
+{
+    if (__popc(cm) > BWD_DIRECT_MAX) {
+        warp_add_terms(v, lane, g2d, pv);
+    } else if (any) { // few lanes: each adds its own terms
+        float4 *dst = reinterpret_cast<float4 *>(g2d) + 2 * (size_t)pv;
+        atomicAdd(dst, make_float4(v[0], v[1], v[2], v[3]));
+        atomicAdd(dst + 1, make_float4(v[4], v[5], v[6], 0.f));
+    }
+}
+
+// Back-propagates one chunk of nh staged hits through the lane's pixels.
+template <bool CLAMP, bool STATS, bool STORE, bool FUSED>
+__device__ __forceinline__ void bwd_chunk(const BwdWarp &m, int nh, float ux, float2 uy,
+                                          float amax, int lane, BwdPair &p,
+                                          float *__restrict__ g2d, uint32_t &examined,
+                                          uint32_t &used, StoreRow &rowA, StoreRow &rowB)
+{
+    // two hits in flight: 363 against 368 us on the 4-view step; store mode's
+    // list pointers leave no registers for it (526 against 585 us)
+    constexpr int BWD_UNROLL = STORE ? 1 : 2;
+    for (int j0 = 0; j0 < nh; j0 += BWD_UNROLL) {
+        // BWD_UNROLL hits at a time: their loads and weights first, which do
+        // not depend on one another, then the recursions
+        PairAlpha pr[BWD_UNROLL];
+        bool hasA[BWD_UNROLL], hasB[BWD_UNROLL], any[BWD_UNROLL];
+        float2 tb[BWD_UNROLL], d2[BWD_UNROLL], dy[BWD_UNROLL];
+        float dx[BWD_UNROLL];
+        uint32_t pv[BWD_UNROLL];
+#pragma unroll
+        for (int u = 0; u < BWD_UNROLL; ++u) {
+            const float4 aj = m.a[j0 + u], cj = m.c[j0 + u];
+            const uint2 ip = m.ip[j0 + u];
+            pv[u] = ip.y;
+            d2[u] = pair_d2<FUSED>(ux, uy, aj.x, aj.y, dx[u], dy[u]);
+            const bool bA = ip.x < p.LA, bB = ip.x < p.LB;
+            const bool tA = bA && d2[u].x <= aj.z, tB = bB && d2[u].y <= aj.z;
+            if (STATS) {
+                examined += (uint32_t)bA + (uint32_t)bB;
+                used += (uint32_t)tA + (uint32_t)tB;
+            }
+            any[u] = tA || tB;
+            hasA[u] = hasB[u] = false;
+            tb[u] = f2(0.0f);
+            if (STORE) {
+                hasA[u] = row_next(rowA, tA, tb[u].x);
+                hasB[u] = row_next(rowB, tB, tb[u].y);
+            }
+            pr[u] = pair_alpha<CLAMP>(tA, tB, d2[u], aj, cj, amax, p);
+        }
+#pragma unroll
+        for (int u = 0; u < BWD_UNROLL; ++u) {
+            const uint32_t cm = __ballot_sync(0xffffffffu, any[u]);
+            if (!cm) continue;
+            float v[8];
+            pair_recur(pr[u], d2[u], dx[u], dy[u], p, hasA[u], hasB[u], tb[u], v);
+            bwd_add(cm, any[u], v, lane, g2d, pv[u]);
+        }
+    }
+}
+
+// Backward of one 8 x 8 block with first pixel (sx0, sy0) of view V by one
+// warp: lane l owns the pixels A = (l & 7, l >> 3) and B = (l & 7, 4 + (l >>
+// 3)).  The warp takes the tile list's entries with its block's bit (`bit`)
+// from its queue, back to front, 32 at a time, and keeps those whose disc
+// meets the rectangle of the pixels whose composited list reaches them; the
+// records of the next 32 are in flight while these are processed.  Per hit
+// the lane forms the adjoint at both pixels (packed fp32x2) and adds the two
+// term vectors, so the per-point warp work serves 64 pixels.  s: the start
+// of the tile's list.
+template <bool STATS, bool STORE, bool FUSED>
+__device__ __forceinline__ void bwd_pair_item(const DevView *V, int sx0, int sy0, uint32_t s,
+                                              uint32_t bit, const DevOpts &o, int lane,
                                               const uint32_t *__restrict__ keys,
                                               const uint32_t *__restrict__ pv_list,
                                               const float4 *__restrict__ rec,
@@ -912,10 +813,8 @@ __device__ __forceinline__ void bwd_pair_item(const DevView *V, int tx, int ty, 
                                               const uint32_t *__restrict__ n_contrib,
                                               const float *__restrict__ grad_rgb,
                                               float *__restrict__ g2d, uint32_t &examined,
-                                              uint32_t &used, float4 *wbuf, uint2 *wpp,
-                                              WarpQueue &q, const StoreBuf &sto)
+                                              uint32_t &used, BwdWarp &m, const StoreBuf &sto)
 {
-    const int sx0 = tx * TW + (sub % (TW / 8)) * 8, sy0 = ty * TH + (sub / (TW / 8)) * 8;
     PixelGeom g[2];
     g[0] = pixel_geom_at(V, sx0, sy0, lane);
     g[1] = pixel_geom_at(V, sx0, sy0 + 4, lane);
@@ -929,121 +828,87 @@ __device__ __forceinline__ void bwd_pair_item(const DevView *V, int tx, int ty, 
     p.g2 = make_float2(pa.g2, pb.g2);
     p.LA = pa.L;
     p.LB = pb.L;
+    const uint32_t wmax = __reduce_max_sync(0xffffffffu, max(p.LA, p.LB));
+    if (wmax == 0) return;
     // store mode: composited points not yet visited, per pixel
-    const int64_t pixA = STORE && g[0].inside ? pixel_index(g[0]) : 0;
-    const int64_t pixB = STORE && g[1].inside ? pixel_index(g[1]) : 0;
-    uint32_t kA = 0, kB = 0;
+    StoreRow rowA, rowB;
     if (STORE) {
-        if (g[0].inside) kA = sto.n[pixA];
-        if (g[1].inside) kB = sto.n[pixB];
+        rowA = store_row(sto, g[0].inside ? pixel_index(g[0]) : 0, g[0].inside);
+        rowB = store_row(sto, g[1].inside ? pixel_index(g[1]) : 0, g[1].inside);
     }
+    const uint32_t lt = lanemask_lt_r();
     const float ux = g[0].ux;
     const float2 uy = make_float2(g[0].uy, g[1].uy);
-    const uint32_t wmax = __reduce_max_sync(0xffffffffu, max(pa.L, pb.L));
-    if (wmax == 0) return;
     int64_t c = (int64_t)((wmax - 1) & ~31u);
     int qn = 0;
     uint32_t qh = 0;
-    while (true) {
-        queue_fill_back(keys, pv_list, s, wmax, bit, c, qn, qh, q, lane);
-        if (qn == 0) break;
-        uint32_t rel = 0, pv = 0;
-        const int take = queue_take(q, qn, qh, lane, rel, pv);
-        const bool valid = lane < take;
-        float4 a = make_float4(0.f, 0.f, -1.f, 0.f);
-        if (valid) a = __ldg(rec + 2 * (size_t)pv);
-        // pixels whose composited list reaches the chunk's nearest entry; every
-        // lane takes part in the reductions, whatever its entry
+    uint32_t rel = 0, pv = 0;
+    float4 ra = make_float4(0.f, 0.f, -1.f, 0.f), rc = ra;
+    int take = 0;
+    auto fetch = [&]() {
+        queue_fill_back(keys, pv_list, s, wmax, bit, c, qn, qh, m.q, lane);
+        take = qn > 0 ? queue_take(m.q, qn, qh, lane, rel, pv) : 0;
+        if (lane < take) {
+            ra = __ldg(rec + 2 * (size_t)pv);
+            rc = __ldg(rec + 2 * (size_t)pv + 1);
+        }
+    };
+    fetch();
+    while (take > 0) {
+        // pixels whose composited list reaches the chunk's nearest entry;
+        // every lane takes part in the reductions, whatever its entry
         const uint32_t lowest = __shfl_sync(0xffffffffu, rel, take - 1);
         const bool act[2] = {p.LA > lowest, p.LB > lowest};
         const PixelGeom ar = active_rect_rows<2>(g, act);
-        const bool hit = valid && disc_meets_rect(a, ar);
-        uint32_t m = __ballot_sync(0xffffffffu, hit);
-        if (hit) {
-            wbuf[lane] = a;
-            wbuf[32 + lane] = __ldg(rec + 2 * (size_t)pv + 1);
-            wpp[lane] = make_uint2(rel, pv);
-        }
+        const bool hit = lane < take && disc_meets_rect(ra, ar);
+        const uint32_t hm = __ballot_sync(0xffffffffu, hit);
+        // amplitudes that may reach the clamp (a NaN counts as one)
+        const bool clamp = __any_sync(0xffffffffu, hit && !(rc.x < o.alpha_max));
+        const int nh = __popc(hm);
+        const int slot = hit ? __popc(hm & lt) : nh + __popc(~hm & lt);
+        // the slots behind the hits are filled with points no pixel includes
+        m.a[slot] = hit ? ra : make_float4(0.f, 0.f, -1.f, 0.f);
+        m.c[slot] = rc;
+        m.ip[slot] = make_uint2(rel, pv);
         __syncwarp();
-        while (m) {
-            const int j = __ffs(m) - 1; // back to front: queue order
-            m &= m - 1;
-            const float4 aj = wbuf[j];
-            const uint2 pp = wpp[j]; // list position, point-view
-            const uint32_t idx = pp.x;
-            float dx;
-            float2 dy;
-            const float2 d2 = pair_d2(ux, uy, aj.x, aj.y, dx, dy);
-            const bool bA = idx < p.LA, bB = idx < p.LB;
-            const bool cA = bA && d2.x <= aj.z, cB = bB && d2.y <= aj.z;
-            if (STATS) {
-                examined += (uint32_t)bA + (uint32_t)bB;
-                used += (uint32_t)cA + (uint32_t)cB;
-            }
-            const bool any = cA || cB;
-            const uint32_t cm = __ballot_sync(0xffffffffu, any);
-            if (cm) {
-                float v[8];
-                uint32_t has_tb = 0u;
-                float2 tb = make_float2(0.0f, 0.0f);
-                if (STORE) {
-                    if (cA && --kA < (uint32_t)sto.depth) {
-                        has_tb |= 1u;
-                        tb.x = sto.T[pixA * sto.depth + kA];
-                    }
-                    if (cB && --kB < (uint32_t)sto.depth) {
-                        has_tb |= 2u;
-                        tb.y = sto.T[pixB * sto.depth + kB];
-                    }
-                }
-                pair_adjoint(make_float2(cA ? 1.0f : 0.0f, cB ? 1.0f : 0.0f), d2, dx, dy, aj,
-                             wbuf[32 + j], o.alpha_max, p, v, has_tb, tb);
-                if (__popc(cm) > BWD_PAIR_DIRECT_MAX) {
-                    warp_add_terms(v, lane, g2d, pp.y);
-                } else if (any) { // few lanes: each adds its own terms
-                    float4 *dst = reinterpret_cast<float4 *>(g2d) + 2 * (size_t)pp.y;
-                    atomicAdd(dst, make_float4(v[0], v[1], v[2], v[3]));
-                    atomicAdd(dst + 1, make_float4(v[4], v[5], v[6], 0.f));
-                }
-            }
-        }
+        fetch();
+        if (clamp)
+            bwd_chunk<true, STATS, STORE, FUSED>(m, nh, ux, uy, o.alpha_max, lane, p, g2d,
+                                                 examined, used, rowA, rowB);
+        else
+            bwd_chunk<false, STATS, STORE, FUSED>(m, nh, ux, uy, o.alpha_max, lane, p, g2d,
+                                                  examined, used, rowA, rowB);
         __syncwarp(); // chunk consumed before the buffers are refilled
     }
 }
 
-// Bit of the 8 x 8 block holding the 8 x 4 sub-block w of a TW-wide tile
-// in the pair keys' block masks (0 when a tile is a single block).
-template <int TW, int TH>
-__device__ __forceinline__ uint32_t stream_block_bit(int w)
-{
-    constexpr int BPR = TW / 8;
-    return block_bits(TW, TH) ? 1u << (((w / BPR) >> 1) * BPR + w % BPR) : 0u;
-}
-
-template <int TW, int TH, bool STORE>
-__global__ void __launch_bounds__(TW * TH)
+// Warp-streamed: one block per tile, warp w takes the tile's 8 x 8 block w.
+template <int TW, int TH, bool COUNT, bool STORE>
+__global__ void __launch_bounds__(TW * TH / 2)
 raster_fwd_stream_kernel(Batch b, DevOpts o, const uint2 *__restrict__ ranges,
                          const uint32_t *__restrict__ keys, const uint32_t *__restrict__ pv_list,
                          const float4 *__restrict__ rec, float *__restrict__ out_rgb,
                          float *__restrict__ T_final, uint32_t *__restrict__ n_contrib,
                          unsigned long long *__restrict__ stats, StoreBuf sto)
 {
-    constexpr int NW = TW * TH / 32;
-    __shared__ float4 s_buf[NW][64];
-    __shared__ uint32_t s_pos[NW][32];
-    __shared__ WarpQueue s_q[NW];
+    __shared__ FwdWarp s_fwd[TW * TH / 64];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    uint32_t ex = 0, co = 0;
+    const DevView *V = &b.views[find_view_by_tile(b, blockIdx.x)];
+    const uint32_t local = blockIdx.x - V->tile_base;
+    const int tx = (int)(local % (uint32_t)V->tiles_x), ty = (int)(local / (uint32_t)V->tiles_x);
+    const int sx0 = tx * TW + (w % (TW / 8)) * 8, sy0 = ty * TH + (w / (TW / 8)) * 8;
+    const uint32_t bit = block_bits(TW, TH) ? 1u << w : 0u;
     const uint2 rg = ranges[blockIdx.x];
-    fwd_stream_item<true, STORE>(pixel_geom<TW, TH>(b, blockIdx.x, w, lane), rg.x,
-                    rg.y > rg.x ? rg.y : rg.x,
-                    stream_block_bit<TW, TH>(w), o, lane, keys, pv_list, rec, out_rgb, T_final,
-                    n_contrib, ex, co, s_buf[w], s_pos[w], s_q[w], sto);
-    add_stats(stats, ex, co, lane);
+    uint32_t ex = 0, co = 0;
+    fwd_pair_item<COUNT, STORE, false>(pixel_geom_at(V, sx0, sy0, lane),
+                                pixel_geom_at(V, sx0, sy0 + 4, lane), rg.x,
+                                rg.y > rg.x ? rg.y : rg.x, bit, o, lane, keys, pv_list, rec,
+                                out_rgb, T_final, n_contrib, ex, co, s_fwd[w], sto);
+    if (COUNT) add_stats(stats, ex, co, lane);
 }
 
-template <int TW, int TH, bool STORE>
-__global__ void __launch_bounds__(TW * TH)
+template <int TW, int TH, bool STATS, bool STORE>
+__global__ void __launch_bounds__(TW * TH / 2)
 raster_bwd_stream_kernel(Batch b, DevOpts o, const uint2 *__restrict__ ranges,
                          const uint32_t *__restrict__ keys, const uint32_t *__restrict__ pv_list,
                          const float4 *__restrict__ rec, const float *__restrict__ T_final,
@@ -1051,18 +916,17 @@ raster_bwd_stream_kernel(Batch b, DevOpts o, const uint2 *__restrict__ ranges,
                          float *__restrict__ g2d, unsigned long long *__restrict__ stats,
                          StoreBuf sto)
 {
-    constexpr int NW = TW * TH / 32;
-    __shared__ float4 s_buf[NW][64];
-    __shared__ uint32_t s_pv[NW][32];
-    __shared__ uint32_t s_pos[NW][32];
-    __shared__ WarpQueue s_q[NW];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    __shared__ BwdWarp s_bwd[TW * TH / 64];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5; // warp w: the tile's 8 x 8 block w
+    const DevView *V = &b.views[find_view_by_tile(b, blockIdx.x)];
+    const uint32_t local = blockIdx.x - V->tile_base;
+    const int tx = (int)(local % (uint32_t)V->tiles_x), ty = (int)(local / (uint32_t)V->tiles_x);
+    const uint32_t bit = block_bits(TW, TH) ? 1u << w : 0u;
     uint32_t ex = 0, us = 0;
-    bwd_stream_item<TW, TH, STORE>(b, o, blockIdx.x, w, stream_block_bit<TW, TH>(w), lane,
-                                   ranges, keys,
-                            pv_list, rec, T_final, n_contrib, grad_rgb, g2d, ex, us, s_buf[w],
-                            s_pv[w], s_pos[w], s_q[w], sto);
-    add_stats(stats ? stats + 2 : nullptr, ex, us, lane);
+    bwd_pair_item<STATS, STORE, false>(V, tx * TW + (w % (TW / 8)) * 8, ty * TH + (w / (TW / 8)) * 8,
+                                ranges[blockIdx.x].x, bit, o, lane, keys, pv_list, rec, T_final,
+                                n_contrib, grad_rgb, g2d, ex, us, s_bwd[w], sto);
+    if (STATS) add_stats(stats ? stats + 2 : nullptr, ex, us, lane);
 }
 
 // ------------------------------------------------------------ persistent
@@ -1070,6 +934,7 @@ raster_bwd_stream_kernel(Batch b, DevOpts o, const uint2 *__restrict__ ranges,
 // counter over `order` (tiles sorted longest list first), so long tiles
 // start early and no warp idles while work remains.
 constexpr int PERSIST_THREADS = 256;
+constexpr int BWD_PERSIST_BLOCKS = 4;
 constexpr int FWD_PERSIST_BLOCKS = 5; // forward blocks per SM (see the kernel)
 
 __device__ __forceinline__ uint32_t next_item(uint32_t *work, int lane)
@@ -1092,12 +957,13 @@ __device__ __forceinline__ uint4 tile_desc(const Batch &b, const uint2 *ranges, 
     return make_uint4((uint32_t)v, tx | (ty << 16), r.x, r.y > r.x ? r.y : r.x);
 }
 
-// STATS: count examined / composited pairs into stats (which must then be
-// non-null); without, the loops carry no counting.  The forward's 8 x 8
-// warps run five blocks per SM (48 registers): 5.47 ms on the 1M-point,
-// 64-view step against 5.66 at four (six spill).  The backward runs best at
-// its natural four blocks (five: 11.1 -> 11.9 ms).
-template <int TW, int TH, bool STATS, bool STORE>
+// COUNT / STATS: count composited points and, with stats non-null, the
+// examined / composited pairs; without, the loops carry no counting.  The
+// forward's warps run five blocks per SM (48 registers): 4.05 ms on the
+// 1M-point, 64-view step against 4.10 at four and 4.27 at six (unrolled by
+// two).  The backward runs best at four (64 registers): 8.87 ms, 9.07 at
+// three, 8.96 at five.
+template <int TW, int TH, bool COUNT, bool STORE>
 __global__ void __launch_bounds__(PERSIST_THREADS, FWD_PERSIST_BLOCKS)
 raster_fwd_persist_kernel(Batch b, DevOpts o, const uint2 *__restrict__ ranges,
                           const uint32_t *__restrict__ keys, const uint32_t *__restrict__ pv_list,
@@ -1108,9 +974,7 @@ raster_fwd_persist_kernel(Batch b, DevOpts o, const uint2 *__restrict__ ranges,
 {
     constexpr uint32_t SUBS = (TW / 8) * (TH / 8);
     constexpr int NW = PERSIST_THREADS / 32;
-    __shared__ float4 s_buf[NW][64];
-    __shared__ uint32_t s_pos[NW][32];
-    __shared__ WarpQueue s_q[NW];
+    __shared__ FwdWarp s_fwd[NW];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const uint32_t n_items = b.n_tiles * SUBS;
     uint32_t ex = 0, co = 0;
@@ -1121,16 +985,17 @@ raster_fwd_persist_kernel(Batch b, DevOpts o, const uint2 *__restrict__ ranges,
         const int sx0 = (int)(d.y & 0xffffu) * TW + (sub % (TW / 8)) * 8;
         const int sy0 = (int)(d.y >> 16) * TH + (sub / (TW / 8)) * 8;
         const uint32_t bit = block_bits(TW, TH) ? 1u << sub : 0u;
-        fwd_pair_item<STATS, STORE>(pixel_geom_at(V, sx0, sy0, lane),
-                                    pixel_geom_at(V, sx0, sy0 + 4, lane),
-                             d.z, d.w, bit, o, lane, keys, pv_list, rec, out_rgb, T_final,
-                             n_contrib, ex, co, s_buf[w], s_pos[w], s_q[w], sto);
+        fwd_pair_item<COUNT, STORE, true>(pixel_geom_at(V, sx0, sy0, lane),
+                                    pixel_geom_at(V, sx0, sy0 + 4, lane), d.z, d.w, bit, o, lane,
+                                    keys, pv_list, rec, out_rgb, T_final, n_contrib, ex, co,
+                                    s_fwd[w], sto);
+        __syncwarp(); // the item's shared memory is read before the next one writes it
     }
-    if (STATS) add_stats(stats, ex, co, lane);
+    if (COUNT) add_stats(stats, ex, co, lane);
 }
 
 template <int TW, int TH, bool STATS, bool STORE>
-__global__ void __launch_bounds__(PERSIST_THREADS)
+__global__ void __launch_bounds__(PERSIST_THREADS, BWD_PERSIST_BLOCKS)
 raster_bwd_persist_kernel(Batch b, DevOpts o, const uint2 *__restrict__ ranges,
                           const uint32_t *__restrict__ keys, const uint32_t *__restrict__ pv_list,
                           const float4 *__restrict__ rec, const float *__restrict__ T_final,
@@ -1141,10 +1006,7 @@ raster_bwd_persist_kernel(Batch b, DevOpts o, const uint2 *__restrict__ ranges,
 {
     // 8 x 8 blocks, numbered like the key masks
     constexpr uint32_t SUBS = (TW / 8) * (TH / 8);
-    constexpr int NW = PERSIST_THREADS / 32;
-    __shared__ float4 s_buf[NW][64];
-    __shared__ uint2 s_pp[NW][32];
-    __shared__ WarpQueue s_q[NW];
+    __shared__ BwdWarp s_bwd[PERSIST_THREADS / 32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const uint32_t n_items = b.n_tiles * SUBS;
     uint32_t ex = 0, us = 0;
@@ -1152,13 +1014,13 @@ raster_bwd_persist_kernel(Batch b, DevOpts o, const uint2 *__restrict__ ranges,
         const uint4 d = order[it / SUBS];
         const int sub = (int)(it % SUBS);
         const uint32_t bit = block_bits(TW, TH) ? 1u << sub : 0u;
-        bwd_pair_item<TW, TH, STATS, STORE>(&b.views[d.x], (int)(d.y & 0xffffu), (int)(d.y >> 16),
-                                            d.z,
-                                     bit, o, sub, lane, keys, pv_list, rec, T_final, n_contrib,
-                                     grad_rgb, g2d, ex, us, s_buf[w], s_pp[w], s_q[w],
-                                     sto);
+        const int sx0 = (int)(d.y & 0xffffu) * TW + (sub % (TW / 8)) * 8;
+        const int sy0 = (int)(d.y >> 16) * TH + (sub / (TW / 8)) * 8;
+        bwd_pair_item<STATS, STORE, true>(&b.views[d.x], sx0, sy0, d.z, bit, o, lane, keys, pv_list, rec,
+                                    T_final, n_contrib, grad_rgb, g2d, ex, us, s_bwd[w], sto);
+        __syncwarp(); // the item's shared memory is read before the next one writes it
     }
-    if (STATS) add_stats(stats + 2, ex, us, lane);
+    if (STATS) add_stats(stats ? stats + 2 : nullptr, ex, us, lane);
 }
 
 // Tile order, longest list first: bucket = floor(log2(length)), buckets in
@@ -1402,35 +1264,47 @@ int persist_grid(const void *kernel)
     return sms * (per_sm > 0 ? per_sm : 1);
 }
 
-template <int TW, int TH, bool STATS, bool STORE>
-void fwd_persist_launch(const Batch &b, const DevOpts &o, const uint2 *ranges,
-                        const uint32_t *keys, const uint32_t *pv_list, const float4 *rec,
-                        float *out_rgb, float *T_final, uint32_t *n_contrib,
-                        unsigned long long *stats, const uint4 *order, uint32_t *work,
-                        cudaStream_t s, const StoreBuf &sto)
+template <int TW, int TH, bool COUNT, bool STORE>
+void fwd_launch(const Batch &b, const DevOpts &o, const uint2 *ranges, const uint32_t *keys,
+                const uint32_t *pv_list, const float4 *rec, float *out_rgb, float *T_final,
+                uint32_t *n_contrib, unsigned long long *stats, const uint4 *order, uint32_t *work,
+                cudaStream_t s, const StoreBuf &sto)
 {
-    static const int grid =
-        persist_grid((const void *)raster_fwd_persist_kernel<TW, TH, STATS, STORE>);
-    raster_fwd_persist_kernel<TW, TH, STATS, STORE><<<grid, PERSIST_THREADS, 0, s>>>(
-        b, o, ranges, keys, pv_list, rec, out_rgb, T_final, n_contrib, stats, order, work, sto);
+    if (order) {
+        static const int grid =
+            persist_grid((const void *)raster_fwd_persist_kernel<TW, TH, COUNT, STORE>);
+        raster_fwd_persist_kernel<TW, TH, COUNT, STORE><<<grid, PERSIST_THREADS, 0, s>>>(
+            b, o, ranges, keys, pv_list, rec, out_rgb, T_final, n_contrib, stats, order, work,
+            sto);
+    } else {
+        raster_fwd_stream_kernel<TW, TH, COUNT, STORE><<<b.n_tiles, TW * TH / 2, 0, s>>>(
+            b, o, ranges, keys, pv_list, rec, out_rgb, T_final, n_contrib, stats, sto);
+    }
 }
 
 template <int TW, int TH, bool STATS, bool STORE>
-void bwd_persist_launch(const Batch &b, const DevOpts &o, const uint2 *ranges,
-                        const uint32_t *keys, const uint32_t *pv_list, const float4 *rec,
-                        const float *T_final, const uint32_t *n_contrib, const float *grad_rgb,
-                        float4 *g2d, unsigned long long *stats, const uint4 *order, uint32_t *work,
-                        cudaStream_t s, const StoreBuf &sto)
+void bwd_launch(const Batch &b, const DevOpts &o, const uint2 *ranges, const uint32_t *keys,
+                const uint32_t *pv_list, const float4 *rec, const float *T_final,
+                const uint32_t *n_contrib, const float *grad_rgb, float4 *g2d,
+                unsigned long long *stats, const uint4 *order, uint32_t *work, cudaStream_t s,
+                const StoreBuf &sto)
 {
-    static const int grid =
-        persist_grid((const void *)raster_bwd_persist_kernel<TW, TH, STATS, STORE>);
-    raster_bwd_persist_kernel<TW, TH, STATS, STORE><<<grid, PERSIST_THREADS, 0, s>>>(
-        b, o, ranges, keys, pv_list, rec, T_final, n_contrib, grad_rgb, (float *)g2d, stats,
-        order, work + 1, sto);
+    if (order) {
+        static const int grid =
+            persist_grid((const void *)raster_bwd_persist_kernel<TW, TH, STATS, STORE>);
+        raster_bwd_persist_kernel<TW, TH, STATS, STORE><<<grid, PERSIST_THREADS, 0, s>>>(
+            b, o, ranges, keys, pv_list, rec, T_final, n_contrib, grad_rgb, (float *)g2d, stats,
+            order, work + 1, sto);
+    } else {
+        raster_bwd_stream_kernel<TW, TH, STATS, STORE><<<b.n_tiles, TW * TH / 2, 0, s>>>(
+            b, o, ranges, keys, pv_list, rec, T_final, n_contrib, grad_rgb, (float *)g2d, stats,
+            sto);
+    }
 }
 
-// The kernels are instantiated with and without pair counting (STATS) and
-// store mode (STORE), so that the variants the graphs run carry neither.
+// The kernels are instantiated with and without pair counting (STATS, COUNT)
+// and store mode (STORE, which counts too), so that the variants the graphs
+// run carry neither; the count cap needs the forward's counting variant.
 template <int TW, int TH>
 void fwd_dispatch(const Batch &b, const DevOpts &o, int depth, const uint2 *ranges,
                   const uint32_t *keys, const uint32_t *pv_list, const float4 *rec,
@@ -1439,18 +1313,12 @@ void fwd_dispatch(const Batch &b, const DevOpts &o, int depth, const uint2 *rang
                   uint32_t *work, cudaStream_t s, const StoreBuf &sto)
 {
     const bool store = sto.T != nullptr;
-    if (depth == 0 && order) {
-        auto f = stats ? (store ? fwd_persist_launch<TW, TH, true, true>
-                                : fwd_persist_launch<TW, TH, true, false>)
-                       : (store ? fwd_persist_launch<TW, TH, false, true>
-                                : fwd_persist_launch<TW, TH, false, false>);
+    if (depth == 0) {
+        auto f = store ? fwd_launch<TW, TH, true, true>
+                 : stats || o.max_per_pixel ? fwd_launch<TW, TH, true, false>
+                                            : fwd_launch<TW, TH, false, false>;
         f(b, o, ranges, keys, pv_list, rec, out_rgb, T_final, n_contrib, stats, order, work, s,
           sto);
-    } else if (depth == 0) {
-        auto k = store ? raster_fwd_stream_kernel<TW, TH, true>
-                       : raster_fwd_stream_kernel<TW, TH, false>;
-        k<<<b.n_tiles, TW * TH, 0, s>>>(b, o, ranges, keys, pv_list, rec, out_rgb, T_final,
-                                        n_contrib, stats, sto);
     } else {
         const size_t smem =
             (size_t)depth * (2 * sizeof(float4) + (TW * TH / 32) * sizeof(uint16_t));
@@ -1473,18 +1341,12 @@ void bwd_dispatch(const Batch &b, const DevOpts &o, int depth, const uint2 *rang
                   cudaStream_t s, const StoreBuf &sto)
 {
     const bool store = sto.T != nullptr;
-    if (depth == 0 && order) {
-        auto f = stats ? (store ? bwd_persist_launch<TW, TH, true, true>
-                                : bwd_persist_launch<TW, TH, true, false>)
-                       : (store ? bwd_persist_launch<TW, TH, false, true>
-                                : bwd_persist_launch<TW, TH, false, false>);
+    if (depth == 0) {
+        auto f = store ? bwd_launch<TW, TH, true, true>
+                 : stats ? bwd_launch<TW, TH, true, false>
+                         : bwd_launch<TW, TH, false, false>;
         f(b, o, ranges, keys, pv_list, rec, T_final, n_contrib, grad_rgb, g2d, stats, order, work,
           s, sto);
-    } else if (depth == 0) {
-        auto k = store ? raster_bwd_stream_kernel<TW, TH, true>
-                       : raster_bwd_stream_kernel<TW, TH, false>;
-        k<<<b.n_tiles, TW * TH, 0, s>>>(b, o, ranges, keys, pv_list, rec, T_final, n_contrib,
-                                        grad_rgb, (float *)g2d, stats, sto);
     } else {
         const size_t smem = (size_t)depth * (4 * sizeof(float4) + sizeof(uint32_t) +
                                              (TW * TH / 32) * sizeof(uint16_t));
