@@ -22,8 +22,8 @@ int nearest_maps(TempBufs &tb, const float *p1, int64_t n1, const SearchIndex &S
     float *d12, *d21;
     PBR_TRY(tb.alloc(&d12, sizeof(float) * n1));
     PBR_TRY(tb.alloc(&d21, sizeof(float) * n2));
-    PBR_TRY(run_knn(tb, p1, n1, p2, n2, S2, 1, 1, 0, nn12, d12, s));
-    PBR_TRY(run_knn(tb, p2, n2, p1, n1, S1, 1, 1, 0, nn21, d21, s));
+    PBR_TRY(run_knn(tb, p1, n1, &S1.fine, p2, n2, S2, 1, 1, 0, nn12, d12, s));
+    PBR_TRY(run_knn(tb, p2, n2, &S2.fine, p1, n1, S1, 1, 1, 0, nn21, d21, s));
     return PBR_OK;
 }
 
@@ -199,7 +199,7 @@ extern "C" int pbr_frame_init(pbr_ctx *ctx, const pbr_points *prev, float *pos2,
     float *d2;
     PBR_TRY(tb.alloc(&idx, sizeof(int32_t) * k * n2));
     PBR_TRY(tb.alloc(&d2, sizeof(float) * k * n2));
-    PBR_TRY(run_knn(tb, pos2, n2, p1, n1, S1, k, keff, 0, idx, d2, s));
+    PBR_TRY(run_knn(tb, pos2, n2, nullptr, p1, n1, S1, k, keff, 0, idx, d2, s));
     launch_generate(idx, n2, k, keff, PointArrays{p1, prev->sh, prev->opacity, prev->radius, nsh},
                     PointArraysOut{nullptr, sh2, opacity2, radius2, nsh}, 0, s, 3);
     if (loss_history)

@@ -30,10 +30,8 @@ int read_count(const unsigned long long *dev, int64_t *out, cudaStream_t s)
 constexpr int64_t MAX_TABLE_CELLS = 1ll << 28;
 
 // Sorted (cell id, index) list of n points on grid gp; ends in (*keys, *vals).
-// With `table` set, also the dense cell-start table of grids small enough
-// for one (else *table = NULL).
 int sorted_cells(TempBufs &tb, const float *pos, int64_t n, const GridParams *gp, int n_cells,
-                 uint32_t **keys, uint32_t **vals, cudaStream_t s, uint32_t **table = nullptr)
+                 uint32_t **keys, uint32_t **vals, cudaStream_t s)
 {
     uint32_t *k0, *v0, *k1, *v1;
     void *tmp;
@@ -46,18 +44,36 @@ int sorted_cells(TempBufs &tb, const float *pos, int64_t n, const GridParams *gp
     radix_sort_pairs(k0, v0, k1, v1, nullptr, n, key_bits_of(n_cells), tmp, s);
     *keys = k0;
     *vals = v0;
-    if (table) {
-        *table = nullptr;
-        const int64_t cells = (int64_t)n_cells * n_cells * n_cells;
-        if (cells <= MAX_TABLE_CELLS) {
-            void *stmp;
-            PBR_TRY(tb.alloc(table, sizeof(uint32_t) * (cells + 1)));
-            PBR_TRY(tb.alloc(&stmp, scan_temp_bytes(cells + 1)));
-            launch_cell_start(k0, n, cells, *table, stmp, s);
-        }
-    }
     return PBR_OK;
 }
+
+int64_t cells_of(const Grid &G) { return (int64_t)G.cells * G.cells * G.cells; }
+
+// The n points in the cells of grid G: counted into a table, or sorted by id
+// where the table would be too large.  gate: see launch_cell_sort.
+int fill_grid(TempBufs &tb, const float *pos, int64_t n, Grid &G, const uint32_t *gate,
+              cudaStream_t s)
+{
+    const int64_t cells = cells_of(G);
+    PBR_TRY(tb.alloc(&G.pts, sizeof(float4) * n));
+    G.cs = G.rid = nullptr;
+    if (cells > MAX_TABLE_CELLS) {
+        uint32_t *idx;
+        PBR_TRY(sorted_cells(tb, pos, n, G.gp, G.cells, &G.rid, &idx, s));
+        launch_gather_points(pos, idx, n, G.pts, s);
+        return PBR_OK;
+    }
+    uint32_t *ids;
+    void *stmp;
+    PBR_TRY(tb.alloc(&ids, sizeof(uint32_t) * n));
+    PBR_TRY(tb.alloc(&G.cs, sizeof(uint32_t) * (cells + 1)));
+    PBR_TRY(tb.alloc(&stmp, scan_temp_bytes(cells)));
+    launch_cell_sort(pos, n, G.gp, cells, ids, G.cs, G.pts, stmp, gate, s);
+    return PBR_OK;
+}
+
+// Whether S's coarse grid is built only by the searches that need it.
+bool coarse_on_demand(const SearchIndex &S) { return S.has_coarse && cells_of(S.coarse) <= GATED_CELLS; }
 
 } // namespace
 
@@ -86,52 +102,29 @@ int pbr::make_params(TempBufs &tb, const float *pos, int64_t n, int cells, Searc
     return PBR_OK;
 }
 
-// Sorted lists and tables of both levels for the n reference points.
 int pbr::index_points(TempBufs &tb, const float *ref, int64_t n, SearchIndex &S, cudaStream_t s)
 {
     if (n <= 0) return PBR_OK;
-    PBR_TRY(sorted_cells(tb, ref, n, S.fine.gp, S.fine.cells, &S.fine.rid, &S.fine.ridx, s,
-                         &S.fine.cs));
-    if (S.has_coarse)
-        PBR_TRY(sorted_cells(tb, ref, n, S.coarse.gp, S.coarse.cells, &S.coarse.rid,
-                             &S.coarse.ridx, s, &S.coarse.cs));
+    PBR_TRY(fill_grid(tb, ref, n, S.fine, nullptr, s));
+    if (S.has_coarse && !coarse_on_demand(S)) PBR_TRY(fill_grid(tb, ref, n, S.coarse, nullptr, s));
     return PBR_OK;
 }
 
-// Both levels restricted to the kept points (indices renumbered by newpos,
-// the exclusive scan of keep), tables rebuilt in place.
-int pbr::keep_points(TempBufs &tb, SearchIndex &S, int64_t m, int64_t m2, const uint32_t *keep,
-                const uint32_t *newpos, void *scan_tmp, cudaStream_t s)
+int pbr::run_knn(TempBufs &tb, const float *q, int64_t nq, const Grid *qorder, const float *ref,
+                 int64_t nr, const SearchIndex &S, int k, int keff, int self_mode,
+                 int32_t *out_idx, float *out_d2, cudaStream_t s)
 {
-    uint32_t *flags;
-    PBR_TRY(tb.alloc(&flags, sizeof(uint32_t) * m));
-    for (int level = 0; level < (S.has_coarse ? 2 : 1); ++level) {
-        Grid &G = level ? S.coarse : S.fine;
-        uint32_t *sid, *sidx;
-        PBR_TRY(tb.alloc(&sid, sizeof(uint32_t) * m2));
-        PBR_TRY(tb.alloc(&sidx, sizeof(uint32_t) * m2));
-        launch_list_keep(G.rid, G.ridx, keep, newpos, m, flags, sid, sidx, scan_tmp, s);
-        G.rid = sid;
-        G.ridx = sidx;
-        if (G.cs) {
-            void *ctmp;
-            const int64_t cells = (int64_t)G.cells * G.cells * G.cells;
-            PBR_TRY(tb.alloc(&ctmp, scan_temp_bytes(cells + 1)));
-            launch_cell_start(sid, m2, cells, G.cs, ctmp, s);
-        }
-    }
-    return PBR_OK;
-}
-
-int pbr::run_knn(TempBufs &tb, const float *q, int64_t nq, const float *ref, int64_t nr,
-            const SearchIndex &S, int k, int keff, int self_mode, int32_t *out_idx, float *out_d2,
-            cudaStream_t s)
-{
+    if (nq <= 0) return PBR_OK;
     void *ktmp;
     PBR_TRY(tb.alloc(&ktmp, knn_temp_bytes(nq)));
-    const KnnGrid fine = S.fine.view(), coarse = S.coarse.view();
-    launch_knn(q, nq, ref, nr, fine, S.has_coarse ? &coarse : nullptr, k, keff, self_mode,
-               out_idx, out_d2, ktmp, s);
+    const float4 *qpts = self_mode ? S.fine.pts : qorder ? qorder->pts : nullptr;
+    const uint32_t *open = launch_knn(q, qpts, nq, nr, S.fine.view(), k, keff, self_mode, out_idx,
+                                      out_d2, ktmp, s);
+    Grid coarse = S.coarse;
+    if (coarse_on_demand(S) && nr > 0) PBR_TRY(fill_grid(tb, ref, nr, coarse, open, s));
+    const KnnGrid cv = coarse.view();
+    launch_knn_rest(q, nq, ref, nr, S.has_coarse ? &cv : nullptr, k, keff, self_mode, out_idx,
+                    out_d2, ktmp, s);
     return PBR_OK;
 }
 
@@ -166,8 +159,8 @@ extern "C" int pbr_knn(pbr_ctx *ctx, const float *ref_pos, int64_t n_ref, const 
     SearchIndex S;
     PBR_TRY(make_params(tb, ref_pos, n_ref, grid_n > 0 ? grid_n : auto_cells(n_ref), S, s));
     PBR_TRY(index_points(tb, ref_pos, n_ref, S, s));
-    PBR_TRY(run_knn(tb, query_pos, n_query, ref_pos, n_ref, S, k, keff, self ? 1 : 0, out_idx,
-                    out_d2, s));
+    PBR_TRY(run_knn(tb, query_pos, n_query, nullptr, ref_pos, n_ref, S, k, keff, self ? 1 : 0,
+                    out_idx, out_d2, s));
     PBR_CUDA(cudaGetLastError());
     return PBR_OK;
 }
@@ -247,7 +240,7 @@ extern "C" int pbr_refine_points(pbr_ctx *ctx, const pbr_points *in, const pbr_r
         PBR_TRY(tb.alloc(&nd2, sizeof(float) * k * m));
         {
             StageScope sc(ctx, STG_KNN, s);
-            PBR_TRY(run_knn(tb, R.pos, m, R.pos, m, S, k, keff, 1, nidx, nd2, s));
+            PBR_TRY(run_knn(tb, R.pos, m, nullptr, R.pos, m, S, k, keff, 1, nidx, nd2, s));
         }
         StageScope sc(ctx, STG_REFINE_OTHER, s);
         launch_outlier_flags(nd2, m, k, keff, cfg->eps, keep, s);
@@ -275,7 +268,7 @@ extern "C" int pbr_refine_points(pbr_ctx *ctx, const pbr_points *in, const pbr_r
     if (keff3 > 0) {
         if ((cfg->stages & 2) && m2 < m) {
             StageScope sc(ctx, STG_REFINE_OTHER, s);
-            PBR_TRY(keep_points(tb, S, m, m2, keep, newpos, stmp, s));
+            PBR_TRY(index_points(tb, out_pos, m2, S, s)); // the survivors, same cube
         }
         int32_t *nidx;
         float *nd2;
@@ -283,7 +276,7 @@ extern "C" int pbr_refine_points(pbr_ctx *ctx, const pbr_points *in, const pbr_r
         PBR_TRY(tb.alloc(&nd2, sizeof(float) * k * m2));
         {
             StageScope sc(ctx, STG_KNN, s);
-            PBR_TRY(run_knn(tb, out_pos, m2, out_pos, m2, S, k, keff3, 1, nidx, nd2, s));
+            PBR_TRY(run_knn(tb, out_pos, m2, nullptr, out_pos, m2, S, k, keff3, 1, nidx, nd2, s));
         }
         StageScope sc(ctx, STG_REFINE_OTHER, s);
         launch_generate(nidx, m2, k, keff3,

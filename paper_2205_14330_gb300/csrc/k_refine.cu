@@ -11,22 +11,31 @@
 // whose parameters are the run's means, one warp per voxel with lanes over
 // the parameters, compensated fp32 sums in ascending input index.
 //
-// kNN: one warp per query; lane j holds the j-th best (d2, index) so far,
-// d2 = (dx dx + dy dy) + dz dz in fp32 round-to-nearest, ties by lower
-// index.  The search visits cubic shells of cells around the query's cell,
-// r = r0, r0 + 1, ...; shell r is (2r+1)^2 rows along x (a whole row where
-// |dy| or |dz| is r, else the row's two end cells), one row per lane.  The
-// points of a run of consecutive cells are a contiguous slice of the
-// id-sorted array, read from a dense cell-start table (binary search when
-// the grid is too large for one).  Runs of up to 32 points are walked by
-// their lanes side by side, longer ones by the whole warp.  Once shell r is
+// kNN: d2 = (dx dx + dy dy) + dz dz in fp32 round-to-nearest, ties by lower
+// index.  The reference points lie in cell order as {x, y, z, index} (a
+// counting sort: the order inside a cell is arbitrary, and the result does
+// not depend on it), with a dense cell-start table, so the points of a run of
+// consecutive cells are a contiguous slice.  A search visits cubic shells of
+// cells around the query's cell; shell r is (2r+1)^2 rows along x (a whole row
+// where |dy| or |dz| is r, else the row's two end cells).  Once shell r is
 // done every unvisited point lies beyond a face of the visited cube of
 // cells, so the search stops when the K-th best d2 is below the squared
 // distance to the nearest such face (less a relative slack for the
 // roundings of d2 and an absolute one for the cell coordinates), or when
-// every cell has been seen.  A query still open after a fixed number of
-// shells (neighbours across a wide empty region) is finished by an
-// exhaustive scan, one block per query.
+// every cell has been seen.  Three kernels, each taking the queries the one
+// before leaves open:
+//   - one thread per query (knn_thread_kernel): the query's list in registers,
+//     a few shells, rows beyond the K-th best skipped; queries in cell order
+//     where there is one, so that a warp's lanes walk the same rows;
+//   - one warp per query (knn_kernel) on a grid 8 times coarser, built only
+//     when a query is left open: lane j holds the j-th best so far, one row per
+//     lane; runs of up to 32 points are walked by their lanes side by side,
+//     longer ones by the whole warp;
+//   - an exhaustive scan, one block per query (neighbours across a wide
+//     empty region).
+// Sets too small for the first kernel, lists above its 16 entries and grids
+// too large for a cell table (binary search over the sorted ids) start with a
+// warp per query.
 //
 // Outlier removal: per point, the population standard deviation of its K
 // neighbour distances, fp32 sums in neighbour order; survivors are
@@ -103,16 +112,36 @@ bbox_partial_kernel(const float *__restrict__ pos, int64_t n, float *__restrict_
     }
 }
 
-__global__ void grid_params_kernel(const float *__restrict__ part, int n_parts, int n_cells,
-                                   GridParams *gp)
+// One block: the box of the partial boxes (minima and maxima, so the order
+// does not matter) and the grid over it.  A single thread walking the 608
+// partial boxes took 43 us, more than any other kernel of a small search.
+__global__ void __launch_bounds__(BBOX_THREADS)
+grid_params_kernel(const float *__restrict__ part, int n_parts, int n_cells, GridParams *gp)
 {
-    if (threadIdx.x != 0) return;
-    float lo[3] = {FLT_MAX, FLT_MAX, FLT_MAX}, hi[3] = {-FLT_MAX, -FLT_MAX, -FLT_MAX};
-    for (int b = 0; b < n_parts; ++b)
-        for (int a = 0; a < 3; ++a) {
-            lo[a] = fminf(lo[a], part[6 * b + a]);
-            hi[a] = fmaxf(hi[a], part[6 * b + 3 + a]);
+    __shared__ float s_v[6][BBOX_THREADS / 32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+#pragma unroll
+    for (int a = 0; a < 6; ++a) {
+        float v = a < 3 ? FLT_MAX : -FLT_MAX;
+        for (int b = threadIdx.x; b < n_parts; b += BBOX_THREADS)
+            v = a < 3 ? fminf(v, part[6 * b + a]) : fmaxf(v, part[6 * b + a]);
+        for (int o = 16; o > 0; o >>= 1) {
+            const float t = __shfl_xor_sync(FULL, v, o);
+            v = a < 3 ? fminf(v, t) : fmaxf(v, t);
         }
+        if (lane == 0) s_v[a][w] = v;
+    }
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    float lo[3], hi[3];
+    for (int a = 0; a < 3; ++a) {
+        lo[a] = s_v[a][0];
+        hi[a] = s_v[3 + a][0];
+        for (int j = 1; j < BBOX_THREADS / 32; ++j) {
+            lo[a] = fminf(lo[a], s_v[a][j]);
+            hi[a] = fmaxf(hi[a], s_v[3 + a][j]);
+        }
+    }
     float side = 0.0f, amax = 0.0f;
     for (int a = 0; a < 3; ++a) {
         side = fmaxf(side, __fsub_rn(hi[a], lo[a]));
@@ -126,6 +155,14 @@ __global__ void grid_params_kernel(const float *__restrict__ part, int n_parts, 
     gp->slack = 4.0e-6f * (side + amax);
 }
 
+__device__ __forceinline__ uint32_t cell_id(const GridParams &g, float x, float y, float z)
+{
+    const int ix = cell_coord(x, g.lo[0], g.h, g.n, true);
+    const int iy = cell_coord(y, g.lo[1], g.h, g.n, true);
+    const int iz = cell_coord(z, g.lo[2], g.h, g.n, true);
+    return ((uint32_t)iz * (uint32_t)g.n + (uint32_t)iy) * (uint32_t)g.n + (uint32_t)ix;
+}
+
 __global__ void cell_ids_kernel(const float *__restrict__ pos, int64_t n,
                                 const GridParams *__restrict__ gp, uint32_t *__restrict__ keys,
                                 uint32_t *__restrict__ vals)
@@ -133,11 +170,93 @@ __global__ void cell_ids_kernel(const float *__restrict__ pos, int64_t n,
     const GridParams g = *gp;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x) {
-        const int ix = cell_coord(pos[3 * i], g.lo[0], g.h, g.n, true);
-        const int iy = cell_coord(pos[3 * i + 1], g.lo[1], g.h, g.n, true);
-        const int iz = cell_coord(pos[3 * i + 2], g.lo[2], g.h, g.n, true);
-        keys[i] = ((uint32_t)iz * (uint32_t)g.n + (uint32_t)iy) * (uint32_t)g.n + (uint32_t)ix;
+        keys[i] = cell_id(g, pos[3 * i], pos[3 * i + 1], pos[3 * i + 2]);
         vals[i] = (uint32_t)i;
+    }
+}
+
+// Points in cell order by counting: points per cell into table[cell + 1],
+// the exclusive scan of those turns table[cell + 1] into the first slot of
+// `cell`, and the scatter's atomics move it past its last point, which is
+// the first slot of cell + 1: table[c] ends as the start of cell c.
+// gate: when set, the kernels do nothing while *gate is 0.
+__global__ void cell_hist_kernel(const float *__restrict__ pos, int64_t n,
+                                 const GridParams *__restrict__ gp, uint32_t *__restrict__ ids,
+                                 uint32_t *__restrict__ table, const uint32_t *gate)
+{
+    if (gate && *gate == 0) return;
+    const GridParams g = *gp;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        const uint32_t c = cell_id(g, pos[3 * i], pos[3 * i + 1], pos[3 * i + 2]);
+        ids[i] = c;
+        atomicAdd(table + 1 + c, 1u);
+    }
+}
+
+__global__ void cell_scatter_kernel(const float *__restrict__ pos, int64_t n,
+                                    const uint32_t *__restrict__ ids, uint32_t *__restrict__ table,
+                                    float4 *__restrict__ pts, const uint32_t *gate)
+{
+    if (gate && *gate == 0) return;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+         i += (int64_t)gridDim.x * blockDim.x)
+        pts[atomicAdd(table + 1 + ids[i], 1u)] =
+            make_float4(pos[3 * i], pos[3 * i + 1], pos[3 * i + 2], __uint_as_float((uint32_t)i));
+}
+
+// Exclusive scan of p[0..n) in place by one block, for tables small enough
+// (GATED_CELLS) that three launches would cost more.
+__global__ void __launch_bounds__(1024) gated_scan_kernel(uint32_t *p, int n, const uint32_t *gate)
+{
+    if (gate && *gate == 0) return;
+    __shared__ uint32_t s_w[32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    uint32_t run = 0;
+    for (int base = 0; base < n; base += 4096) {
+        const int i = base + 4 * (int)threadIdx.x;
+        uint32_t v[4], sum = 0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            v[k] = i + k < n ? p[i + k] : 0u;
+            sum += v[k];
+        }
+        uint32_t inc = sum;
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t t = __shfl_up_sync(FULL, inc, o);
+            if (lane >= o) inc += t;
+        }
+        if (lane == 31) s_w[w] = inc;
+        __syncthreads();
+        if (w == 0) {
+            uint32_t x = s_w[lane];
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t t = __shfl_up_sync(FULL, x, o);
+                if (lane >= o) x += t;
+            }
+            s_w[lane] = x;
+        }
+        __syncthreads();
+        uint32_t at = run + inc - sum + (w > 0 ? s_w[w - 1] : 0u);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            if (i + k < n) p[i + k] = at;
+            at += v[k];
+        }
+        run += s_w[31];
+        __syncthreads();
+    }
+}
+
+// Points in the order of a sorted (id, index) list (grids without a table).
+__global__ void gather_points_kernel(const float *__restrict__ pos, const uint32_t *__restrict__ idx,
+                                     int64_t n, float4 *__restrict__ pts)
+{
+    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < n;
+         j += (int64_t)gridDim.x * blockDim.x) {
+        const uint32_t i = idx[j];
+        pts[j] = make_float4(pos[3 * (size_t)i], pos[3 * (size_t)i + 1], pos[3 * (size_t)i + 2],
+                             __uint_as_float(i));
     }
 }
 
@@ -290,17 +409,16 @@ __device__ __forceinline__ void cell_range(const uint32_t *__restrict__ cs,
     t = hi;
 }
 
-// Candidate j of the sorted list against the query: squared distance and
-// whether it would enter the current list.
-__device__ __forceinline__ bool knn_candidate(uint32_t j, const uint32_t *__restrict__ ridx,
-                                              const float *__restrict__ rpos, float qx, float qy,
-                                              float qz, uint32_t self_idx, float kd, uint32_t ki,
-                                              float &d2, uint32_t &ri)
+// Candidate j of the points in cell order against the query: squared
+// distance and whether it would enter the current list.
+__device__ __forceinline__ bool knn_candidate(uint32_t j, const float4 *__restrict__ pts, float qx,
+                                              float qy, float qz, uint32_t self_idx, float kd,
+                                              uint32_t ki, float &d2, uint32_t &ri)
 {
-    ri = __ldg(ridx + j);
+    const float4 c = __ldg(pts + j);
+    ri = __float_as_uint(c.w);
     if (ri == self_idx) return false;
-    d2 = sq_dist(qx, qy, qz, __ldg(rpos + 3 * (size_t)ri), __ldg(rpos + 3 * (size_t)ri + 1),
-                 __ldg(rpos + 3 * (size_t)ri + 2));
+    d2 = sq_dist(qx, qy, qz, c.x, c.y, c.z);
     return d2 < kd || (d2 == kd && ri < ki);
 }
 
@@ -338,6 +456,22 @@ __device__ __forceinline__ float unvisited_bound(const GridParams &g, int r, int
     return bound == FLT_MAX ? FLT_MAX : bound * 0.99999f - g.slack;
 }
 
+// Lower bound on the distance along one axis from coordinate p to cell c of
+// the grid (the slack as in unvisited_bound).
+__device__ __forceinline__ float cell_gap(const GridParams &g, float p, float lo, int c)
+{
+    const float d = fmaxf((lo + (float)c * g.h) - p, p - (lo + (float)(c + 1) * g.h));
+    return fmaxf(d * 0.99999f - g.slack, 0.0f);
+}
+
+// Whether row (y, z) of cells may hold a point as near as squared distance kd.
+__device__ __forceinline__ bool row_open(const GridParams &g, float qy, float qz, int y, int z,
+                                         float kd)
+{
+    const float a = cell_gap(g, qy, g.lo[1], y), b = cell_gap(g, qz, g.lo[2], z);
+    return !(__fadd_rn(__fmul_rn(a, a), __fmul_rn(b, b)) > kd);
+}
+
 // Writes the warp's list (lane j = j-th best) as row q of the output.
 __device__ __forceinline__ void knn_write(int64_t q, int k, int keff, int lane, float bd,
                                           uint32_t bi, int32_t *__restrict__ out_idx,
@@ -363,13 +497,12 @@ constexpr int KNN_MAX_SHELLS = 16;
 // *n_defer) and their rows left unwritten.
 __global__ void __launch_bounds__(256)
 knn_kernel(const float *__restrict__ qpos, int64_t nq_all, const uint32_t *__restrict__ qlist,
-           const uint32_t *__restrict__ nq_dev, const float *__restrict__ rpos, uint32_t nr,
-           KnnGrid grid, int k, int keff, int self_mode, int32_t *__restrict__ out_idx,
+           const uint32_t *__restrict__ nq_dev, uint32_t nr, KnnGrid grid, int k, int keff, int self_mode, int32_t *__restrict__ out_idx,
            float *__restrict__ out_d2, uint32_t *__restrict__ defer, uint32_t *__restrict__ n_defer)
 {
     const GridParams g = *grid.gp;
     const uint32_t *__restrict__ rid = grid.rid;
-    const uint32_t *__restrict__ ridx = grid.ridx;
+    const float4 *__restrict__ pts = grid.pts;
     const uint32_t *__restrict__ cs = grid.cs;
     const int lane = threadIdx.x & 31;
     const int n = g.n;
@@ -399,8 +532,9 @@ knn_kernel(const float *__restrict__ qpos, int64_t nq_all, const uint32_t *__res
                     // this lane's row: up to two index ranges of the sorted list
                     const int row = base + lane;
                     uint32_t s0 = 0, t0 = 0, s1 = 0, t1 = 0;
-                    if (row < rows) {
-                        const int dy = dy0 + row % ny, dz = dz0 + row / ny;
+                    const int dy = dy0 + row % ny, dz = dz0 + row / ny;
+                    // rows beyond the K-th best are skipped
+                    if (row < rows && row_open(g, qy, qz, cy + dy, cz + dz, kd)) {
                         const uint32_t rb =
                             ((uint32_t)(cz + dz) * (uint32_t)n + (uint32_t)(cy + dy)) * (uint32_t)n;
                         if (abs(dy) == r || abs(dz) == r) {
@@ -430,8 +564,8 @@ knn_kernel(const float *__restrict__ qpos, int64_t nq_all, const uint32_t *__res
                                 const uint32_t j = j0 + lane;
                                 float d2 = FLT_MAX;
                                 uint32_t ri = 0;
-                                const bool better = j < re && knn_candidate(j, ridx, rpos, qx, qy, qz,
-                                                                            self_idx, kd, ki, d2, ri);
+                                const bool better = j < re && knn_candidate(j, pts, qx, qy, qz, self_idx, kd,
+                                                                            ki, d2, ri);
                                 knn_insert_all(__ballot_sync(FULL, better), d2, ri, bd, bi, keff,
                                                kmask, lane, kd, ki);
                             }
@@ -448,7 +582,7 @@ knn_kernel(const float *__restrict__ qpos, int64_t nq_all, const uint32_t *__res
                         bool better = false;
                         if (has) {
                             const uint32_t j = s0 < t0 ? s0++ : s1++;
-                            better = knn_candidate(j, ridx, rpos, qx, qy, qz, self_idx, kd, ki, d2, ri);
+                            better = knn_candidate(j, pts, qx, qy, qz, self_idx, kd, ki, d2, ri);
                         }
                         knn_insert_all(__ballot_sync(FULL, better), d2, ri, bd, bi, keff, kmask,
                                        lane, kd, ki);
@@ -465,6 +599,145 @@ knn_kernel(const float *__restrict__ qpos, int64_t nq_all, const uint32_t *__res
             }
         }
         if (keff_done) knn_write(q, k, keff, lane, bd, bi, out_idx, out_d2);
+    }
+}
+
+// One thread per query, on grids with a cell table: the first shells of the
+// search, up to KT (>= k) entries in registers.  Rows of cells whose slab is
+// farther away than the K-th best are skipped.  Queries come from qpts (a
+// cloud in cell order, {x, y, z, index}) or, without one, from qpos in the
+// order given; self: the queries are the reference points.  Queries still
+// open after THREAD_SHELLS shells are appended to `defer`.
+// A warp per query spends its 32 lanes on the few points of a cell and an
+// insertion per accepted point on the whole warp; a thread per query keeps
+// 32 queries of neighbouring cells in one warp, whose lanes read the same
+// rows.  Bound by the latency of its gathers (the nine slices' bounds are
+// loaded together).  200k points on surfaces, nearest point: 325 -> 36 us a
+// search; 1M-point cloud reduced to its voxels with 1% outliers, 8 nearest:
+// 1410 -> 310 us (134 here, 175 on the coarse grid for the outliers; 238
+// there before it skipped rows; three shells here: 174 and no fewer left).
+constexpr int THREAD_SHELLS = 2;
+
+template <int KT>
+__global__ void __launch_bounds__(128)
+knn_thread_kernel(const float4 *__restrict__ qpts, const float *__restrict__ qpos, int64_t nq,
+                  KnnGrid grid, int k, int keff, int self_mode, int32_t *__restrict__ out_idx,
+                  float *__restrict__ out_d2, uint32_t *__restrict__ defer,
+                  uint32_t *__restrict__ n_defer)
+{
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= nq) return;
+    const GridParams g = *grid.gp;
+    const float4 *__restrict__ pts = grid.pts;
+    const uint32_t *__restrict__ cs = grid.cs;
+    const int n = g.n;
+    float qx, qy, qz;
+    uint32_t q;
+    if (qpts) {
+        const float4 v = __ldg(qpts + t);
+        qx = v.x;
+        qy = v.y;
+        qz = v.z;
+        q = __float_as_uint(v.w);
+    } else {
+        qx = __ldg(qpos + 3 * t);
+        qy = __ldg(qpos + 3 * t + 1);
+        qz = __ldg(qpos + 3 * t + 2);
+        q = (uint32_t)t;
+    }
+    const uint32_t self_idx = self_mode ? q : 0xffffffffu;
+    float bd[KT];
+    uint32_t bi[KT];
+#pragma unroll
+    for (int m = 0; m < KT; ++m) {
+        bd[m] = FLT_MAX;
+        bi[m] = 0xffffffffu;
+    }
+    const int cx = cell_coord(qx, g.lo[0], g.h, n, self_mode);
+    const int cy = cell_coord(qy, g.lo[1], g.h, n, self_mode);
+    const int cz = cell_coord(qz, g.lo[2], g.h, n, self_mode);
+
+    // the points of slots [s, e): bubble each through the sorted list
+    auto visit = [&](uint32_t s, uint32_t e) {
+        for (uint32_t j = s; j < e; ++j) {
+            const float4 c = __ldg(pts + j);
+            uint32_t ri = __float_as_uint(c.w);
+            float d2 = sq_dist(qx, qy, qz, c.x, c.y, c.z);
+            if (ri == self_idx || !(d2 < bd[KT - 1] || (d2 == bd[KT - 1] && ri < bi[KT - 1])))
+                continue;
+#pragma unroll
+            for (int m = 0; m < KT; ++m) {
+                const bool before = d2 < bd[m] || (d2 == bd[m] && ri < bi[m]);
+                const float od = bd[m];
+                const uint32_t oi = bi[m];
+                bd[m] = before ? d2 : od;
+                bi[m] = before ? ri : oi;
+                d2 = before ? od : d2;
+                ri = before ? oi : ri;
+            }
+        }
+    };
+    // whether row (y, z) of cells meets the grid and may hold a better point
+    auto open = [&](int y, int z) {
+        return y >= 0 && y < n && z >= 0 && z < n && row_open(g, qy, qz, y, z, bd[KT - 1]);
+    };
+    auto row_base = [&](int y, int z) { return ((uint32_t)z * (uint32_t)n + (uint32_t)y) * (uint32_t)n; };
+    auto settled = [&](int r) {
+        const float bound = unvisited_bound(g, r, cx, cy, cz, qx, qy, qz);
+        if (bound == FLT_MAX) return true; // every cell visited
+        return bd[KT - 1] < FLT_MAX && bound > 0.0f && bd[KT - 1] < __fmul_rn(bound, bound);
+    };
+
+    bool done = keff == 0;
+    if (!done) { // shells 0 and 1: the nine rows' slices first, the query's own row leading
+        constexpr int OY[9] = {0, -1, 1, 0, 0, -1, -1, 1, 1}, OZ[9] = {0, 0, 0, -1, 1, -1, 1, -1, 1};
+        const int x0 = max(cx - 1, 0), x1 = min(cx + 1, n - 1);
+        uint32_t s[9], e[9];
+#pragma unroll
+        for (int i = 0; i < 9; ++i) {
+            const int y = cy + OY[i], z = cz + OZ[i];
+            const bool in = x0 <= x1 && y >= 0 && y < n && z >= 0 && z < n;
+            const uint32_t rb = in ? row_base(y, z) : 0u;
+            s[i] = in ? __ldg(cs + rb + (uint32_t)x0) : 0u;
+            e[i] = in ? __ldg(cs + rb + (uint32_t)x1 + 1) : 0u;
+        }
+#pragma unroll
+        for (int i = 0; i < 9; ++i)
+            if (s[i] < e[i] && open(cy + OY[i], cz + OZ[i])) visit(s[i], e[i]);
+        done = settled(1);
+    }
+    for (int r = 2; r <= THREAD_SHELLS && !done; ++r) {
+        const int x0 = max(cx - r, 0), x1 = min(cx + r, n - 1);
+        for (int dz = -r; dz <= r; ++dz)
+            for (int dy = -r; dy <= r; ++dy) {
+                if (!open(cy + dy, cz + dz)) continue;
+                const uint32_t rb = row_base(cy + dy, cz + dz);
+                if (abs(dy) == r || abs(dz) == r) {
+                    if (x0 <= x1) visit(__ldg(cs + rb + (uint32_t)x0), __ldg(cs + rb + (uint32_t)x1 + 1));
+                } else {
+                    if (cx - r >= 0 && cx - r < n)
+                        visit(__ldg(cs + rb + (uint32_t)(cx - r)), __ldg(cs + rb + (uint32_t)(cx - r) + 1));
+                    if (cx + r >= 0 && cx + r < n)
+                        visit(__ldg(cs + rb + (uint32_t)(cx + r)), __ldg(cs + rb + (uint32_t)(cx + r) + 1));
+                }
+            }
+        done = settled(r);
+    }
+    if (!done) {
+        defer[atomicAdd(n_defer, 1u)] = q;
+        return;
+    }
+    for (int m = 0; m < k; ++m) { // entries past the list stay padding
+        int32_t oi = -1;
+        float od = FLT_MAX;
+#pragma unroll
+        for (int j = 0; j < KT; ++j)
+            if (j == m && m < keff) {
+                oi = (int32_t)bi[j];
+                od = bd[j];
+            }
+        out_idx[(int64_t)q * k + m] = oi;
+        out_d2[(int64_t)q * k + m] = od;
     }
 }
 
@@ -517,14 +790,6 @@ knn_exhaustive_kernel(const float *__restrict__ qpos, const float *__restrict__ 
     }
 }
 
-__global__ void cell_count_kernel(const uint32_t *__restrict__ rid, int64_t n,
-                                  uint32_t *__restrict__ count)
-{
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x)
-        atomicAdd(count + rid[i], 1u);
-}
-
 // ---------------------------------------------------------- outliers
 __global__ void outlier_flags_kernel(const float *__restrict__ d2, int64_t n, int k, int keff,
                                      float eps, uint32_t *__restrict__ keep)
@@ -561,32 +826,6 @@ compact_points_kernel(const uint32_t *__restrict__ keep, const uint32_t *__restr
         if (!keep[i]) continue;
         const int64_t o = pos[i];
         for (int a = lane; a < nattr; a += 32) out.put(o, a, in.get((uint32_t)i, a));
-    }
-}
-
-// The sorted (cell id, index) list restricted to kept points, indices
-// renumbered: flags[j] = keep[idx[j]] first, then the scatter.
-__global__ void list_keep_kernel(const uint32_t *__restrict__ ridx, const uint32_t *__restrict__ keep,
-                                 int64_t n, uint32_t *__restrict__ flags)
-{
-    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < n;
-         j += (int64_t)gridDim.x * blockDim.x)
-        flags[j] = keep[ridx[j]];
-}
-
-__global__ void list_compact_kernel(const uint32_t *__restrict__ rid, const uint32_t *__restrict__ ridx,
-                                    const uint32_t *__restrict__ keep,
-                                    const uint32_t *__restrict__ newpos,
-                                    const uint32_t *__restrict__ lpos, int64_t n,
-                                    uint32_t *__restrict__ rid_out, uint32_t *__restrict__ ridx_out)
-{
-    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < n;
-         j += (int64_t)gridDim.x * blockDim.x) {
-        const uint32_t i = ridx[j];
-        if (keep[i]) {
-            rid_out[lpos[j]] = rid[j];
-            ridx_out[lpos[j]] = newpos[i];
-        }
     }
 }
 
@@ -636,7 +875,7 @@ void launch_grid_params(const float *pos, int64_t n, int n_cells, GridParams *gp
     float *part = (float *)temp;
     const unsigned blocks = grid_for(n, BBOX_THREADS, BBOX_PARTS);
     bbox_partial_kernel<<<blocks, BBOX_THREADS, 0, s>>>(pos, n, part);
-    grid_params_kernel<<<1, 32, 0, s>>>(part, (int)blocks, n_cells, gp);
+    grid_params_kernel<<<1, BBOX_THREADS, 0, s>>>(part, (int)blocks, n_cells, gp);
     count_launches(2);
 }
 
@@ -671,39 +910,93 @@ void launch_voxel_mean(const uint32_t *order, const uint32_t *starts, int64_t n_
 
 size_t knn_temp_bytes(int64_t nq) { return sizeof(uint32_t) * (size_t)(2 * nq + 2); }
 
-void launch_knn(const float *qpos, int64_t nq, const float *rpos, int64_t nr, const KnnGrid &fine,
-                const KnnGrid *coarse, int k, int keff, int self_mode, int32_t *out_idx,
-                float *out_d2, void *temp, cudaStream_t s)
+// Queries per search from which a thread per query is the faster start: 4096
+// for each entry of its list, at least 8192.  Below, its few warps leave most
+// SMs idle, and the longer a thread's list the longer its insertions (a whole
+// self search, thread / warp per query, in us; k = 1: 8k points 96 / 98, 16k
+// 86 / 91, 64k 83 / 148; k = 8: 16k 121 / 109, 64k 128 / 198; k = 16: 64k
+// 277 / 253, 300k 450 / 1002).
+inline bool thread_per_query(int64_t nq, int k) { return nq >= 4096 * (int64_t)(k > 2 ? k : 2); }
+
+namespace {
+
+template <int KT>
+void thread_search(const float4 *qpts, const float *qpos, int64_t nq, const KnnGrid &g, int k,
+                   int keff, int self_mode, int32_t *out_idx, float *out_d2, uint32_t *defer,
+                   uint32_t *n_defer, cudaStream_t s)
 {
-    if (nq <= 0) return;
-    uint32_t *cnt = (uint32_t *)temp, *d1 = cnt + 2, *d2 = d1 + nq;
+    knn_thread_kernel<KT><<<(unsigned)((nq + 127) / 128), 128, 0, s>>>(
+        qpts, qpos, nq, g, k, keff, self_mode, out_idx, out_d2, defer, n_defer);
+}
+
+} // namespace
+
+const uint32_t *launch_knn(const float *qpos, const float4 *qpts, int64_t nq, int64_t nr,
+                           const KnnGrid &fine, int k, int keff, int self_mode, int32_t *out_idx,
+                           float *out_d2, void *temp, cudaStream_t s)
+{
+    uint32_t *cnt = (uint32_t *)temp, *d1 = cnt + 2;
     cudaMemsetAsync(cnt, 0, 2 * sizeof(uint32_t), s);
-    knn_kernel<<<grid_for(nq, 8, MAX_BLOCKS), 256, 0, s>>>(qpos, nq, nullptr, nullptr, rpos,
-                                                          (uint32_t)nr, fine, k, keff, self_mode,
-                                                          out_idx, out_d2, d1, cnt);
+    if (thread_per_query(nq, k) && k <= 16 && fine.cs) {
+        auto f = k == 1   ? thread_search<1>
+                 : k == 2 ? thread_search<2>
+                 : k <= 4 ? thread_search<4>
+                 : k <= 8 ? thread_search<8>
+                 : k <= 12 ? thread_search<12>
+                           : thread_search<16>;
+        f(qpts, qpos, nq, fine, k, keff, self_mode, out_idx, out_d2, d1, cnt, s);
+    } else {
+        knn_kernel<<<grid_for(nq, 8, MAX_BLOCKS), 256, 0, s>>>(qpos, nq, nullptr, nullptr,
+                                                              (uint32_t)nr, fine, k, keff,
+                                                              self_mode, out_idx, out_d2, d1, cnt);
+    }
+    count_launches(1);
+    return cnt;
+}
+
+void launch_knn_rest(const float *qpos, int64_t nq, const float *rpos, int64_t nr,
+                     const KnnGrid *coarse, int k, int keff, int self_mode, int32_t *out_idx,
+                     float *out_d2, void *temp, cudaStream_t s)
+{
+    uint32_t *cnt = (uint32_t *)temp, *d1 = cnt + 2, *d2 = d1 + nq;
     const uint32_t *last = d1, *n_last = cnt;
     if (coarse) {
-        knn_kernel<<<grid_for(nq, 8, 152 * 8), 256, 0, s>>>(qpos, 0, d1, cnt, rpos, (uint32_t)nr,
-                                                          *coarse, k, keff, self_mode, out_idx,
-                                                          out_d2, d2, cnt + 1);
+        knn_kernel<<<grid_for(nq, 8, 152 * 8), 256, 0, s>>>(qpos, 0, d1, cnt, (uint32_t)nr, *coarse,
+                                                          k, keff, self_mode, out_idx, out_d2, d2,
+                                                          cnt + 1);
         last = d2;
         n_last = cnt + 1;
         count_launches(1);
     }
     knn_exhaustive_kernel<<<304, 256, 0, s>>>(qpos, rpos, (uint32_t)nr, k, keff, self_mode, last,
                                               n_last, out_idx, out_d2);
+    count_launches(1);
+}
+
+void launch_cell_sort(const float *pos, int64_t n, const GridParams *gp, int64_t n_cells_total,
+                      uint32_t *ids, uint32_t *table, float4 *pts, void *scan_temp,
+                      const uint32_t *gate, cudaStream_t s)
+{
+    cudaMemsetAsync(table, 0, sizeof(uint32_t) * (size_t)(n_cells_total + 1), s);
+    if (n <= 0) return;
+    const unsigned g = grid_for(n, 256, MAX_BLOCKS);
+    cell_hist_kernel<<<g, 256, 0, s>>>(pos, n, gp, ids, table, gate);
+    if (n_cells_total <= GATED_CELLS) {
+        gated_scan_kernel<<<1, 1024, 0, s>>>(table + 1, (int)n_cells_total, gate);
+        count_launches(1);
+    } else {
+        launch_exclusive_scan(table + 1, table + 1, n_cells_total, nullptr, scan_temp, s);
+    }
+    cell_scatter_kernel<<<g, 256, 0, s>>>(pos, n, ids, table, pts, gate);
     count_launches(2);
 }
 
-void launch_cell_start(const uint32_t *rid, int64_t n, int64_t n_cells_total,
-                       uint32_t *cell_start, void *scan_temp, cudaStream_t s)
+void launch_gather_points(const float *pos, const uint32_t *idx, int64_t n, float4 *pts,
+                          cudaStream_t s)
 {
-    cudaMemsetAsync(cell_start, 0, sizeof(uint32_t) * (size_t)(n_cells_total + 1), s);
-    if (n > 0) {
-        cell_count_kernel<<<grid_for(n, 256, MAX_BLOCKS), 256, 0, s>>>(rid, n, cell_start);
-        count_launches(1);
-    }
-    launch_exclusive_scan(cell_start, cell_start, n_cells_total + 1, nullptr, scan_temp, s);
+    if (n <= 0) return;
+    gather_points_kernel<<<grid_for(n, 256, MAX_BLOCKS), 256, 0, s>>>(pos, idx, n, pts);
+    count_launches(1);
 }
 
 void launch_outlier_flags(const float *d2, int64_t n, int k, int keff, float eps, uint32_t *keep,
@@ -722,18 +1015,6 @@ void launch_compact_points(const uint32_t *keep, const uint32_t *pos, int64_t n,
         keep, pos, n, Params{in.pos, in.sh, in.op, in.rad, in.nsh},
         OutParams{out.pos, out.sh, out.op, out.rad, out.nsh});
     count_launches(1);
-}
-
-void launch_list_keep(const uint32_t *rid, const uint32_t *ridx, const uint32_t *keep,
-                      const uint32_t *newpos, int64_t n, uint32_t *flags, uint32_t *rid_out,
-                      uint32_t *ridx_out, void *scan_temp, cudaStream_t s)
-{
-    if (n <= 0) return;
-    const unsigned g = grid_for(n, 256, MAX_BLOCKS);
-    list_keep_kernel<<<g, 256, 0, s>>>(ridx, keep, n, flags);
-    launch_exclusive_scan(flags, flags, n, nullptr, scan_temp, s);
-    list_compact_kernel<<<g, 256, 0, s>>>(rid, ridx, keep, newpos, flags, n, rid_out, ridx_out);
-    count_launches(2);
 }
 
 void launch_fill_u32(uint32_t *p, int64_t n, uint32_t v, cudaStream_t s)

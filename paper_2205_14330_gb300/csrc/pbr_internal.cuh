@@ -268,33 +268,42 @@ void launch_run_starts(const uint32_t *keys, int64_t n, uint32_t *flags, uint32_
                        unsigned long long *n_runs, void *scan_temp, cudaStream_t s);
 void launch_voxel_mean(const uint32_t *order, const uint32_t *starts, int64_t n_runs, int64_t n,
                        const PointArrays &in, const PointArraysOut &out, cudaStream_t s);
-// One search grid over the reference points: parameters, (cell id, index)
-// list sorted by id, dense cell-start table (or NULL).
+// One search grid over the reference points: parameters, the points in cell
+// order as {x, y, z, index}, the dense cell-start table (or NULL), and, without
+// a table, the sorted cell ids.
 struct KnnGrid {
     const GridParams *gp;
-    const uint32_t *rid, *ridx, *cs;
+    const float4 *pts;
+    const uint32_t *cs, *rid;
 };
 // Exact K nearest reference points per query; rows of k entries, keff =
-// entries filled.  Searches `fine`, then `coarse` (may be NULL) for queries
-// left open, then scans every point for what is still open.
+// entries filled.  launch_knn searches `fine` and returns the device counter
+// of the queries it left open (kept in temp); launch_knn_rest searches
+// `coarse` (may be NULL) for those, then scans every point for what is still
+// open.  qpts: the queries in cell order as {x, y, z, index}, or NULL.
 // temp: knn_temp_bytes(nq).
 size_t knn_temp_bytes(int64_t nq);
-void launch_knn(const float *qpos, int64_t nq, const float *rpos, int64_t nr, const KnnGrid &fine,
-                const KnnGrid *coarse, int k, int keff, int self_mode, int32_t *out_idx,
-                float *out_d2, void *temp, cudaStream_t s);
-// cell_start[c] = first index of cell c in the sorted list (c <= cells);
-// scan_temp: scan_temp_bytes(cells + 1).
-void launch_cell_start(const uint32_t *rid, int64_t n, int64_t n_cells_total,
-                       uint32_t *cell_start, void *scan_temp, cudaStream_t s);
+const uint32_t *launch_knn(const float *qpos, const float4 *qpts, int64_t nq, int64_t nr,
+                           const KnnGrid &fine, int k, int keff, int self_mode, int32_t *out_idx,
+                           float *out_d2, void *temp, cudaStream_t s);
+void launch_knn_rest(const float *qpos, int64_t nq, const float *rpos, int64_t nr,
+                     const KnnGrid *coarse, int k, int keff, int self_mode, int32_t *out_idx,
+                     float *out_d2, void *temp, cudaStream_t s);
+// Points in cell order by a counting sort: pts[n], table[c] = first slot of
+// cell c (n_cells_total + 1 entries); ids: n words of scratch; scan_temp:
+// scan_temp_bytes(n_cells_total).  gate (device, may be NULL; grids of at
+// most GATED_CELLS cells only): nothing is built while *gate is 0.
+constexpr int64_t GATED_CELLS = 1 << 16;
+void launch_cell_sort(const float *pos, int64_t n, const GridParams *gp, int64_t n_cells_total,
+                      uint32_t *ids, uint32_t *table, float4 *pts, void *scan_temp,
+                      const uint32_t *gate, cudaStream_t s);
+// pts[j] = point idx[j] as {x, y, z, index}.
+void launch_gather_points(const float *pos, const uint32_t *idx, int64_t n, float4 *pts,
+                          cudaStream_t s);
 void launch_outlier_flags(const float *d2, int64_t n, int k, int keff, float eps, uint32_t *keep,
                           cudaStream_t s);
 void launch_compact_points(const uint32_t *keep, const uint32_t *pos, int64_t n,
                            const PointArrays &in, const PointArraysOut &out, cudaStream_t s);
-// Restricts a sorted (id, index) list to kept points, renumbering indices
-// with newpos (the exclusive scan of keep).  flags: n words of scratch.
-void launch_list_keep(const uint32_t *rid, const uint32_t *ridx, const uint32_t *keep,
-                      const uint32_t *newpos, int64_t n, uint32_t *flags, uint32_t *rid_out,
-                      uint32_t *ridx_out, void *scan_temp, cudaStream_t s);
 void launch_fill_u32(uint32_t *p, int64_t n, uint32_t v, cudaStream_t s);
 // Row out_base + q of `out` = mean of the parameters of points nbr[q][0..keff)
 // of `in`, for parameters a_begin.. (0: position first; 3: SH, opacity,
