@@ -133,43 +133,44 @@ extern "C" int pbr_visual_hull_init(pbr_ctx *ctx, const float lo[3], const float
     TempBufs tb(s);
     HullView *views;
     PBR_TRY(upload_views(tb, cams, n_cams, z_near, &views, s));
-    constexpr int64_t BATCH = 1ll << 22;
-    float *cand;
-    uint32_t *flags, *rank;
-    void *stmp;
-    unsigned long long *tot, *last;
-    PBR_TRY(tb.alloc(&cand, sizeof(float) * 3 * BATCH));
-    PBR_TRY(tb.alloc(&flags, sizeof(uint32_t) * BATCH));
-    PBR_TRY(tb.alloc(&rank, sizeof(uint32_t) * BATCH));
-    PBR_TRY(tb.alloc(&stmp, scan_temp_bytes(BATCH)));
-    PBR_TRY(tb.alloc(&tot, sizeof(unsigned long long)));
-    PBR_TRY(tb.alloc(&last, sizeof(unsigned long long)));
-
-    // batches of candidates in counter order; the first n_target accepted
+    // Batches of candidates in counter order; the first n_target accepted.
+    // A batch costs a host synchronisation, candidates beyond the last one
+    // taken cost their draws: the first batch allows for one candidate in 32
+    // accepted, the next ones for the share seen so far and a little more.
+    constexpr int64_t BATCH = 1ll << 24, LEAST = 1ll << 16;
+    auto sized = [&](double want) {
+        const int64_t c = want < (double)BATCH ? (int64_t)want : BATCH;
+        return std::max(LEAST, (c + HULL_BLOCK - 1) / HULL_BLOCK * HULL_BLOCK);
+    };
+    int64_t size = sized(32.0 * (double)n_target);
+    uint32_t *bits, *counts;
+    unsigned long long *result;
+    PBR_TRY(tb.alloc(&bits, (size_t)(BATCH / 8)));
+    PBR_TRY(tb.alloc(&counts, sizeof(uint32_t) * (BATCH / HULL_BLOCK)));
+    PBR_TRY(tb.alloc(&result, 2 * sizeof(unsigned long long)));
     int64_t done = 0, drawn = 0;
     while (done < n_target && drawn < max_candidates) {
-        const int64_t cnt = std::min<int64_t>(BATCH, max_candidates - drawn);
-        launch_hull_candidates(seed, (uint64_t)drawn, cnt, lo, ext, views, n_cams, masks, z_near,
-                               cand, flags, s);
-        launch_exclusive_scan(flags, rank, cnt, tot, stmp, s);
+        const int64_t cnt = std::min<int64_t>(size, max_candidates - drawn);
         const uint32_t need = (uint32_t)(n_target - done);
-        launch_hull_take(cand, flags, rank, cnt, need, out_pos, done, last, s);
-        unsigned long long acc = 0;
-        PBR_TRY(read_u64(tot, &acc, s));
-        if ((int64_t)acc >= (int64_t)need) {
-            unsigned long long li = 0;
-            PBR_TRY(read_u64(last, &li, s));
-            drawn += (int64_t)li + 1;
+        launch_hull_batch(seed, (uint64_t)drawn, cnt, lo, ext, views, n_cams, masks, z_near, bits,
+                          counts, need, out_pos, done, result, s);
+        unsigned long long got[2] = {0, 0};
+        PBR_CUDA(cudaMemcpyAsync(got, result, sizeof got, cudaMemcpyDeviceToHost, s));
+        PBR_CUDA(cudaStreamSynchronize(s));
+        if ((int64_t)got[0] >= (int64_t)need) {
+            drawn += (int64_t)got[1] + 1;
             done = n_target;
         } else {
             drawn += cnt;
-            done += (int64_t)acc;
+            done += (int64_t)got[0];
+            size = done > 0 ? sized(1.05 * (double)(n_target - done) * (double)drawn / (double)done)
+                            : BATCH;
         }
     }
     // SH of the kept points: standard normals
     if (out_sh && done > 0) {
         const int64_t coef = 3ll * (sh_degree + 1) * (sh_degree + 1);
-        launch_sh_normals(seed ^ SH_STREAM, 0, done * coef, out_sh, s);
+        launch_sh_normals(seed ^ SH_STREAM, done * coef, out_sh, s);
     }
     *n_out = done;
     *n_drawn = drawn;

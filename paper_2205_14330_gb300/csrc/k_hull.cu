@@ -29,10 +29,12 @@ __device__ __forceinline__ float uniform24(uint64_t z)
     return (float)(uint32_t)(z >> 40) * 5.9604644775390625e-8f; // 2^-24, exact
 }
 
-__device__ bool consistent(float px, float py, float pz, const HullView *__restrict__ views,
-                           int nv, const uint8_t *__restrict__ masks, float z_near)
+// Whether the point lands on a foreground pixel of every view in [v0, v1).
+__device__ __forceinline__ bool consistent(float px, float py, float pz,
+                                           const HullView *__restrict__ views, int v0, int v1,
+                                           const uint8_t *__restrict__ masks, float z_near)
 {
-    for (int v = 0; v < nv; ++v) {
+    for (int v = v0; v < v1; ++v) {
         const HullView &V = views[v];
         float X[3];
 #pragma unroll
@@ -58,72 +60,175 @@ cc_flags_kernel(const float *__restrict__ pos, int64_t n, const HullView *__rest
 {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x) {
-        const bool ok = consistent(pos[3 * i], pos[3 * i + 1], pos[3 * i + 2], views, nv, masks,
+        const bool ok = consistent(pos[3 * i], pos[3 * i + 1], pos[3 * i + 2], views, 0, nv, masks,
                                    z_near);
         if (flags8) flags8[i] = ok ? 1 : 0;
         if (flags32) flags32[i] = ok ? 1u : 0u;
     }
 }
 
-// Candidates first .. first + count - 1: position and consistency flag.
-__global__ void __launch_bounds__(256)
-hull_candidates_kernel(uint64_t seed, uint64_t first, int64_t count, float lo0, float lo1,
-                       float lo2, float ex0, float ex1, float ex2,
-                       const HullView *__restrict__ views, int nv,
-                       const uint8_t *__restrict__ masks, float z_near, float *__restrict__ cand,
-                       uint32_t *__restrict__ flags)
+// Position of candidate j of stream `seed` in the box.
+struct HullBox {
+    uint64_t seed;
+    float lo[3], ex[3];
+};
+
+__device__ __forceinline__ void candidate(const HullBox &b, uint64_t j, float p[3])
 {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const uint64_t j = first + (uint64_t)i;
-        const float x = __fadd_rn(__fmul_rn(ex0, uniform24(splitmix64(seed, 3 * j))), lo0);
-        const float y = __fadd_rn(__fmul_rn(ex1, uniform24(splitmix64(seed, 3 * j + 1))), lo1);
-        const float z = __fadd_rn(__fmul_rn(ex2, uniform24(splitmix64(seed, 3 * j + 2))), lo2);
-        cand[3 * i] = x;
-        cand[3 * i + 1] = y;
-        cand[3 * i + 2] = z;
-        flags[i] = consistent(x, y, z, views, nv, masks, z_near) ? 1u : 0u;
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+        p[a] = __fadd_rn(__fmul_rn(b.ex[a], uniform24(splitmix64(b.seed, 3 * j + a))), b.lo[a]);
+}
+
+// Acceptance of HULL_BLOCK candidates per block, as a bit each (candidate i
+// of the batch in bit i & 31 of word i / 32) and a count per block.
+// A warp of candidates runs until its last one fails, so testing every view
+// at once keeps a warp for all views while a few lanes live (196 us for 4 M
+// candidates and 16 views).  The views are taken in groups of 1, 1, 2, 4, ...
+// instead, the survivors of each group packed into a shared queue, so that
+// the next group runs with full warps; a survivor's position is drawn again
+// (kept in shared memory it cost occupancy: 95 -> 127 us for 6.4 M
+// candidates).  Bound by issue (three draws a candidate, two exact divisions
+// a test) and by the latency of the mask reads.
+constexpr int HULL_THREADS = 256;
+
+__global__ void __launch_bounds__(HULL_THREADS)
+hull_accept_kernel(HullBox box, uint64_t first, int64_t count, const HullView *__restrict__ views,
+                   int nv, const uint8_t *__restrict__ masks, float z_near,
+                   uint32_t *__restrict__ bits, uint32_t *__restrict__ counts)
+{
+    __shared__ uint16_t s_q[2][HULL_BLOCK];
+    __shared__ uint32_t s_bits[HULL_BLOCK / 32];
+    __shared__ uint32_t s_n[2];
+    const int64_t base = (int64_t)blockIdx.x * HULL_BLOCK;
+    const int lane = threadIdx.x & 31;
+    for (int j = threadIdx.x; j < HULL_BLOCK / 32; j += HULL_THREADS) s_bits[j] = 0;
+    if (threadIdx.x < 2) s_n[threadIdx.x] = 0;
+    __syncthreads();
+    int n = (int)(count - base < HULL_BLOCK ? count - base : HULL_BLOCK);
+    int cur = 0;
+    bool all = true; // the first group tests every candidate, without a queue
+    for (int v0 = 0; v0 < nv && n > 0;) {
+        const int v1 = v0 < 2 ? v0 + 1 : (2 * v0 < nv ? 2 * v0 : nv);
+        for (int q0 = 0; q0 < n; q0 += HULL_THREADS) {
+            const int q = q0 + (int)threadIdx.x;
+            bool ok = false;
+            uint32_t i = 0;
+            if (q < n) {
+                i = all ? (uint32_t)q : s_q[cur][q];
+                float p[3];
+                candidate(box, first + (uint64_t)base + i, p);
+                ok = consistent(p[0], p[1], p[2], views, v0, v1, masks, z_near);
+            }
+            const uint32_t m = __ballot_sync(0xffffffffu, ok);
+            uint32_t at = 0;
+            if (lane == 0 && m) at = atomicAdd(&s_n[cur ^ 1], (uint32_t)__popc(m));
+            at = __shfl_sync(0xffffffffu, at, 0);
+            if (ok) s_q[cur ^ 1][at + __popc(m & ((1u << lane) - 1u))] = (uint16_t)i;
+        }
+        __syncthreads();
+        cur ^= 1;
+        n = (int)s_n[cur];
+        if (threadIdx.x == 0) s_n[cur ^ 1] = 0;
+        __syncthreads();
+        all = false;
+        v0 = v1;
     }
+    for (int q = threadIdx.x; q < n; q += HULL_THREADS) {
+        const uint32_t i = all ? (uint32_t)q : s_q[cur][q];
+        atomicOr(&s_bits[i >> 5], 1u << (i & 31));
+    }
+    __syncthreads();
+    for (int j = threadIdx.x; j < HULL_BLOCK / 32; j += HULL_THREADS)
+        bits[(int64_t)blockIdx.x * (HULL_BLOCK / 32) + j] = s_bits[j];
+    if (threadIdx.x == 0) counts[blockIdx.x] = (uint32_t)n;
+}
+
+// One block: exclusive scan of the nb block counts in place, out[0] = total.
+__global__ void __launch_bounds__(1024)
+hull_scan_kernel(uint32_t *counts, int nb, unsigned long long *out)
+{
+    __shared__ uint32_t s_w[32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    uint32_t run = 0;
+    for (int base = 0; base < nb; base += 1024) {
+        const int i = base + (int)threadIdx.x;
+        const uint32_t v = i < nb ? counts[i] : 0u;
+        uint32_t inc = v;
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t t = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += t;
+        }
+        if (lane == 31) s_w[w] = inc;
+        __syncthreads();
+        if (w == 0) {
+            uint32_t x = s_w[lane];
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t t = __shfl_up_sync(0xffffffffu, x, o);
+                if (lane >= o) x += t;
+            }
+            s_w[lane] = x;
+        }
+        __syncthreads();
+        if (i < nb) counts[i] = run + inc - v + (w > 0 ? s_w[w - 1] : 0u);
+        run += s_w[31];
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) out[0] = run;
 }
 
 // Accepted candidates of rank < need go to out[done + rank]; the candidate
-// of rank need - 1 reports its index.
-__global__ void hull_take_kernel(const float *__restrict__ cand, const uint32_t *__restrict__ flags,
-                                 const uint32_t *__restrict__ rank, int64_t count, uint32_t need,
-                                 float *__restrict__ out, int64_t done,
-                                 unsigned long long *last)
+// of rank need - 1 reports its index.  One thread per word of bits.
+__global__ void __launch_bounds__(HULL_BLOCK / 32)
+hull_take_kernel(HullBox box, uint64_t first, const uint32_t *__restrict__ bits,
+                 const uint32_t *__restrict__ offsets, uint32_t need, float *__restrict__ out,
+                 int64_t done, unsigned long long *last)
 {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        if (!flags[i]) continue;
-        const uint32_t k = rank[i];
-        if (k >= need) continue;
-        const int64_t o = done + k;
-        out[3 * o] = cand[3 * i];
-        out[3 * o + 1] = cand[3 * i + 1];
-        out[3 * o + 2] = cand[3 * i + 2];
-        if (k == need - 1) *last = (unsigned long long)i;
+    constexpr int WORDS = HULL_BLOCK / 32;
+    __shared__ uint32_t s_w[WORDS / 32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t word = (int64_t)blockIdx.x * WORDS + threadIdx.x;
+    uint32_t m = bits[word];
+    const uint32_t c = (uint32_t)__popc(m);
+    uint32_t inc = c;
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t t = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += t;
+    }
+    if (lane == 31) s_w[w] = inc;
+    __syncthreads();
+    uint32_t k = offsets[blockIdx.x] + inc - c;
+    for (int j = 0; j < w; ++j) k += s_w[j];
+    for (; m && k < need; m &= m - 1, ++k) {
+        const uint64_t i = 32ull * (uint64_t)word + (uint64_t)(__ffs(m) - 1);
+        float p[3];
+        candidate(box, first + i, p);
+        float *dst = out + 3 * (done + k);
+        dst[0] = p[0];
+        dst[1] = p[1];
+        dst[2] = p[2];
+        if (k == need - 1) *last = i;
     }
 }
 
-// Standard normals for coefficients [c0, c0 + count) of the flattened
-// [points, coefficients] array, Box-Muller on stream seed: pair p = c / 2
-// uses outputs 2p and 2p + 1.  fp32 (logf, sincospif): no decision depends
-// on these values, and fp64 transcendentals run at a small fraction of the
-// fp32 rate on this GPU.  u1 and u2 are exact in fp32 (24-bit integers times
-// 2^-24).
-__global__ void sh_normals_kernel(uint64_t seed, int64_t c0, int64_t count,
-                                  float *__restrict__ out)
+// Standard normals for the flattened [points, coefficients] array, Box-Muller
+// on stream seed: coefficients 2p and 2p + 1 are the cosine and the sine of
+// pair p, from outputs 2p and 2p + 1; one thread per pair.  fp32 (logf,
+// sincospif): no decision depends on these values, and fp64 transcendentals
+// run at a small fraction of the fp32 rate on this GPU.  u1 and u2 are exact
+// in fp32 (24-bit integers times 2^-24).
+__global__ void sh_normals_kernel(uint64_t seed, int64_t count, float *__restrict__ out)
 {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const uint64_t c = (uint64_t)(c0 + i), p = c >> 1;
-        const float u1 = ((float)(uint32_t)(splitmix64(seed, 2 * p) >> 40) + 1.0f) * 0x1p-24f;
-        const float u2 = (float)(uint32_t)(splitmix64(seed, 2 * p + 1) >> 40) * 0x1p-24f;
+    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; 2 * p < count;
+         p += (int64_t)gridDim.x * blockDim.x) {
+        const float u1 =
+            ((float)(uint32_t)(splitmix64(seed, 2 * (uint64_t)p) >> 40) + 1.0f) * 0x1p-24f;
+        const float u2 = (float)(uint32_t)(splitmix64(seed, 2 * (uint64_t)p + 1) >> 40) * 0x1p-24f;
         const float r = sqrtf(-2.0f * logf(u1));
         float sn, cs;
         sincospif(2.0f * u2, &sn, &cs);
-        out[i] = (c & 1) ? r * sn : r * cs;
+        out[2 * p] = r * cs;
+        if (2 * p + 1 < count) out[2 * p + 1] = r * sn;
     }
 }
 
@@ -146,32 +251,31 @@ void launch_consistency(const float *pos, int64_t n, const HullView *views, int 
     count_launches(1);
 }
 
-void launch_hull_candidates(uint64_t seed, uint64_t first, int64_t count, const float lo[3],
-                            const float ext[3], const HullView *views, int nv,
-                            const uint8_t *masks, float z_near, float *cand, uint32_t *flags,
-                            cudaStream_t s)
-{
-    if (count <= 0) return;
-    hull_candidates_kernel<<<grid_of(count), 256, 0, s>>>(seed, first, count, lo[0], lo[1], lo[2],
-                                                          ext[0], ext[1], ext[2], views, nv,
-                                                          masks, z_near, cand, flags);
-    count_launches(1);
-}
-
-void launch_hull_take(const float *cand, const uint32_t *flags, const uint32_t *rank,
-                      int64_t count, uint32_t need, float *out, int64_t done,
-                      unsigned long long *last, cudaStream_t s)
+void launch_hull_batch(uint64_t seed, uint64_t first, int64_t count, const float lo[3],
+                       const float ext[3], const HullView *views, int nv, const uint8_t *masks,
+                       float z_near, uint32_t *bits, uint32_t *counts, uint32_t need, float *out,
+                       int64_t done, unsigned long long *result, cudaStream_t s)
 {
     if (count <= 0 || need == 0) return;
-    hull_take_kernel<<<grid_of(count), 256, 0, s>>>(cand, flags, rank, count, need, out, done,
-                                                     last);
-    count_launches(1);
+    HullBox box;
+    box.seed = seed;
+    for (int a = 0; a < 3; ++a) {
+        box.lo[a] = lo[a];
+        box.ex[a] = ext[a];
+    }
+    const unsigned nb = (unsigned)((count + HULL_BLOCK - 1) / HULL_BLOCK);
+    hull_accept_kernel<<<nb, HULL_THREADS, 0, s>>>(box, first, count, views, nv, masks, z_near,
+                                                   bits, counts);
+    hull_scan_kernel<<<1, 1024, 0, s>>>(counts, (int)nb, result);
+    hull_take_kernel<<<nb, HULL_BLOCK / 32, 0, s>>>(box, first, bits, counts, need, out, done,
+                                                    result + 1);
+    count_launches(3);
 }
 
-void launch_sh_normals(uint64_t seed, int64_t c0, int64_t count, float *out, cudaStream_t s)
+void launch_sh_normals(uint64_t seed, int64_t count, float *out, cudaStream_t s)
 {
     if (count <= 0) return;
-    sh_normals_kernel<<<grid_of(count), 256, 0, s>>>(seed, c0, count, out);
+    sh_normals_kernel<<<grid_of((count + 1) / 2), 256, 0, s>>>(seed, count, out);
     count_launches(1);
 }
 

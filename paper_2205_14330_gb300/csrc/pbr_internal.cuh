@@ -334,19 +334,18 @@ struct HullView {
 void launch_consistency(const float *pos, int64_t n, const HullView *views, int nv,
                         const uint8_t *masks, float z_near, uint8_t *flags8, uint32_t *flags32,
                         cudaStream_t s);
-// Candidates first .. first + count - 1 of stream `seed` in the box lo +
-// [0, ext): positions and flags.
-void launch_hull_candidates(uint64_t seed, uint64_t first, int64_t count, const float lo[3],
-                            const float ext[3], const HullView *views, int nv,
-                            const uint8_t *masks, float z_near, float *cand, uint32_t *flags,
-                            cudaStream_t s);
-// Accepted candidates of rank (exclusive scan of flags) below `need` to
-// out[done + rank]; *last = index of the candidate of rank need - 1.
-void launch_hull_take(const float *cand, const uint32_t *flags, const uint32_t *rank,
-                      int64_t count, uint32_t need, float *out, int64_t done,
-                      unsigned long long *last, cudaStream_t s);
-// out[i] = standard normal number c0 + i of stream `seed` (Box-Muller).
-void launch_sh_normals(uint64_t seed, int64_t c0, int64_t count, float *out, cudaStream_t s);
+// Candidates first .. first + count - 1 of stream `seed` in the box lo + [0,
+// ext): the first `need` accepted ones go to out[done ..].  result[0] (device)
+// receives the number accepted, result[1] the batch index of the need-th one
+// when there is one.  Scratch: a bit per candidate (count rounded up to
+// HULL_BLOCK) and a count per HULL_BLOCK candidates.
+constexpr int HULL_BLOCK = 4096;
+void launch_hull_batch(uint64_t seed, uint64_t first, int64_t count, const float lo[3],
+                       const float ext[3], const HullView *views, int nv, const uint8_t *masks,
+                       float z_near, uint32_t *bits, uint32_t *counts, uint32_t need, float *out,
+                       int64_t done, unsigned long long *result, cudaStream_t s);
+// out[i] = standard normal number i of stream `seed` (Box-Muller).
+void launch_sh_normals(uint64_t seed, int64_t count, float *out, cudaStream_t s);
 
 // ---- raster (k_raster.cu)
 // Store mode (bwd_mode 2): T[k * n_pix + pix] = the transmittance pixel pix
