@@ -444,10 +444,10 @@ int pbr::forward_eager(pbr_ctx *c, pbr_state *st, float *out_rgb, cudaStream_t s
         StageScope t(c, STG_DEPTH_SORT, s);
         if (direct)
             radix_sort_pairs(zbits, vv, vk2, vv2, nullptr, npv, depth_bits, temp, s, zlo, marker,
-                             true);
+                             true, 0, status);
         else
             radix_sort_pairs(vk, vv, vk2, vv2, n_vis_dev, (int64_t)n_vis, depth_bits, temp, s,
-                             zlo);
+                             zlo, 0xffffffffu, false, 0, status);
     }
     // 3. duplicate per covered tile, in depth order
     uint32_t *tk = st->tile_keys, *tv = st->tile_vals;
@@ -461,7 +461,7 @@ int pbr::forward_eager(pbr_ctx *c, pbr_state *st, float *out_rgb, cudaStream_t s
         StageScope t(c, STG_TILE_SORT, s);
         radix_sort_pairs(tk, tv, pk2, pv2, n_pairs_dev, (int64_t)n_pairs,
                          key_bits_for(L.n_tiles), temp, s, 0, 0xffffffffu, false,
-                         block_bits(o.tile_w, o.tile_h));
+                         block_bits(o.tile_w, o.tile_h), status);
     }
     if (tk != st->tile_keys) { // result landed in the alternate buffers: swap ownership
         for (void *&p : tmp.ptrs) {

@@ -18,6 +18,7 @@
 // last call's contents: counters and tile ranges are cleared on every call,
 // and calls whose GPU work overlaps (different streams, or other host
 // threads) race on it.
+#include <algorithm>
 #include <mutex>
 
 #include "api_internal.h"
@@ -134,14 +135,18 @@ extern "C" int pbr_render_forward_noalloc(const pbr_points *scenes, int32_t n_sc
 
     // phase 2: the list buffers, sized by the counts
     const int64_t cap_sort = n_vis > n_pairs ? (int64_t)n_vis : (int64_t)n_pairs;
-    size_t temp_bytes = scan_temp_bytes(npv);
-    if (radix_temp_bytes(cap_sort) > temp_bytes) temp_bytes = radix_temp_bytes(cap_sort);
-    if (emit_temp_bytes((int64_t)n_vis) > temp_bytes) temp_bytes = emit_temp_bytes((int64_t)n_vis);
+    const size_t other_temp = std::max(scan_temp_bytes(npv), emit_temp_bytes((int64_t)n_vis));
+    const size_t radix_temp = std::max(radix_temp_bytes(cap_sort),
+                                       std::max(radix_temp_bytes((int64_t)n_vis),
+                                                radix_temp_bytes((int64_t)n_pairs)));
     uint32_t *vk = cv.take<uint32_t>(4 * n_vis), *vv = cv.take<uint32_t>(4 * n_vis);
     uint32_t *vk2 = cv.take<uint32_t>(4 * n_vis), *vv2 = cv.take<uint32_t>(4 * n_vis);
     uint32_t *tk = cv.take<uint32_t>(4 * n_pairs), *tv = cv.take<uint32_t>(4 * n_pairs);
     uint32_t *pk2 = cv.take<uint32_t>(4 * n_pairs), *pv2 = cv.take<uint32_t>(4 * n_pairs);
-    void *temp = cv.take<void>(temp_bytes);
+    // the faster sort where its scratch fits behind the lists, else the one
+    // that needs least
+    const bool least = ((cv.need + 255) & ~(size_t)255) + std::max(other_temp, radix_temp) > cv.cap;
+    void *temp = cv.take<void>(std::max(other_temp, least ? radix_temp_bytes_least(cap_sort) : radix_temp));
     if (!cv.fits() || n_pairs >= UINT32_MAX)
         return set_error(PBR_ERR_CAPACITY,
                          "pbr_render_forward_noalloc: %llu (tile, point-view) pairs need %zu bytes "
@@ -151,14 +156,15 @@ extern "C" int pbr_render_forward_noalloc(const pbr_points *scenes, int32_t n_sc
     const uint32_t *n_vis_dev = (const uint32_t *)(counters + 1);
     const uint32_t *n_pairs_dev = (const uint32_t *)(counters + 0);
     launch_compact_visible(ntiles, zbits, npv, vk, vv, nullptr, temp, s);
-    radix_sort_pairs(vk, vv, vk2, vv2, n_vis_dev, (int64_t)n_vis, 32, temp, s);
+    radix_sort_pairs(vk, vv, vk2, vv2, n_vis_dev, (int64_t)n_vis, 32, temp, s, 0, 0xffffffffu,
+                     false, 0, status, least);
     launch_emit_pairs(b, o, vv, n_vis_dev, (int64_t)n_vis, ntiles, nt8, rect, tk, tv,
                       (int64_t)n_pairs, status, temp, s);
     int key_bits = 1;
     while (key_bits < 32 && ((L.n_tiles - 1) >> key_bits)) ++key_bits;
     const int sb = block_bits(o.tile_w, o.tile_h);
     radix_sort_pairs(tk, tv, pk2, pv2, n_pairs_dev, (int64_t)n_pairs, key_bits, temp, s, 0,
-                     0xffffffffu, false, sb);
+                     0xffffffffu, false, sb, status, least);
     PBR_CUDA(cudaMemsetAsync(ranges, 0, sizeof(uint2) * L.n_tiles, s));
     launch_tile_ranges(tk, n_pairs_dev, (int64_t)n_pairs, ranges, L.n_tiles, sb, s);
     launch_raster_fwd(b, o, opts->batch_depth, ranges, tk, tv, rec, out_rgb, T_final, n_contrib,

@@ -17,10 +17,14 @@
 //                         (tile, depth, pv) -- the order Eqs. 6-7 need
 //   5. tile_ranges      : [start, end) of every tile in the sorted list
 //
-// Scans are reduce-then-scan (three kernels, no inter-block waiting).  The
+// Scans are reduce-then-scan (three kernels, no inter-block waiting).  A
 // radix pass ranks keys stably inside a block with per-warp peer masks
 // (shared-memory OR) and shared atomics, and reorders them in shared memory
-// so that the scatter writes contiguous runs.
+// so that the scatter writes contiguous runs.  Short sorts run in one sweep
+// (one histogram of every digit, then a kernel per pass with look-back), long
+// ones with a histogram, a scan and a scatter per pass.
+#include <algorithm>
+
 #include "pbr_internal.cuh"
 
 namespace pbr {
@@ -429,6 +433,304 @@ radix_scatter_kernel(const uint32_t *__restrict__ keys_in, const uint32_t *__res
     }
 }
 
+// ------------------------------------------------- one-sweep radix sort
+// All digit histograms of a sort come from one read of its keys; a pass is
+// then one kernel: every block ranks its tile of keys, publishes the tile's
+// digit counts and adds up those of the tiles before it (decoupled
+// look-back) while its keys are being placed in shared memory.
+// A state word holds a digit count of one tile or its sum over all tiles up to
+// it (28 bits) under a tag: 2 pass + 1 or 2 pass + 2; words of an earlier
+// pass carry smaller tags, so one clear serves all passes.  Tiles are taken
+// from a counter, so every tile before a block's own is running or done and
+// each wait ends; the waits are bounded all the same (SWEEP_SPINS polls, then
+// ST_SORT_STALL in *status and whatever order results).
+constexpr int SWEEP_PASSES = 4;
+constexpr uint32_t SWEEP_COUNT = 0x0fffffffu; // counts a state word can hold
+constexpr int SWEEP_SPINS = 1 << 22;
+constexpr int64_t SWEEP_HIST_BLOCKS = 152 * 8;
+// Sorts of up to SWEEP_MOST entries run in one sweep, those below SWEEP_SMALL
+// with small tiles.  Depth and tile sort of one batch together (keys of 24 and
+// 11-16 bits, us; three-kernel passes / large tiles / small tiles): 4k point-
+// views 95 / 57 / 46, 60k 112 / 65 / 57, 130k 115 / 69 / 64, 260k 117 / 73 /
+// 74, 1M 137 / 106 / 138, 4M 268 / 264 / 405, 8M 437 / 471 / 761, 32M 1620 /
+// 1820 / -.  Small sorts gain by the launches (two and one a pass against
+// five a pass); large ones lose more to the look-back's reads of the tiles'
+// counts, 2 KB a tile and step, than the second read of the keys costs.
+constexpr int64_t SWEEP_SMALL = 1 << 17, SWEEP_MOST = 1 << 22;
+// words before the tiles' states: digit offsets, tile counters, done counter
+constexpr int SWEEP_HEAD = SWEEP_PASSES * RBINS + 16;
+
+struct SweepDigits {
+    uint32_t key_lo, key_max;
+    int shift[SWEEP_PASSES], width[SWEEP_PASSES], passes;
+};
+
+// Digit counts of all passes; the last block to finish turns them into the
+// digits' first output positions.  Four keys a thread and step.
+__global__ void __launch_bounds__(SORT_THREADS)
+sweep_hist_kernel(const uint32_t *__restrict__ keys, const uint32_t *n_dev, int64_t cap,
+                  SweepDigits dg, uint32_t *head)
+{
+    __shared__ uint32_t s_h[SWEEP_PASSES][RBINS];
+    __shared__ uint32_t s_w[SORT_WARPS];
+    __shared__ bool s_last;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    for (int j = threadIdx.x; j < SWEEP_PASSES * RBINS; j += SORT_THREADS) (&s_h[0][0])[j] = 0;
+    __syncthreads();
+    const int64_t n = dev_count(n_dev, cap);
+    const int64_t n4 = n >> 2, step = (int64_t)gridDim.x * SORT_THREADS;
+    auto count = [&](uint32_t key) {
+        uint32_t k = key - dg.key_lo;
+        k = k < dg.key_max ? k : dg.key_max;
+#pragma unroll
+        for (int p = 0; p < SWEEP_PASSES; ++p)
+            if (p < dg.passes)
+                atomicAdd(&s_h[p][(k >> dg.shift[p]) & ((1u << dg.width[p]) - 1u)], 1u);
+    };
+    const int64_t t0 = (int64_t)blockIdx.x * SORT_THREADS + threadIdx.x;
+    for (int64_t i = t0; i < n4; i += step) {
+        const uint4 q = reinterpret_cast<const uint4 *>(keys)[i];
+        count(q.x);
+        count(q.y);
+        count(q.z);
+        count(q.w);
+    }
+    if (t0 < (n & 3)) count(keys[4 * n4 + t0]);
+    __syncthreads();
+    for (int j = threadIdx.x; j < dg.passes * RBINS; j += SORT_THREADS) {
+        const uint32_t c = (&s_h[0][0])[j];
+        if (c) atomicAdd(head + j, c);
+    }
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0)
+        s_last = atomicAdd(head + SWEEP_PASSES * RBINS + SWEEP_PASSES, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    constexpr int PER = RBINS / SORT_THREADS;
+    for (int p = 0; p < dg.passes; ++p) {
+        uint32_t v[PER], sum = 0;
+#pragma unroll
+        for (int k = 0; k < PER; ++k) {
+            v[k] = __ldcg(head + p * RBINS + threadIdx.x * PER + k);
+            sum += v[k];
+        }
+        const uint32_t inc = warp_incl_scan(sum);
+        if (lane == 31) s_w[w] = inc;
+        __syncthreads();
+        uint32_t at = inc - sum;
+        for (int j = 0; j < w; ++j) at += s_w[j];
+#pragma unroll
+        for (int k = 0; k < PER; ++k) {
+            head[p * RBINS + threadIdx.x * PER + k] = at;
+            at += v[k];
+        }
+        __syncthreads();
+    }
+}
+
+__device__ __forceinline__ uint32_t ld_state(const uint32_t *p)
+{
+    uint32_t v;
+    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+
+__device__ __forceinline__ void st_state(uint32_t *p, uint32_t v)
+{
+    asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+
+// Sum of the digit's counts over the tiles before `tile` (state: the digit's
+// column, one word per tile at a stride of RBINS).
+__device__ uint32_t look_back(const uint32_t *state, uint32_t tile, uint32_t agg_tag,
+                              uint32_t *status)
+{
+    uint32_t sum = 0;
+    int spins = 0;
+    for (int64_t t = (int64_t)tile - 1; t >= 0;) {
+        // four predecessors at a time
+        uint32_t v[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) v[k] = t - k >= 0 ? ld_state(state + (t - k) * RBINS) : 0u;
+        int used = 0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            if (used != k || t - k < 0) continue; // an earlier one was not ready
+            const uint32_t tag = v[k] >> 28;
+            if (tag < agg_tag) continue; // not ready yet
+            sum += v[k] & SWEEP_COUNT;
+            if (tag > agg_tag) return sum; // sum over every tile up to that one
+            ++used;
+        }
+        t -= used;
+        if (used == 0 && ++spins > SWEEP_SPINS) {
+            if (status) atomicOr(status, ST_SORT_STALL);
+            return sum;
+        }
+    }
+    return sum;
+}
+
+template <int ITEMS>
+__host__ __device__ constexpr size_t sweep_smem()
+{
+    constexpr int TILE = SORT_THREADS * ITEMS;
+    constexpr int PM = SORT_WARPS * RBINS; // peer masks share the ranked keys' space
+    return sizeof(uint32_t) * ((TILE > PM ? TILE : PM) + 2 * TILE + SORT_WARPS * RBINS +
+                               3 * RBINS + SORT_WARPS + 1);
+}
+
+template <int ITEMS>
+__global__ void __launch_bounds__(SORT_THREADS)
+sweep_pass_kernel(const uint32_t *__restrict__ keys_in, const uint32_t *__restrict__ vals_in,
+                  uint32_t *__restrict__ keys_out, uint32_t *__restrict__ vals_out,
+                  const uint32_t *n_dev, int64_t cap, uint32_t key_lo, uint32_t key_max, int shift,
+                  int width, int pass, uint32_t *head, bool index_vals, uint32_t *status)
+{
+    constexpr int TILE = SORT_THREADS * ITEMS;
+    constexpr int PM = SORT_WARPS * RBINS;
+    extern __shared__ uint32_t s_mem[];
+    uint32_t *s_k = s_mem;                        // [TILE] keys, ranked order (peer masks first)
+    uint32_t *s_v = s_k + (TILE > PM ? TILE : PM); // [TILE] values, ranked order
+    uint32_t *s_vin = s_v + TILE;                 // [TILE] values, input order
+    uint32_t(*s_wh)[RBINS] = (uint32_t(*)[RBINS])(s_vin + TILE); // [warps][RBINS]
+    uint32_t *s_tot = s_vin + TILE + SORT_WARPS * RBINS;
+    uint32_t *s_dbase = s_tot + RBINS;
+    uint32_t *s_gbase = s_dbase + RBINS;
+    uint32_t *s_scan = s_gbase + RBINS;
+    uint32_t *s_tile = s_scan + SORT_WARPS;
+    const int64_t n = dev_count(n_dev, cap);
+    if (threadIdx.x == 0) s_tile[0] = atomicAdd(head + SWEEP_PASSES * RBINS + pass, 1u);
+    for (int j = threadIdx.x; j < SORT_WARPS * RBINS; j += SORT_THREADS) {
+        (&s_wh[0][0])[j] = 0;
+        s_k[j] = 0;
+    }
+    __syncthreads();
+    const uint32_t tile = s_tile[0];
+    const int64_t blk = (int64_t)tile * TILE;
+    if (blk >= n) return;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const uint32_t mask = (1u << width) - 1u;
+    const int bins = 1 << width;
+    uint32_t *s_pm = s_k + w * RBINS; // this warp's peer masks
+    const int64_t base = blk + (int64_t)w * 32 * ITEMS;
+    uint32_t key[ITEMS], rank[ITEMS];
+    const int lbase = w * 32 * ITEMS + lane; // local index of round 0
+#pragma unroll
+    for (int r = 0; r < ITEMS; ++r) {
+        const int64_t i = base + r * 32 + lane;
+        const bool ok = i < n;
+        key[r] = ok ? keys_in[i] : 0u;
+        s_vin[lbase + r * 32] = ok ? (index_vals ? (uint32_t)i : vals_in[i]) : 0u;
+    }
+    const uint32_t lt = lanemask_lt();
+    const bool full = blk + TILE <= n; // every key of the tile is in range
+    // stable rank inside the warp, as in radix_scatter_kernel
+#pragma unroll
+    for (int r = 0; r < ITEMS; ++r) {
+        const bool ok = base + r * 32 + lane < n;
+        const uint32_t d = ok ? digit_of(key[r], key_lo, key_max, shift, mask) : (uint32_t)RBINS;
+        uint32_t peers;
+        if (full || __all_sync(0xffffffffu, ok)) {
+            atomicOr(&s_pm[d], 1u << lane);
+            __syncwarp();
+            peers = s_pm[d];
+            __syncwarp();
+        } else {
+            peers = peers_by_ballot(d, false);
+        }
+        uint32_t old = 0;
+        if (d < RBINS && (peers & lt) == 0) {
+            old = atomicAdd(&s_wh[w][d], (uint32_t)__popc(peers));
+            s_pm[d] = 0;
+        }
+        __syncwarp(); // peer words clear before the next round's ORs
+        rank[r] = (uint32_t)(__ffs(peers) - 1) | ((uint32_t)__popc(peers & lt) << 5) | (old << 10);
+    }
+#pragma unroll
+    for (int r = 0; r < ITEMS; ++r) {
+        const uint32_t packed = rank[r];
+        const uint32_t base_r = __shfl_sync(0xffffffffu, packed >> 10, packed & 31);
+        rank[r] = base_r + ((packed >> 5) & 31);
+    }
+    __syncthreads();
+    // per digit: exclusive prefix over warps, and the tile's count, published
+    constexpr int PER = RBINS / SORT_THREADS;
+    uint32_t *states = head + SWEEP_HEAD;
+    const uint32_t agg = 2u * (uint32_t)pass + 1u;
+    uint32_t mine[PER];
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+        const int dd = threadIdx.x + k * SORT_THREADS;
+        uint32_t t = 0;
+        if (dd < bins) {
+#pragma unroll
+            for (int j = 0; j < SORT_WARPS; ++j) {
+                const uint32_t x = s_wh[j][dd];
+                s_wh[j][dd] = t;
+                t += x;
+            }
+            st_state(states + (size_t)tile * RBINS + dd, t | ((tile == 0 ? agg + 1u : agg) << 28));
+        }
+        s_tot[dd] = t;
+        mine[k] = t;
+    }
+    __syncthreads();
+    // block exclusive scan of the digit totals
+    {
+        uint32_t loc[PER], sum = 0;
+#pragma unroll
+        for (int q = 0; q < PER; ++q) {
+            loc[q] = s_tot[threadIdx.x * PER + q];
+            sum += loc[q];
+        }
+        const uint32_t inc = warp_incl_scan(sum);
+        if (lane == 31) s_scan[w] = inc;
+        __syncthreads();
+        uint32_t off = inc - sum;
+        for (int j = 0; j < w; ++j) off += s_scan[j];
+#pragma unroll
+        for (int q = 0; q < PER; ++q) {
+            s_dbase[threadIdx.x * PER + q] = off;
+            off += loc[q];
+        }
+    }
+    __syncthreads();
+    // place the tile in digit order, then add up the tiles before it
+#pragma unroll
+    for (int r = 0; r < ITEMS; ++r) {
+        if (base + r * 32 + lane < n) {
+            const uint32_t d = digit_of(key[r], key_lo, key_max, shift, mask);
+            const uint32_t l = s_dbase[d] + s_wh[w][d] + rank[r];
+            s_k[l] = key[r];
+            s_v[l] = s_vin[lbase + r * 32];
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+        const int dd = threadIdx.x + k * SORT_THREADS;
+        if (dd < bins) {
+            uint32_t before = 0;
+            if (tile > 0) {
+                before = look_back(states + dd, tile, agg, status);
+                st_state(states + (size_t)tile * RBINS + dd, (before + mine[k]) | ((agg + 1u) << 28));
+            }
+            // output position of ranked slot j of digit d: s_gbase[d] + j
+            s_gbase[dd] = head[pass * RBINS + dd] + before - s_dbase[dd];
+        }
+    }
+    __syncthreads();
+    const int cnt = (int)(n - blk < TILE ? n - blk : TILE);
+    for (int j = threadIdx.x; j < cnt; j += SORT_THREADS) {
+        const uint32_t k = s_k[j];
+        const uint32_t g = s_gbase[digit_of(k, key_lo, key_max, shift, mask)] + (uint32_t)j;
+        keys_out[g] = k;
+        vals_out[g] = s_v[j];
+    }
+}
+
 // ------------------------------------------------------------ emission
 // Tile counts in depth order (the scan that places each point-view's run of
 // pairs reads them).
@@ -668,12 +970,56 @@ void launch_exclusive_scan(const uint32_t *in, uint32_t *out, int64_t n,
     run_scan(LoadU32{in}, ActStore{out}, nullptr, n, temp, total, nullptr, s);
 }
 
-size_t radix_temp_bytes(int64_t cap)
+namespace {
+
+// Items a thread of a one-sweep pass: large tiles, unless they leave most of
+// the SMs idle.
+int sweep_items(int64_t cap) { return cap >= SWEEP_SMALL ? 16 : 4; }
+
+size_t sweep_temp_bytes(int64_t cap)
+{
+    const int64_t tile = SORT_THREADS * sweep_items(cap);
+    return sizeof(uint32_t) * (size_t)(SWEEP_HEAD + (cap + tile - 1) / tile * RBINS);
+}
+
+bool one_sweep(int64_t cap) { return cap <= SWEEP_MOST; }
+static_assert(SWEEP_MOST <= (int64_t)SWEEP_COUNT, "a state word holds the counts");
+
+template <int ITEMS>
+void sweep_pass(const uint32_t *keys, const uint32_t *vals, uint32_t *keys_alt, uint32_t *vals_alt,
+                const uint32_t *n_dev, int64_t cap, const SweepDigits &dg, int pass, uint32_t *head,
+                bool index_vals, uint32_t *status, cudaStream_t s)
+{
+    static const bool attr = cudaFuncSetAttribute(sweep_pass_kernel<ITEMS>,
+                                                  cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                  (int)sweep_smem<ITEMS>()) == cudaSuccess;
+    (void)attr;
+    const int64_t tile = SORT_THREADS * ITEMS;
+    sweep_pass_kernel<ITEMS><<<(unsigned)((cap + tile - 1) / tile), SORT_THREADS,
+                               sweep_smem<ITEMS>(), s>>>(
+        keys, vals, keys_alt, vals_alt, n_dev, cap, dg.key_lo, dg.key_max, dg.shift[pass],
+        dg.width[pass], pass, head, index_vals, status);
+}
+
+size_t three_kernel_temp_bytes(int64_t cap)
 {
     const int64_t nb = (cap + SORT_TILE - 1) / SORT_TILE;
     const int64_t hist = (nb > 0 ? nb : 1) * RBINS;
     return (size_t)hist * sizeof(uint32_t) + scan_temp_bytes(hist);
 }
+
+} // namespace
+
+// Enough for every list of up to cap entries (small tiles need more words a
+// key than large ones).
+size_t radix_temp_bytes(int64_t cap)
+{
+    size_t b = sweep_temp_bytes(std::min(cap, SWEEP_MOST));
+    if (cap >= SWEEP_SMALL) b = std::max(b, sweep_temp_bytes(SWEEP_SMALL - 1));
+    return one_sweep(cap) ? b : std::max(b, three_kernel_temp_bytes(cap));
+}
+
+size_t radix_temp_bytes_least(int64_t cap) { return three_kernel_temp_bytes(cap); }
 
 int radix_passes(int key_bits)
 {
@@ -683,12 +1029,44 @@ int radix_passes(int key_bits)
 void radix_sort_pairs(uint32_t *&keys, uint32_t *&vals, uint32_t *&keys_alt, uint32_t *&vals_alt,
                       const uint32_t *n_dev, int64_t cap, int key_bits, void *temp,
                       cudaStream_t s, uint32_t key_lo, uint32_t key_max, bool index_vals,
-                      int bit_lo)
+                      int bit_lo, uint32_t *status, bool least_temp)
 {
     if (cap <= 0) return;
     if (key_bits <= 0) {
         if (!index_vals) return; // all keys equal: already in stable order
         key_bits = 1;            // one pass still writes the index values
+    }
+    const int passes = radix_passes(key_bits);
+    const int width = (key_bits + passes - 1) / passes;
+    auto swap = [&] {
+        uint32_t *tk = keys, *tv = vals;
+        keys = keys_alt;
+        vals = vals_alt;
+        keys_alt = tk;
+        vals_alt = tv;
+    };
+    if (one_sweep(cap) && !least_temp) {
+        SweepDigits dg;
+        dg.key_lo = key_lo;
+        dg.key_max = key_max;
+        dg.passes = passes;
+        for (int p = 0; p < SWEEP_PASSES; ++p) {
+            dg.shift[p] = p < passes ? bit_lo + p * width : 0;
+            dg.width[p] = p < passes ? (key_bits - p * width < width ? key_bits - p * width : width) : 1;
+        }
+        uint32_t *head = (uint32_t *)temp;
+        cudaMemsetAsync(head, 0, sweep_temp_bytes(cap), s);
+        int64_t hb = (cap + 4 * SORT_THREADS - 1) / (4 * SORT_THREADS);
+        if (hb > SWEEP_HIST_BLOCKS) hb = SWEEP_HIST_BLOCKS;
+        sweep_hist_kernel<<<(unsigned)hb, SORT_THREADS, 0, s>>>(keys, n_dev, cap, dg, head);
+        for (int p = 0; p < passes; ++p) {
+            auto f = sweep_items(cap) == 16 ? sweep_pass<16> : sweep_pass<4>;
+            f(keys, vals, keys_alt, vals_alt, n_dev, cap, dg, p, head, index_vals && p == 0, status,
+              s);
+            swap();
+        }
+        count_launches(1 + passes);
+        return;
     }
     static const bool attr = cudaFuncSetAttribute(radix_scatter_kernel,
                                                   cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -697,8 +1075,6 @@ void radix_sort_pairs(uint32_t *&keys, uint32_t *&vals, uint32_t *&keys_alt, uin
     const int64_t nb = (cap + SORT_TILE - 1) / SORT_TILE;
     uint32_t *hist = (uint32_t *)temp;
     void *scan_tmp = hist + nb * RBINS;
-    const int passes = radix_passes(key_bits);
-    const int width = (key_bits + passes - 1) / passes;
     for (int shift = bit_lo; shift < bit_lo + key_bits; shift += width) {
         const int wd = bit_lo + key_bits - shift < width ? bit_lo + key_bits - shift : width;
         radix_hist_kernel<<<(unsigned)((nb + HIST_TILES - 1) / HIST_TILES), SORT_THREADS, 0, s>>>(
@@ -708,11 +1084,7 @@ void radix_sort_pairs(uint32_t *&keys, uint32_t *&vals, uint32_t *&keys_alt, uin
             keys, vals, keys_alt, vals_alt, n_dev, cap, key_lo, key_max, shift, wd, hist, nb,
             index_vals && shift == bit_lo);
         count_launches(2);
-        uint32_t *tk = keys, *tv = vals;
-        keys = keys_alt;
-        vals = vals_alt;
-        keys_alt = tk;
-        vals_alt = tv;
+        swap();
     }
 }
 
