@@ -3,6 +3,7 @@
 // backward passes of the point-splat renderer (Sec. 3.1-3.3).
 #include <algorithm>
 #include <atomic>
+#include <cmath>
 #include <cstdio>
 #include <cstring>
 #include <mutex>
@@ -301,6 +302,58 @@ int pbr::build_layout(const pbr_points *scenes, int32_t n_scenes, const int32_t 
     return PBR_OK;
 }
 
+// A warp on half a block has half the pixels to serve per step, so the
+// longest list is walked sooner and twice as many warps share the chip; but a
+// point reaching both halves is stepped through twice.  Half blocks pay while
+// the longest block's walk is a large share of the whole: with v the hits a
+// view's block visits (its list, or what saturates it: some 28 layers of
+// splats covering c of its 64 pixels), the batch is worth sum(v) / max(v)
+// equal blocks, and the line lies at 130000 / r of them forward and 45000 / r
+// backward, r the mean cutoff radius in pixels.  r comes from the pair count:
+// a point lists (1 + 2 r / tile_w)(1 + 2 r / tile_h) tiles, r = k f with f the
+// view's focal length in pixels, summed over the views and solved for k.
+// Measured, one pixel a lane / two (us; 16 x 16 tiles, streamed): 120k points,
+// 2 views of 500 x 400 (6.3k blocks, r 2.3): forward 47 / 52, backward 97 /
+// 107; 120k, 4 views of 800^2 (40k, 3.7): 91 / 89, 232 / 183; 45k large
+// points, 1024 x 768 (12.3k, 16): 34 / 33, 93 / 68; 125k, five views of
+// 104 x 141 to 647 x 549 (worth 2k): 217 / 311, 298 / 450; 808k, eight views
+// of 235 x 230 to 1737 x 835, persistent (worth 10k, 6.3): 398 / 534, 1038 /
+// 802.
+RasterLanes pbr::raster_lanes(const HostLayout &L, const DevOpts &o, int64_t n_vis,
+                              int64_t n_pairs)
+{
+    RasterLanes r;
+    if (L.n_pv <= 0 || n_vis <= 0) return r;
+    auto focal = [&](const DevView &V) {
+        return o.radius_mode == 0 ? std::fabs((double)V.fx) : 0.5 * std::min(V.W, V.H);
+    };
+    const double share = (double)n_vis / (double)L.n_pv, tw = o.tile_w, th = o.tile_h;
+    double a = 0.0, b = 0.0, c = -(double)n_pairs; // a k^2 + b k + c = 0
+    for (const DevView &V : L.views) {
+        const double n = share * (double)L.scenes[V.scene].n, f = focal(V);
+        a += n * f * f * 4.0 / (tw * th);
+        b += n * f * 2.0 * (1.0 / tw + 1.0 / th);
+        c += n;
+    }
+    const double k = c < 0.0 && a > 0.0 ? (-b + std::sqrt(b * b - 4.0 * a * c)) / (2.0 * a) : 0.0;
+    double most = 0.0, sum = 0.0, sum_r = 0.0;
+    for (const DevView &V : L.views) {
+        const double blocks = (double)((V.W + 7) / 8) * ((V.H + 7) / 8);
+        const double rc = std::max(k * focal(V), 0.5), w = 8.0 + 2.0 * rc;
+        const double cover = 64.0 * 3.14159265 * rc * rc / (w * w); // pixels of a block per hit
+        const double v = std::min(share * (double)L.scenes[V.scene].n * (w * w / 64.0) / blocks,
+                                  28.0 * 64.0 / cover);
+        most = std::max(most, v);
+        sum += blocks * v;
+        sum_r += blocks * v * rc;
+    }
+    if (!(most > 0.0)) return r;
+    const double worth = sum / most, mean_r = sum_r / sum;
+    r.fwd_two = worth * mean_r >= 130000.0;
+    r.bwd_two = worth * mean_r >= 45000.0;
+    return r;
+}
+
 // ------------------------------------------------------------ allocation
 int pbr::dalloc(void **p, size_t bytes, cudaStream_t s)
 {
@@ -495,7 +548,8 @@ int pbr::forward_eager(pbr_ctx *c, pbr_state *st, float *out_rgb, cudaStream_t s
         launch_raster_fwd(b, o, st->batch_depth, st->ranges, st->tile_keys, st->tile_vals,
                           st->rec, out_rgb,
                           st->T_final, st->n_contrib,
-                          st->opts.no_pair_stats ? nullptr : st->counters + 2, s, st->tile_order,
+                          st->opts.no_pair_stats ? nullptr : st->counters + 2, s,
+                          raster_lanes(L, o, st->n_vis, st->n_pairs).fwd_two, st->tile_order,
                           st->work, st->store());
     }
     PBR_CUDA(cudaGetLastError());
@@ -643,6 +697,7 @@ extern "C" int pbr_render_backward(pbr_ctx *c, pbr_state *st, const float *grad_
                           st->tile_vals, st->rec,
                           st->T_final, st->n_contrib, grad_rgb, g2d,
                           st->opts.no_pair_stats ? nullptr : st->counters + 2, s,
+                          raster_lanes(L, st->dopts, st->n_vis, st->n_pairs).bwd_two,
                           st->tile_order, st->work, st->store());
     }
     {

@@ -60,6 +60,12 @@ size_t forward_bytes(const HostLayout &L, int64_t n_vis, int64_t n_pairs,
 // (the point backward runs over the points of viewed scenes only).
 void zero_unviewed_grads(const HostLayout &L, float *grad_pos, float *grad_sh,
                          float *grad_opacity, cudaStream_t s);
+// Whether the compositing warps of a batch take 8 x 8 blocks (two pixels a
+// lane) or halves of them, from its sizes and list counts.
+struct RasterLanes {
+    bool fwd_two = true, bwd_two = true;
+};
+RasterLanes raster_lanes(const HostLayout &L, const DevOpts &o, int64_t n_vis, int64_t n_pairs);
 int dalloc(void **p, size_t bytes, cudaStream_t s);
 void dfree(void *p, cudaStream_t s);
 void serve_shutdown(pbr_ctx *c);

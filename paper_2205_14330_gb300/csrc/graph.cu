@@ -86,6 +86,7 @@ struct pbr_graph {
     // to depth_marker), instead of compacting the visible ones first
     bool direct_depth = false;
     uint32_t depth_marker = 0xffffffffu;
+    RasterLanes lanes;
     // buffers (cudaMalloc, stable addresses for the graphs)
     std::vector<void *> allocs;
     DevView *d_views = nullptr;
@@ -201,7 +202,8 @@ void enqueue_forward(pbr_graph *g, cudaStream_t s)
     const bool persist = g->opts.persistent && g->opts.batch_depth == 0;
     if (persist) launch_tile_order(b, g->ranges, L.n_tiles, g->order, g->work, s);
     launch_raster_fwd(b, o, g->opts.batch_depth, g->ranges, tk, tv, g->rec, g->out_rgb, g->T_final,
-                      g->n_contrib, nullptr, s, persist ? g->order : nullptr, g->work);
+                      g->n_contrib, nullptr, s, g->lanes.fwd_two, persist ? g->order : nullptr,
+                      g->work);
 }
 
 void enqueue_backward(pbr_graph *g, const float *grad_rgb, cudaStream_t s)
@@ -213,7 +215,7 @@ void enqueue_backward(pbr_graph *g, const float *grad_rgb, cudaStream_t s)
     if (persist) reset_work_counters(g->work, s);
     launch_raster_bwd(b, g->dopts, g->opts.batch_depth, g->ranges, g->keys_final, g->vals_final,
                       g->rec,
-                      g->T_final, g->n_contrib, grad_rgb, g->g2d, nullptr, s,
+                      g->T_final, g->n_contrib, grad_rgb, g->g2d, nullptr, s, g->lanes.bwd_two,
                       persist ? g->order : nullptr, g->work);
     launch_preprocess_bwd(b, g->dopts, g->g2d, g->grad_pos, g->grad_sh, g->grad_opacity, s);
     zero_unviewed_grads(L, g->grad_pos, g->grad_sh, g->grad_opacity, s);
@@ -308,6 +310,7 @@ int plan_and_capture(pbr_graph *g, cudaStream_t user_stream)
     }
     const uint64_t n_pairs = g->host[0], n_vis = g->host[1];
     const uint32_t zlo = ((uint32_t *)g->host)[12], zhi = ((uint32_t *)g->host)[13];
+    g->lanes = raster_lanes(L, g->dopts, (int64_t)n_vis, (int64_t)n_pairs);
     g->cap_vis = L.n_pv;
     g->cap_pairs = (int64_t)std::ceil((double)n_pairs * (1.0 + g->headroom)) + 4096;
     if (g->cap_pairs >= (int64_t)UINT32_MAX) g->cap_pairs = (int64_t)UINT32_MAX - 1;

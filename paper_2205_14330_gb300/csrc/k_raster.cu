@@ -29,13 +29,14 @@
 // entries of its own block, and it skips those whose cutoff disc misses its
 // still active pixels.  Three schedules:
 //   - warp-streamed (batch depth 0, default): a block covers one TW x TH
-//     screen tile, each warp an 8 x 8 block of it; a lane owns two pixels of
-//     a column, four rows apart.  Every warp walks its entries by itself, 32
-//     per step, culls them with one ballot, steps through the hits in
-//     lockstep and stops as soon as its own pixels have saturated.  No block
-//     barriers.
+//     screen tile, each warp an 8 x 8 block of it (a lane owns two pixels of
+//     a column, four rows apart) or, where few long lists decide the time,
+//     half of one (one pixel a lane; the rule is raster_lanes').  Every warp
+//     walks its entries by itself, 32 per step, culls them with one ballot,
+//     steps through the hits in lockstep and stops as soon as its own pixels
+//     have saturated.  No block barriers.
 //   - persistent (batch depth 0, persistent): the same walk in one launch;
-//     warps take (tile, 8 x 8 block) items longest list first from an atomic
+//     warps take (tile, unit) items longest list first from an atomic
 //     counter.
 //   - block-staged (batch depth > 0): the block stages `depth` records in
 //     shared memory and each warp culls the batch into its own list; block
@@ -496,8 +497,8 @@ struct FwdWarp {
     WarpQueue q;
 };
 
-// Forward of one 8 x 8 block by one warp: lane l owns the pixels (l & 7, l >>
-// 3) and (l & 7, 4 + (l >> 3)), gA and gB.  The warp takes the tile list's
+// Forward of one 8 x 8 block by one warp: lane l owns the pixels A = (l & 7, l
+// >> 3) and B = (l & 7, 4 + (l >> 3)).  The warp takes the tile list's
 // entries with its block's bit (`bit`) 32 at a time from its queue, culls
 // them against the rectangle of its active pixels and stages the hits in list
 // order; then it steps through them, every lane testing and blending the
@@ -508,10 +509,11 @@ struct FwdWarp {
 // COUNT: the points composited per pixel are counted (pair counts, store
 // mode, the count cap).
 // FUSED: the rounding of the squared distance (pair_d2).
-template <bool COUNT, bool STORE, bool FUSED>
-__device__ __forceinline__ void fwd_pair_item(const PixelGeom &gA, const PixelGeom &gB,
-                                              uint32_t s, uint32_t e, uint32_t bit,
-                                              const DevOpts &o, int lane,
+// NP: pixels a lane owns; with 1 the warp's pixels are the 8 x 4 sub-block
+// with first pixel (sx0, sy0), and what concerns pixel B compiles away.
+template <int NP, bool COUNT, bool STORE, bool FUSED>
+__device__ __forceinline__ void fwd_pair_item(const DevView *V, int sx0, int sy0, uint32_t s,
+                                              uint32_t e, uint32_t bit, const DevOpts &o, int lane,
                                               const uint32_t *__restrict__ keys,
                                               const uint32_t *__restrict__ pv_list,
                                               const float4 *__restrict__ rec,
@@ -521,12 +523,15 @@ __device__ __forceinline__ void fwd_pair_item(const PixelGeom &gA, const PixelGe
                                               uint32_t &examined_acc, uint32_t &composited_acc,
                                               FwdWarp &m, const StoreBuf &sto)
 {
+    PixelGeom g[NP];
+#pragma unroll
+    for (int q = 0; q < NP; ++q) g[q] = pixel_geom_at(V, sx0, sy0 + 4 * q, lane);
+    const PixelGeom &gA = g[0], &gB = g[NP - 1];
     const int64_t pixA = STORE && gA.inside ? pixel_index(gA) : 0;
     const int64_t pixB = STORE && gB.inside ? pixel_index(gB) : 0;
-    float2 T = make_float2(gA.inside ? 1.0f : -1.0f, gB.inside ? 1.0f : -1.0f);
+    float2 T = make_float2(gA.inside ? 1.0f : -1.0f, NP == 2 && gB.inside ? 1.0f : -1.0f);
     float2 C0 = f2(0.0f), C1 = f2(0.0f), C2 = f2(0.0f);
     uint32_t cntA = 0, cntB = 0, lastA = 0, lastB = 0, examined = 0;
-    const PixelGeom g2[2] = {gA, gB};
     const float ux = gA.ux;
     const float2 uy = make_float2(gA.uy, gB.uy);
     const float eps = o.t_eps, amax = o.alpha_max;
@@ -537,8 +542,10 @@ __device__ __forceinline__ void fwd_pair_item(const PixelGeom &gA, const PixelGe
     int qn = 0;
     uint32_t qh = 0;
     while (true) {
-        const bool act[2] = {T.x >= eps && cntA < cmax, T.y >= eps && cntB < cmax};
-        if (!__any_sync(0xffffffffu, act[0] || act[1])) break;
+        bool act[NP];
+        act[NP - 1] = T.y >= eps && cntB < cmax;
+        act[0] = T.x >= eps && cntA < cmax;
+        if (!__any_sync(0xffffffffu, act[0] || act[NP - 1])) break;
         queue_fill_front(keys, pv_list, s, e, bit, p, qn, qh, m.q, lane);
         if (qn == 0) break;
         uint32_t rel = 0, pv = 0;
@@ -550,7 +557,7 @@ __device__ __forceinline__ void fwd_pair_item(const PixelGeom &gA, const PixelGe
             c = __ldg(rec + 2 * (size_t)pv + 1);
         }
         // every lane takes part in the reductions, whatever its entry
-        const PixelGeom ar = active_rect_rows<2>(g2, act);
+        const PixelGeom ar = active_rect_rows<NP>(g, act);
         const bool hit = valid && disc_meets_rect(a, ar);
         const uint32_t hm = __ballot_sync(0xffffffffu, hit);
         const int nh = __popc(hm);
@@ -560,7 +567,7 @@ __device__ __forceinline__ void fwd_pair_item(const PixelGeom &gA, const PixelGe
         m.c[slot] = hit ? c : make_float4(0.f, 0.f, 0.f, 0.f);
         m.pos[slot] = rel;
         __syncwarp();
-        if (COUNT) examined += (uint32_t)nh * ((uint32_t)act[0] + (uint32_t)act[1]);
+        if (COUNT) examined += (uint32_t)nh * ((uint32_t)act[0] + (uint32_t)(NP == 2 && act[NP - 1]));
         // the chunk's last composited hit of each pixel
         int jA = -1, jB = -1;
         constexpr int FWD_UNROLL = STORE ? 2 : 4;
@@ -571,13 +578,14 @@ __device__ __forceinline__ void fwd_pair_item(const PixelGeom &gA, const PixelGe
                 float dx;
                 float2 dy;
                 const float2 d2 = pair_d2<FUSED>(ux, uy, aj.x, aj.y, dx, dy);
-                bool inA = d2.x <= aj.z && T.x >= eps, inB = d2.y <= aj.z && T.y >= eps;
+                bool inA = d2.x <= aj.z && T.x >= eps;
+                bool inB = NP == 2 && d2.y <= aj.z && T.y >= eps;
                 if (COUNT) {
                     inA = inA && cntA < cmax;
                     inB = inB && cntB < cmax;
                 }
                 const float rawA = __fmul_rn(cj.x, ex2_approx(__fmul_rn(d2.x, aj.w)));
-                const float rawB = __fmul_rn(cj.x, ex2_approx(__fmul_rn(d2.y, aj.w)));
+                const float rawB = NP == 2 ? __fmul_rn(cj.x, ex2_approx(__fmul_rn(d2.y, aj.w))) : 0.0f;
                 if (STORE) {
                     if (inA) store_T(sto, pixA, cntA, T.x);
                     if (inB) store_T(sto, pixB, cntB, T.y);
@@ -611,10 +619,10 @@ __device__ __forceinline__ void fwd_pair_item(const PixelGeom &gA, const PixelGe
     }
     if (STORE) {
         if (gA.inside) sto.n[pixA] = cntA;
-        if (gB.inside) sto.n[pixB] = cntB;
+        if (NP == 2 && gB.inside) sto.n[pixB] = cntB;
     }
     write_pixel(gA, o, T.x, C0.x, C1.x, C2.x, lastA, out_rgb, T_final, n_contrib);
-    write_pixel(gB, o, T.y, C0.y, C1.y, C2.y, lastB, out_rgb, T_final, n_contrib);
+    if (NP == 2) write_pixel(gB, o, T.y, C0.y, C1.y, C2.y, lastB, out_rgb, T_final, n_contrib);
 }
 
 // ------------------------------------------------------------- backward
@@ -629,6 +637,9 @@ __device__ __forceinline__ void fwd_pair_item(const PixelGeom &gA, const PixelGe
 // and no reduction, but its shared-memory traffic made the L1 path the bound:
 // 8.84-9.3 ms against 8.87.
 constexpr int BWD_DIRECT_MAX = 24;
+// One-pixel lanes: an earlier form of the loop took 13.0 ms at 12 and 16, 13.4
+// at 20, 14.5 at 2 and 22.1 with atomics only on the same batch.
+constexpr int BWD_DIRECT_MAX_ONE = 16;
 
 // One warp's shared memory of the backward.
 struct BwdWarp {
@@ -680,13 +691,13 @@ struct PairAlpha {
 // squared distances.  CLAMP 0: the point's amplitude is below the clamp, so
 // alpha is too.  Operands that are the point's own stay scalar (a packed
 // operation would need them duplicated).
-template <bool CLAMP>
+template <int NP, bool CLAMP>
 __device__ __forceinline__ PairAlpha pair_alpha(bool tA, bool tB, float2 d2, const float4 a,
                                                 const float4 c, float amax, const BwdPair &p)
 {
     PairAlpha r;
     r.G.x = ex2_approx(__fmul_rn(d2.x, a.w));
-    r.G.y = ex2_approx(__fmul_rn(d2.y, a.w));
+    r.G.y = NP == 2 ? ex2_approx(__fmul_rn(d2.y, a.w)) : 0.0f;
     if (CLAMP) {
         const float rawA = c.x * r.G.x, rawB = c.x * r.G.y;
         r.alpha = make_float2(tA ? fminf(amax, rawA) : 0.0f, tB ? fminf(amax, rawB) : 0.0f);
@@ -696,9 +707,9 @@ __device__ __forceinline__ PairAlpha pair_alpha(bool tA, bool tB, float2 d2, con
         r.alpha = make_float2(c.x * r.G.x, c.x * r.G.y);
     }
     const float2 om = fma2(r.alpha, f2(-1.0f), f2(1.0f));
-    r.rom = make_float2(rcp_approx(om.x), rcp_approx(om.y));
+    r.rom = make_float2(rcp_approx(om.x), NP == 2 ? rcp_approx(om.y) : 1.0f);
     r.cg = make_float2(fmaf(c.w, p.g2.x, fmaf(c.z, p.g1.x, c.y * p.g0.x)),
-                       fmaf(c.w, p.g2.y, fmaf(c.z, p.g1.y, c.y * p.g0.y)));
+                       NP == 2 ? fmaf(c.w, p.g2.y, fmaf(c.z, p.g1.y, c.y * p.g0.y)) : 0.0f);
     return r;
 }
 
@@ -706,6 +717,7 @@ __device__ __forceinline__ PairAlpha pair_alpha(bool tA, bool tB, float2 d2, con
 // pixels: v = {t0, t1, t2, do, dr, dg, db, 0}; updates T and S.  hasA /
 // hasB: tb holds the stored transmittance before the point (store mode)
 // instead of the one recovered by division.
+template <int NP>
 __device__ __forceinline__ void pair_recur(const PairAlpha &r, float2 d2, float dx, float2 dy,
                                            BwdPair &p, bool hasA, bool hasB, float2 tb, float v[8])
 {
@@ -720,22 +732,24 @@ __device__ __forceinline__ void pair_recur(const PairAlpha &r, float2 d2, float 
     const float2 dG = mul2(dalpha, r.G);
     const float2 t1 = mul2(dG, dy), t2 = mul2(dG, d2);
     const float2 t4 = mul2(w, p.g0), t5 = mul2(w, p.g1), t6 = mul2(w, p.g2);
-    v[3] = dG.x + dG.y;
+    auto sum = [](float2 t) { return NP == 2 ? t.x + t.y : t.x; };
+    v[3] = sum(dG);
     v[0] = v[3] * dx;
-    v[1] = t1.x + t1.y;
-    v[2] = t2.x + t2.y;
-    v[4] = t4.x + t4.y;
-    v[5] = t5.x + t5.y;
-    v[6] = t6.x + t6.y;
+    v[1] = sum(t1);
+    v[2] = sum(t2);
+    v[4] = sum(t4);
+    v[5] = sum(t5);
+    v[6] = sum(t6);
     v[7] = 0.0f;
 }
 
 // Adds one point's terms to its slot of the gradient buffer; cm: the lanes
 // with a contributing pixel.
+template <int NP>
 __device__ __forceinline__ void bwd_add(uint32_t cm, bool any, const float v[8], int lane,
                                         float *__restrict__ g2d, uint32_t pv)
 {
-    if (__popc(cm) > BWD_DIRECT_MAX) {
+    if (__popc(cm) > (NP == 2 ? BWD_DIRECT_MAX : BWD_DIRECT_MAX_ONE)) {
         warp_add_terms(v, lane, g2d, pv);
     } else if (any) { // few lanes: each adds its own terms
         float4 *dst = reinterpret_cast<float4 *>(g2d) + 2 * (size_t)pv;
@@ -745,7 +759,7 @@ __device__ __forceinline__ void bwd_add(uint32_t cm, bool any, const float v[8],
 }
 
 // Back-propagates one chunk of nh staged hits through the lane's pixels.
-template <bool CLAMP, bool STATS, bool STORE, bool FUSED>
+template <int NP, bool CLAMP, bool STATS, bool STORE, bool FUSED>
 __device__ __forceinline__ void bwd_chunk(const BwdWarp &m, int nh, float ux, float2 uy,
                                           float amax, int lane, BwdPair &p,
                                           float *__restrict__ g2d, uint32_t &examined,
@@ -768,7 +782,7 @@ __device__ __forceinline__ void bwd_chunk(const BwdWarp &m, int nh, float ux, fl
             const uint2 ip = m.ip[j0 + u];
             pv[u] = ip.y;
             d2[u] = pair_d2<FUSED>(ux, uy, aj.x, aj.y, dx[u], dy[u]);
-            const bool bA = ip.x < p.LA, bB = ip.x < p.LB;
+            const bool bA = ip.x < p.LA, bB = NP == 2 && ip.x < p.LB;
             const bool tA = bA && d2[u].x <= aj.z, tB = bB && d2[u].y <= aj.z;
             if (STATS) {
                 examined += (uint32_t)bA + (uint32_t)bB;
@@ -779,17 +793,17 @@ __device__ __forceinline__ void bwd_chunk(const BwdWarp &m, int nh, float ux, fl
             tb[u] = f2(0.0f);
             if (STORE) {
                 hasA[u] = row_next(rowA, tA, tb[u].x);
-                hasB[u] = row_next(rowB, tB, tb[u].y);
+                if (NP == 2) hasB[u] = row_next(rowB, tB, tb[u].y);
             }
-            pr[u] = pair_alpha<CLAMP>(tA, tB, d2[u], aj, cj, amax, p);
+            pr[u] = pair_alpha<NP, CLAMP>(tA, tB, d2[u], aj, cj, amax, p);
         }
 #pragma unroll
         for (int u = 0; u < BWD_UNROLL; ++u) {
             const uint32_t cm = __ballot_sync(0xffffffffu, any[u]);
             if (!cm) continue;
             float v[8];
-            pair_recur(pr[u], d2[u], dx[u], dy[u], p, hasA[u], hasB[u], tb[u], v);
-            bwd_add(cm, any[u], v, lane, g2d, pv[u]);
+            pair_recur<NP>(pr[u], d2[u], dx[u], dy[u], p, hasA[u], hasB[u], tb[u], v);
+            bwd_add<NP>(cm, any[u], v, lane, g2d, pv[u]);
         }
     }
 }
@@ -802,8 +816,8 @@ __device__ __forceinline__ void bwd_chunk(const BwdWarp &m, int nh, float ux, fl
 // records of the next 32 are in flight while these are processed.  Per hit
 // the lane forms the adjoint at both pixels (packed fp32x2) and adds the two
 // term vectors, so the per-point warp work serves 64 pixels.  s: the start
-// of the tile's list.
-template <bool STATS, bool STORE, bool FUSED>
+// of the tile's list.  NP: see fwd_pair_item.
+template <int NP, bool STATS, bool STORE, bool FUSED>
 __device__ __forceinline__ void bwd_pair_item(const DevView *V, int sx0, int sy0, uint32_t s,
                                               uint32_t bit, const DevOpts &o, int lane,
                                               const uint32_t *__restrict__ keys,
@@ -815,11 +829,12 @@ __device__ __forceinline__ void bwd_pair_item(const DevView *V, int sx0, int sy0
                                               float *__restrict__ g2d, uint32_t &examined,
                                               uint32_t &used, BwdWarp &m, const StoreBuf &sto)
 {
-    PixelGeom g[2];
-    g[0] = pixel_geom_at(V, sx0, sy0, lane);
-    g[1] = pixel_geom_at(V, sx0, sy0 + 4, lane);
+    PixelGeom g[NP];
+#pragma unroll
+    for (int q = 0; q < NP; ++q) g[q] = pixel_geom_at(V, sx0, sy0 + 4 * q, lane);
     const BwdPixel pa = bwd_pixel(g[0], o, T_final, n_contrib, grad_rgb);
-    const BwdPixel pb = bwd_pixel(g[1], o, T_final, n_contrib, grad_rgb);
+    BwdPixel pb{1.0f, 0.f, 0.f, 0.f, 0.f, 0u};
+    if (NP == 2) pb = bwd_pixel(g[NP - 1], o, T_final, n_contrib, grad_rgb);
     BwdPair p;
     p.T = make_float2(pa.T, pb.T);
     p.S = make_float2(pa.S, pb.S);
@@ -834,11 +849,12 @@ __device__ __forceinline__ void bwd_pair_item(const DevView *V, int sx0, int sy0
     StoreRow rowA, rowB;
     if (STORE) {
         rowA = store_row(sto, g[0].inside ? pixel_index(g[0]) : 0, g[0].inside);
-        rowB = store_row(sto, g[1].inside ? pixel_index(g[1]) : 0, g[1].inside);
+        if (NP == 2)
+            rowB = store_row(sto, g[NP - 1].inside ? pixel_index(g[NP - 1]) : 0, g[NP - 1].inside);
     }
     const uint32_t lt = lanemask_lt_r();
     const float ux = g[0].ux;
-    const float2 uy = make_float2(g[0].uy, g[1].uy);
+    const float2 uy = make_float2(g[0].uy, g[NP - 1].uy);
     int64_t c = (int64_t)((wmax - 1) & ~31u);
     int qn = 0;
     uint32_t qh = 0;
@@ -858,8 +874,10 @@ __device__ __forceinline__ void bwd_pair_item(const DevView *V, int sx0, int sy0
         // pixels whose composited list reaches the chunk's nearest entry;
         // every lane takes part in the reductions, whatever its entry
         const uint32_t lowest = __shfl_sync(0xffffffffu, rel, take - 1);
-        const bool act[2] = {p.LA > lowest, p.LB > lowest};
-        const PixelGeom ar = active_rect_rows<2>(g, act);
+        bool act[NP];
+        act[NP - 1] = p.LB > lowest;
+        act[0] = p.LA > lowest;
+        const PixelGeom ar = active_rect_rows<NP>(g, act);
         const bool hit = lane < take && disc_meets_rect(ra, ar);
         const uint32_t hm = __ballot_sync(0xffffffffu, hit);
         // amplitudes that may reach the clamp (a NaN counts as one)
@@ -873,42 +891,59 @@ __device__ __forceinline__ void bwd_pair_item(const DevView *V, int sx0, int sy0
         __syncwarp();
         fetch();
         if (clamp)
-            bwd_chunk<true, STATS, STORE, FUSED>(m, nh, ux, uy, o.alpha_max, lane, p, g2d,
+            bwd_chunk<NP, true, STATS, STORE, FUSED>(m, nh, ux, uy, o.alpha_max, lane, p, g2d,
                                                  examined, used, rowA, rowB);
         else
-            bwd_chunk<false, STATS, STORE, FUSED>(m, nh, ux, uy, o.alpha_max, lane, p, g2d,
+            bwd_chunk<NP, false, STATS, STORE, FUSED>(m, nh, ux, uy, o.alpha_max, lane, p, g2d,
                                                   examined, used, rowA, rowB);
         __syncwarp(); // chunk consumed before the buffers are refilled
     }
 }
 
-// Warp-streamed: one block per tile, warp w takes the tile's 8 x 8 block w.
-template <int TW, int TH, bool COUNT, bool STORE>
-__global__ void __launch_bounds__(TW * TH / 2)
+// First pixel of unit `w` of a tile, and its block's bit in the pair keys'
+// masks (0 when a tile is a single block).  NP 2: the units are the tile's 8 x
+// 8 blocks, numbered like the masks' bits; NP 1: their upper and lower halves.
+template <int TW, int TH, int NP>
+__device__ __forceinline__ uint32_t unit_of(int tx, int ty, int w, int &sx0, int &sy0)
+{
+    const int blk = NP == 2 ? w : w >> 1;
+    sx0 = tx * TW + (blk % (TW / 8)) * 8;
+    sy0 = ty * TH + (blk / (TW / 8)) * 8 + (NP == 2 ? 0 : 4 * (w & 1));
+    return block_bits(TW, TH) ? 1u << blk : 0u;
+}
+
+template <int TW, int TH, int NP>
+__host__ __device__ constexpr int units()
+{
+    return TW * TH / (32 * NP);
+}
+
+// Warp-streamed: one block per tile, warp w takes the tile's unit w.
+template <int TW, int TH, int NP, bool COUNT, bool STORE>
+__global__ void __launch_bounds__(units<TW, TH, NP>() * 32)
 raster_fwd_stream_kernel(Batch b, DevOpts o, const uint2 *__restrict__ ranges,
                          const uint32_t *__restrict__ keys, const uint32_t *__restrict__ pv_list,
                          const float4 *__restrict__ rec, float *__restrict__ out_rgb,
                          float *__restrict__ T_final, uint32_t *__restrict__ n_contrib,
                          unsigned long long *__restrict__ stats, StoreBuf sto)
 {
-    __shared__ FwdWarp s_fwd[TW * TH / 64];
+    __shared__ FwdWarp s_fwd[units<TW, TH, NP>()];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const DevView *V = &b.views[find_view_by_tile(b, blockIdx.x)];
     const uint32_t local = blockIdx.x - V->tile_base;
     const int tx = (int)(local % (uint32_t)V->tiles_x), ty = (int)(local / (uint32_t)V->tiles_x);
-    const int sx0 = tx * TW + (w % (TW / 8)) * 8, sy0 = ty * TH + (w / (TW / 8)) * 8;
-    const uint32_t bit = block_bits(TW, TH) ? 1u << w : 0u;
+    int sx0, sy0;
+    const uint32_t bit = unit_of<TW, TH, NP>(tx, ty, w, sx0, sy0);
     const uint2 rg = ranges[blockIdx.x];
     uint32_t ex = 0, co = 0;
-    fwd_pair_item<COUNT, STORE, false>(pixel_geom_at(V, sx0, sy0, lane),
-                                pixel_geom_at(V, sx0, sy0 + 4, lane), rg.x,
-                                rg.y > rg.x ? rg.y : rg.x, bit, o, lane, keys, pv_list, rec,
-                                out_rgb, T_final, n_contrib, ex, co, s_fwd[w], sto);
+    fwd_pair_item<NP, COUNT, STORE, false>(V, sx0, sy0, rg.x, rg.y > rg.x ? rg.y : rg.x, bit, o,
+                                           lane, keys, pv_list, rec, out_rgb, T_final, n_contrib,
+                                           ex, co, s_fwd[w], sto);
     if (COUNT) add_stats(stats, ex, co, lane);
 }
 
-template <int TW, int TH, bool STATS, bool STORE>
-__global__ void __launch_bounds__(TW * TH / 2)
+template <int TW, int TH, int NP, bool STATS, bool STORE>
+__global__ void __launch_bounds__(units<TW, TH, NP>() * 32)
 raster_bwd_stream_kernel(Batch b, DevOpts o, const uint2 *__restrict__ ranges,
                          const uint32_t *__restrict__ keys, const uint32_t *__restrict__ pv_list,
                          const float4 *__restrict__ rec, const float *__restrict__ T_final,
@@ -916,16 +951,17 @@ raster_bwd_stream_kernel(Batch b, DevOpts o, const uint2 *__restrict__ ranges,
                          float *__restrict__ g2d, unsigned long long *__restrict__ stats,
                          StoreBuf sto)
 {
-    __shared__ BwdWarp s_bwd[TW * TH / 64];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5; // warp w: the tile's 8 x 8 block w
+    __shared__ BwdWarp s_bwd[units<TW, TH, NP>()];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const DevView *V = &b.views[find_view_by_tile(b, blockIdx.x)];
     const uint32_t local = blockIdx.x - V->tile_base;
     const int tx = (int)(local % (uint32_t)V->tiles_x), ty = (int)(local / (uint32_t)V->tiles_x);
-    const uint32_t bit = block_bits(TW, TH) ? 1u << w : 0u;
+    int sx0, sy0;
+    const uint32_t bit = unit_of<TW, TH, NP>(tx, ty, w, sx0, sy0);
     uint32_t ex = 0, us = 0;
-    bwd_pair_item<STATS, STORE, false>(V, tx * TW + (w % (TW / 8)) * 8, ty * TH + (w / (TW / 8)) * 8,
-                                ranges[blockIdx.x].x, bit, o, lane, keys, pv_list, rec, T_final,
-                                n_contrib, grad_rgb, g2d, ex, us, s_bwd[w], sto);
+    bwd_pair_item<NP, STATS, STORE, false>(V, sx0, sy0, ranges[blockIdx.x].x, bit, o, lane, keys,
+                                           pv_list, rec, T_final, n_contrib, grad_rgb, g2d, ex, us,
+                                           s_bwd[w], sto);
     if (STATS) add_stats(stats ? stats + 2 : nullptr, ex, us, lane);
 }
 
@@ -963,7 +999,7 @@ __device__ __forceinline__ uint4 tile_desc(const Batch &b, const uint2 *ranges, 
 // 1M-point, 64-view step against 4.10 at four and 4.27 at six (unrolled by
 // two).  The backward runs best at four (64 registers): 8.87 ms, 9.07 at
 // three, 8.96 at five.
-template <int TW, int TH, bool COUNT, bool STORE>
+template <int TW, int TH, int NP, bool COUNT, bool STORE>
 __global__ void __launch_bounds__(PERSIST_THREADS, FWD_PERSIST_BLOCKS)
 raster_fwd_persist_kernel(Batch b, DevOpts o, const uint2 *__restrict__ ranges,
                           const uint32_t *__restrict__ keys, const uint32_t *__restrict__ pv_list,
@@ -972,7 +1008,7 @@ raster_fwd_persist_kernel(Batch b, DevOpts o, const uint2 *__restrict__ ranges,
                           unsigned long long *__restrict__ stats, const uint4 *__restrict__ order,
                           uint32_t *work, StoreBuf sto)
 {
-    constexpr uint32_t SUBS = (TW / 8) * (TH / 8);
+    constexpr uint32_t SUBS = units<TW, TH, NP>();
     constexpr int NW = PERSIST_THREADS / 32;
     __shared__ FwdWarp s_fwd[NW];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -981,20 +1017,18 @@ raster_fwd_persist_kernel(Batch b, DevOpts o, const uint2 *__restrict__ ranges,
     for (uint32_t it = next_item(work, lane); it < n_items; it = next_item(work, lane)) {
         const uint4 d = order[it / SUBS];
         const int sub = (int)(it % SUBS);
-        const DevView *V = &b.views[d.x];
-        const int sx0 = (int)(d.y & 0xffffu) * TW + (sub % (TW / 8)) * 8;
-        const int sy0 = (int)(d.y >> 16) * TH + (sub / (TW / 8)) * 8;
-        const uint32_t bit = block_bits(TW, TH) ? 1u << sub : 0u;
-        fwd_pair_item<COUNT, STORE, true>(pixel_geom_at(V, sx0, sy0, lane),
-                                    pixel_geom_at(V, sx0, sy0 + 4, lane), d.z, d.w, bit, o, lane,
-                                    keys, pv_list, rec, out_rgb, T_final, n_contrib, ex, co,
-                                    s_fwd[w], sto);
+        int sx0, sy0;
+        const uint32_t bit =
+            unit_of<TW, TH, NP>((int)(d.y & 0xffffu), (int)(d.y >> 16), sub, sx0, sy0);
+        fwd_pair_item<NP, COUNT, STORE, true>(&b.views[d.x], sx0, sy0, d.z, d.w, bit, o, lane,
+                                              keys, pv_list, rec, out_rgb, T_final, n_contrib, ex,
+                                              co, s_fwd[w], sto);
         __syncwarp(); // the item's shared memory is read before the next one writes it
     }
     if (COUNT) add_stats(stats, ex, co, lane);
 }
 
-template <int TW, int TH, bool STATS, bool STORE>
+template <int TW, int TH, int NP, bool STATS, bool STORE>
 __global__ void __launch_bounds__(PERSIST_THREADS, BWD_PERSIST_BLOCKS)
 raster_bwd_persist_kernel(Batch b, DevOpts o, const uint2 *__restrict__ ranges,
                           const uint32_t *__restrict__ keys, const uint32_t *__restrict__ pv_list,
@@ -1004,8 +1038,7 @@ raster_bwd_persist_kernel(Batch b, DevOpts o, const uint2 *__restrict__ ranges,
                           unsigned long long *__restrict__ stats, const uint4 *__restrict__ order,
                           uint32_t *work, StoreBuf sto)
 {
-    // 8 x 8 blocks, numbered like the key masks
-    constexpr uint32_t SUBS = (TW / 8) * (TH / 8);
+    constexpr uint32_t SUBS = units<TW, TH, NP>();
     __shared__ BwdWarp s_bwd[PERSIST_THREADS / 32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const uint32_t n_items = b.n_tiles * SUBS;
@@ -1013,11 +1046,12 @@ raster_bwd_persist_kernel(Batch b, DevOpts o, const uint2 *__restrict__ ranges,
     for (uint32_t it = next_item(work, lane); it < n_items; it = next_item(work, lane)) {
         const uint4 d = order[it / SUBS];
         const int sub = (int)(it % SUBS);
-        const uint32_t bit = block_bits(TW, TH) ? 1u << sub : 0u;
-        const int sx0 = (int)(d.y & 0xffffu) * TW + (sub % (TW / 8)) * 8;
-        const int sy0 = (int)(d.y >> 16) * TH + (sub / (TW / 8)) * 8;
-        bwd_pair_item<STATS, STORE, true>(&b.views[d.x], sx0, sy0, d.z, bit, o, lane, keys, pv_list, rec,
-                                    T_final, n_contrib, grad_rgb, g2d, ex, us, s_bwd[w], sto);
+        int sx0, sy0;
+        const uint32_t bit =
+            unit_of<TW, TH, NP>((int)(d.y & 0xffffu), (int)(d.y >> 16), sub, sx0, sy0);
+        bwd_pair_item<NP, STATS, STORE, true>(&b.views[d.x], sx0, sy0, d.z, bit, o, lane, keys,
+                                              pv_list, rec, T_final, n_contrib, grad_rgb, g2d, ex,
+                                              us, s_bwd[w], sto);
         __syncwarp(); // the item's shared memory is read before the next one writes it
     }
     if (STATS) add_stats(stats ? stats + 2 : nullptr, ex, us, lane);
@@ -1264,7 +1298,7 @@ int persist_grid(const void *kernel)
     return sms * (per_sm > 0 ? per_sm : 1);
 }
 
-template <int TW, int TH, bool COUNT, bool STORE>
+template <int TW, int TH, int NP, bool COUNT, bool STORE>
 void fwd_launch(const Batch &b, const DevOpts &o, const uint2 *ranges, const uint32_t *keys,
                 const uint32_t *pv_list, const float4 *rec, float *out_rgb, float *T_final,
                 uint32_t *n_contrib, unsigned long long *stats, const uint4 *order, uint32_t *work,
@@ -1272,17 +1306,17 @@ void fwd_launch(const Batch &b, const DevOpts &o, const uint2 *ranges, const uin
 {
     if (order) {
         static const int grid =
-            persist_grid((const void *)raster_fwd_persist_kernel<TW, TH, COUNT, STORE>);
-        raster_fwd_persist_kernel<TW, TH, COUNT, STORE><<<grid, PERSIST_THREADS, 0, s>>>(
+            persist_grid((const void *)raster_fwd_persist_kernel<TW, TH, NP, COUNT, STORE>);
+        raster_fwd_persist_kernel<TW, TH, NP, COUNT, STORE><<<grid, PERSIST_THREADS, 0, s>>>(
             b, o, ranges, keys, pv_list, rec, out_rgb, T_final, n_contrib, stats, order, work,
             sto);
     } else {
-        raster_fwd_stream_kernel<TW, TH, COUNT, STORE><<<b.n_tiles, TW * TH / 2, 0, s>>>(
+        raster_fwd_stream_kernel<TW, TH, NP, COUNT, STORE><<<b.n_tiles, units<TW, TH, NP>() * 32, 0, s>>>(
             b, o, ranges, keys, pv_list, rec, out_rgb, T_final, n_contrib, stats, sto);
     }
 }
 
-template <int TW, int TH, bool STATS, bool STORE>
+template <int TW, int TH, int NP, bool STATS, bool STORE>
 void bwd_launch(const Batch &b, const DevOpts &o, const uint2 *ranges, const uint32_t *keys,
                 const uint32_t *pv_list, const float4 *rec, const float *T_final,
                 const uint32_t *n_contrib, const float *grad_rgb, float4 *g2d,
@@ -1291,12 +1325,12 @@ void bwd_launch(const Batch &b, const DevOpts &o, const uint2 *ranges, const uin
 {
     if (order) {
         static const int grid =
-            persist_grid((const void *)raster_bwd_persist_kernel<TW, TH, STATS, STORE>);
-        raster_bwd_persist_kernel<TW, TH, STATS, STORE><<<grid, PERSIST_THREADS, 0, s>>>(
+            persist_grid((const void *)raster_bwd_persist_kernel<TW, TH, NP, STATS, STORE>);
+        raster_bwd_persist_kernel<TW, TH, NP, STATS, STORE><<<grid, PERSIST_THREADS, 0, s>>>(
             b, o, ranges, keys, pv_list, rec, T_final, n_contrib, grad_rgb, (float *)g2d, stats,
             order, work + 1, sto);
     } else {
-        raster_bwd_stream_kernel<TW, TH, STATS, STORE><<<b.n_tiles, TW * TH / 2, 0, s>>>(
+        raster_bwd_stream_kernel<TW, TH, NP, STATS, STORE><<<b.n_tiles, units<TW, TH, NP>() * 32, 0, s>>>(
             b, o, ranges, keys, pv_list, rec, T_final, n_contrib, grad_rgb, (float *)g2d, stats,
             sto);
     }
@@ -1310,13 +1344,17 @@ void fwd_dispatch(const Batch &b, const DevOpts &o, int depth, const uint2 *rang
                   const uint32_t *keys, const uint32_t *pv_list, const float4 *rec,
                   float *out_rgb, float *T_final,
                   uint32_t *n_contrib, unsigned long long *stats, const uint4 *order,
-                  uint32_t *work, cudaStream_t s, const StoreBuf &sto)
+                  uint32_t *work, cudaStream_t s, const StoreBuf &sto, bool two)
 {
     const bool store = sto.T != nullptr;
     if (depth == 0) {
-        auto f = store ? fwd_launch<TW, TH, true, true>
-                 : stats || o.max_per_pixel ? fwd_launch<TW, TH, true, false>
-                                            : fwd_launch<TW, TH, false, false>;
+        const bool count = stats || o.max_per_pixel;
+        auto f = two ? (store ? fwd_launch<TW, TH, 2, true, true>
+                        : count ? fwd_launch<TW, TH, 2, true, false>
+                                : fwd_launch<TW, TH, 2, false, false>)
+                     : (store ? fwd_launch<TW, TH, 1, true, true>
+                        : count ? fwd_launch<TW, TH, 1, true, false>
+                                : fwd_launch<TW, TH, 1, false, false>);
         f(b, o, ranges, keys, pv_list, rec, out_rgb, T_final, n_contrib, stats, order, work, s,
           sto);
     } else {
@@ -1338,13 +1376,16 @@ void bwd_dispatch(const Batch &b, const DevOpts &o, int depth, const uint2 *rang
                   const float *T_final,
                   const uint32_t *n_contrib, const float *grad_rgb, float4 *g2d,
                   unsigned long long *stats, const uint4 *order, uint32_t *work,
-                  cudaStream_t s, const StoreBuf &sto)
+                  cudaStream_t s, const StoreBuf &sto, bool two)
 {
     const bool store = sto.T != nullptr;
     if (depth == 0) {
-        auto f = store ? bwd_launch<TW, TH, true, true>
-                 : stats ? bwd_launch<TW, TH, true, false>
-                         : bwd_launch<TW, TH, false, false>;
+        auto f = two ? (store ? bwd_launch<TW, TH, 2, true, true>
+                        : stats ? bwd_launch<TW, TH, 2, true, false>
+                                : bwd_launch<TW, TH, 2, false, false>)
+                     : (store ? bwd_launch<TW, TH, 1, true, true>
+                        : stats ? bwd_launch<TW, TH, 1, true, false>
+                                : bwd_launch<TW, TH, 1, false, false>);
         f(b, o, ranges, keys, pv_list, rec, T_final, n_contrib, grad_rgb, g2d, stats, order, work,
           s, sto);
     } else {
@@ -1382,37 +1423,37 @@ void reset_work_counters(uint32_t *work, cudaStream_t s)
 void launch_raster_fwd(const Batch &b, const DevOpts &o, int depth, const uint2 *ranges,
                        const uint32_t *keys, const uint32_t *pv_list, const float4 *rec,
                        float *out_rgb, float *T_final, uint32_t *n_contrib,
-                       unsigned long long *stats, cudaStream_t s, const uint4 *order,
+                       unsigned long long *stats, cudaStream_t s, bool two, const uint4 *order,
                        uint32_t *work, const StoreBuf &sto)
 {
     if (b.n_tiles == 0) return;
     if (o.tile_w == 8 && o.tile_h == 8)
         fwd_dispatch<8, 8>(b, o, depth, ranges, keys, pv_list, rec, out_rgb, T_final, n_contrib,
-                           stats, order, work, s, sto);
+                           stats, order, work, s, sto, two);
     else if (o.tile_w == 16 && o.tile_h == 32)
         fwd_dispatch<16, 32>(b, o, depth, ranges, keys, pv_list, rec, out_rgb, T_final,
-                             n_contrib, stats, order, work, s, sto);
+                             n_contrib, stats, order, work, s, sto, two);
     else
         fwd_dispatch<16, 16>(b, o, depth, ranges, keys, pv_list, rec, out_rgb, T_final,
-                             n_contrib, stats, order, work, s, sto);
+                             n_contrib, stats, order, work, s, sto, two);
 }
 
 void launch_raster_bwd(const Batch &b, const DevOpts &o, int depth, const uint2 *ranges,
                        const uint32_t *keys, const uint32_t *pv_list, const float4 *rec,
                        const float *T_final, const uint32_t *n_contrib, const float *grad_rgb,
-                       float4 *g2d, unsigned long long *stats, cudaStream_t s,
+                       float4 *g2d, unsigned long long *stats, cudaStream_t s, bool two,
                        const uint4 *order, uint32_t *work, const StoreBuf &sto)
 {
     if (b.n_tiles == 0) return;
     if (o.tile_w == 8 && o.tile_h == 8)
         bwd_dispatch<8, 8>(b, o, depth, ranges, keys, pv_list, rec, T_final, n_contrib, grad_rgb,
-                           g2d, stats, order, work, s, sto);
+                           g2d, stats, order, work, s, sto, two);
     else if (o.tile_w == 16 && o.tile_h == 32)
         bwd_dispatch<16, 32>(b, o, depth, ranges, keys, pv_list, rec, T_final, n_contrib,
-                             grad_rgb, g2d, stats, order, work, s, sto);
+                             grad_rgb, g2d, stats, order, work, s, sto, two);
     else
         bwd_dispatch<16, 16>(b, o, depth, ranges, keys, pv_list, rec, T_final, n_contrib,
-                             grad_rgb, g2d, stats, order, work, s, sto);
+                             grad_rgb, g2d, stats, order, work, s, sto, two);
 }
 
 } // namespace pbr

@@ -365,6 +365,8 @@ struct StoreBuf {
     int64_t n_pix = 0;
 };
 
+// two: a warp of the warp-streamed and persistent schedules takes an 8 x 8
+// block, two pixels a lane; else half of one (see raster_lanes).
 // batch_depth 0 = warp-streamed, > 0 = block-staged.  With order/work set
 // (warp-streamed only) the launch is persistent: warps pull (tile,
 // sub-block) items from work[0] (forward) / work[1] (backward) over `order`.
@@ -376,13 +378,13 @@ void launch_raster_fwd(const Batch &b, const DevOpts &o, int batch_depth, const 
                        const uint32_t *keys, const uint32_t *pv_list, const float4 *rec,
                        float *out_rgb,
                        float *T_final, uint32_t *n_contrib, unsigned long long *stats,
-                       cudaStream_t s, const uint4 *order = nullptr, uint32_t *work = nullptr,
-                       const StoreBuf &sto = StoreBuf());
+                       cudaStream_t s, bool two, const uint4 *order = nullptr,
+                       uint32_t *work = nullptr, const StoreBuf &sto = StoreBuf());
 void launch_raster_bwd(const Batch &b, const DevOpts &o, int batch_depth, const uint2 *ranges,
                        const uint32_t *keys, const uint32_t *pv_list, const float4 *rec,
                        const float *T_final,
                        const uint32_t *n_contrib, const float *grad_rgb, float4 *g2d,
-                       unsigned long long *stats, cudaStream_t s,
+                       unsigned long long *stats, cudaStream_t s, bool two,
                        const uint4 *order = nullptr, uint32_t *work = nullptr,
                        const StoreBuf &sto = StoreBuf());
 // Longest-first tile order for the persistent raster, as tile descriptors

@@ -87,3 +87,37 @@ def test_a_bad_colour_stays_in_its_pixels(env, sched, bad):
     touched = ~np.isfinite(out[1]).all(1)
     assert 0 < touched.sum() < 300
     assert np.array_equal(out[0][~touched], out[1][~touched])
+
+
+@pytest.mark.parametrize("sched", [dict(), dict(persistent=1), dict(bwd_mode=1, tile=(8, 8)),
+                                   dict(bwd_mode=1, persistent=1, tile=(16, 32)),
+                                   dict(max_per_pixel=7), dict(store_depth=5)],
+                         ids=["streamed", "persistent", "8x8", "persistent-16x32", "capped",
+                              "depth-5"])
+def test_half_blocks_and_blocks_agree(env, sched):
+    """A small view alone (a warp per half of an 8 x 8 block) and 900 copies of
+    it in one batch (a warp per block): the same image bit for bit, and the
+    batch's gradients are 900 times the view's (fp32 sums of 900 equal terms:
+    relative error below 900 * 2^-24)."""
+    import torch
+    pbr, R = env
+    rng = np.random.default_rng(8)
+    n, copies = 700, 900
+    pos = rng.uniform(-0.8, 0.8, (n, 3)).astype(np.float32)
+    scene = pbr.Scene(pos, scenes.sh_coeffs(rng, n, 1, std=0.2),
+                      rng.choice(np.float32([0.1, 0.5, 0.99, 1.5]), n),
+                      rng.uniform(0.03, 0.2, n).astype(np.float32), 1)
+    cam = scenes.camera((0.3, 0.2, 2.4), 61, 44)
+    g = torch.from_numpy(rng.normal(size=(61 * 44, 3)).astype(np.float32)).cuda()
+    opts = pbr.default_opts(**sched)
+    img, st = R.forward([scene], [cam], opts)
+    one = R.backward(st, g)
+    last = st.read("n_contrib")
+    st.close()
+    imgs, st = R.forward([scene], [cam] * copies, opts)
+    many = R.backward(st, g.repeat(copies, 1))
+    assert np.array_equal(st.read("n_contrib").reshape(copies, -1), np.tile(last, (copies, 1)))
+    st.close()
+    assert torch.equal(imgs.view(copies, -1, 3), img.view(1, -1, 3).expand(copies, -1, 3))
+    for a, b in zip(many, one):
+        assert _rel(a.cpu().numpy(), copies * b.cpu().numpy().astype(np.float64)) <= 900 * 2.0 ** -24
