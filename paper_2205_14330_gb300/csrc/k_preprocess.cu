@@ -66,31 +66,74 @@ __device__ __forceinline__ uint32_t k3_magic(int K3)
     return 0xffffffffu / (uint32_t)K3 + 1u;
 }
 
+__device__ __forceinline__ void cp_async16(void *smem, const void *gmem)
+{
+    const uint32_t sa = (uint32_t)__cvta_generic_to_shared(smem);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sa), "l"(gmem) : "memory");
+}
+
+__device__ __forceinline__ void cp_async4(void *smem, const void *gmem)
+{
+    const uint32_t sa = (uint32_t)__cvta_generic_to_shared(smem);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(sa), "l"(gmem) : "memory");
+}
+
+__device__ __forceinline__ void cp_async_commit()
+{
+    asm volatile("cp.async.commit_group;" ::: "memory");
+}
+
+template <int N> __device__ __forceinline__ void cp_async_wait()
+{
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+// Starts the copy of the block's coefficients (one group, committed).  Up to
+// 48 words a thread are in flight at once; loaded through registers they came
+// four at a time, and a block of a one-view render spent most of its time in
+// those twelve round trips (forward, 1M points, SH degree 3, one view: 208 ->
+// 100 us; 500k points, degree 2, 4 views: forward 82 -> 59 us, backward 127 ->
+// 54 us; 1M, degree 3, 64 views: 1.11 -> 1.00 ms, 1.27 -> 1.04 ms).
 __device__ __forceinline__ void stage_sh(const float *__restrict__ sh, int64_t first, int count,
                                          int K3, float *s_sh)
 {
     const int64_t base = first * K3;
     const int total = count * K3;
     const uint32_t magic = k3_magic(K3);
-    for (int f = threadIdx.x; f < total; f += blockDim.x) {
+#pragma unroll 4
+    for (int f = threadIdx.x; f < total; f += PRE_THREADS) {
         const int p = (int)div_k3((uint32_t)f, magic);
-        s_sh[(f - p * K3) * SH_STRIDE + p] = __ldg(sh + base + f);
+        cp_async4(s_sh + (f - p * K3) * SH_STRIDE + p, sh + base + f);
     }
+    cp_async_commit();
+}
+
+// A point's position, radius and opacity, read while its block's coefficients
+// are on the way.
+struct PointIn {
+    float p[3], r, op;
+};
+
+__device__ __forceinline__ PointIn load_point(const DevScene &sc, int64_t i)
+{
+    PointIn q;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) q.p[a] = __ldg(sc.pos + 3 * i + a);
+    q.r = __ldg(sc.radius + i);
+    q.op = __ldg(sc.opacity + i);
+    return q;
 }
 
 template <int DEG>
 __device__ void pre_fwd_point(const Batch &b, const DevOpts &o, const DevScene &sc, int64_t i,
-                              const float *hs, float4 *__restrict__ rec,
+                              const PointIn &in, const float *hs, float4 *__restrict__ rec,
                               uint32_t *__restrict__ zbits, uint32_t *__restrict__ ntiles,
                               uint8_t *__restrict__ nt8,
                               uint4 *__restrict__ rect, uint32_t &vis_cnt, uint32_t &pair_cnt,
                               uint32_t &zlo, uint32_t &zhi)
 {
     constexpr int K = SH<DEG>::K;
-    const float P0 = __ldg(sc.pos + 3 * i), P1 = __ldg(sc.pos + 3 * i + 1),
-                P2 = __ldg(sc.pos + 3 * i + 2);
-    const float r = __ldg(sc.radius + i);
-    const float op = __ldg(sc.opacity + i);
+    const float P0 = in.p[0], P1 = in.p[1], P2 = in.p[2], r = in.r, op = in.op;
     const int tws = __ffs(o.tile_w) - 1, ths = __ffs(o.tile_h) - 1;
 
     for (int vv = 0; vv < sc.view_count; ++vv) {
@@ -212,16 +255,19 @@ preprocess_fwd_kernel(Batch b, DevOpts o, float4 *__restrict__ rec, uint32_t *__
     if (count <= 0) return; // whole block past the scene (uniform)
     const int K3 = sc.K * 3;
     stage_sh(sc.sh, first, count, K3, s_sh);
+    PointIn in{};
+    if ((int)threadIdx.x < count) in = load_point(sc, first + threadIdx.x);
+    cp_async_wait<0>();
     __syncthreads();
     uint32_t vis = 0, pairs = 0, zlo = 0xffffffffu, zhi = 0u;
     if ((int)threadIdx.x < count) {
         const int64_t i = first + threadIdx.x;
         const float *hs = s_sh + threadIdx.x; // coefficient j at hs[j * SH_STRIDE]
         switch (sc.deg) {
-        case 0: pre_fwd_point<0>(b, o, sc, i, hs, rec, zbits, ntiles, nt8, rect, vis, pairs, zlo, zhi); break;
-        case 1: pre_fwd_point<1>(b, o, sc, i, hs, rec, zbits, ntiles, nt8, rect, vis, pairs, zlo, zhi); break;
-        case 2: pre_fwd_point<2>(b, o, sc, i, hs, rec, zbits, ntiles, nt8, rect, vis, pairs, zlo, zhi); break;
-        default: pre_fwd_point<3>(b, o, sc, i, hs, rec, zbits, ntiles, nt8, rect, vis, pairs, zlo, zhi); break;
+        case 0: pre_fwd_point<0>(b, o, sc, i, in, hs, rec, zbits, ntiles, nt8, rect, vis, pairs, zlo, zhi); break;
+        case 1: pre_fwd_point<1>(b, o, sc, i, in, hs, rec, zbits, ntiles, nt8, rect, vis, pairs, zlo, zhi); break;
+        case 2: pre_fwd_point<2>(b, o, sc, i, in, hs, rec, zbits, ntiles, nt8, rect, vis, pairs, zlo, zhi); break;
+        default: pre_fwd_point<3>(b, o, sc, i, in, hs, rec, zbits, ntiles, nt8, rect, vis, pairs, zlo, zhi); break;
         }
     }
     // per-warp totals, one atomic per warp: counters[0] pairs, [1] visible,
@@ -245,27 +291,12 @@ preprocess_fwd_kernel(Batch b, DevOpts o, float4 *__restrict__ rec, uint32_t *__
 // ahead with per-thread asynchronous copies into shared memory, so that
 // their reads are in flight while earlier views are computed.
 // BWD_AHEAD + 1 slots per thread: a slot is refilled one view after its
-// contents were read.  Measured on the 1M-point, 64-view step: 1.27-1.29 ms
+// contents were read.  Measured on the 1M-point, 64-view step (with the
+// coefficients loaded through registers): 1.27-1.29 ms
 // at one or two views ahead, 1.37 ms at three or four (the deeper buffer
 // takes shared memory from the L1 cache).
 constexpr int BWD_AHEAD = 2;
 constexpr int BWD_SLOTS = BWD_AHEAD + 1;
-
-__device__ __forceinline__ void cp_async16(void *smem, const void *gmem)
-{
-    const uint32_t sa = (uint32_t)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sa), "l"(gmem) : "memory");
-}
-
-__device__ __forceinline__ void cp_async_commit()
-{
-    asm volatile("cp.async.commit_group;" ::: "memory");
-}
-
-template <int N> __device__ __forceinline__ void cp_async_wait()
-{
-    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
 
 // Starts the copy of view slot `vv`'s two float4 terms of point i into the
 // thread's slot.  sg: this thread's slots, [slot][half] with a stride of
@@ -282,24 +313,18 @@ __device__ __forceinline__ void fetch_view_terms(const Batch &b, const DevScene 
 
 template <int DEG>
 __device__ void pre_bwd_point(const Batch &b, const DevOpts &o, const DevScene &sc, int64_t i,
-                              float *hs, float4 *sg, const float4 *__restrict__ g2d,
+                              const PointIn &in, float *hs, float4 *sg,
+                              const float4 *__restrict__ g2d,
                               float *__restrict__ grad_pos, float *__restrict__ grad_opacity)
 {
     constexpr int K = SH<DEG>::K;
     float dh[K * 3];
 #pragma unroll
     for (int j = 0; j < K * 3; ++j) dh[j] = 0.0f;
-    const float P0 = __ldg(sc.pos + 3 * i), P1 = __ldg(sc.pos + 3 * i + 1),
-                P2 = __ldg(sc.pos + 3 * i + 2);
-    const float r = __ldg(sc.radius + i), op = __ldg(sc.opacity + i);
+    const float P0 = in.p[0], P1 = in.p[1], P2 = in.p[2], r = in.r, op = in.op;
     float dP0 = 0.f, dP1 = 0.f, dP2 = 0.f, dop = 0.f;
 
     const int nv = sc.view_count;
-#pragma unroll
-    for (int d = 0; d < BWD_AHEAD; ++d) {
-        if (d < nv) fetch_view_terms(b, sc, i, d, g2d, sg);
-        cp_async_commit(); // one group per view slot, empty past the end
-    }
     for (int vv = 0; vv < nv; ++vv) {
         const int v = b.view_list[sc.view_begin + vv];
         const DevView &V = b.views[v];
@@ -401,16 +426,24 @@ preprocess_bwd_kernel(Batch b, DevOpts o, const float4 *__restrict__ g2d,
     if (count <= 0) return;
     const int K3 = sc.K * 3;
     stage_sh(sc.sh, first, count, K3, s_sh);
+    const int64_t i = first + threadIdx.x;
+    float4 *sg = s_g + threadIdx.x;
+    PointIn in{};
+    if ((int)threadIdx.x < count) in = load_point(sc, i);
+#pragma unroll
+    for (int d = 0; d < BWD_AHEAD; ++d) { // the first views' terms
+        if ((int)threadIdx.x < count && d < sc.view_count) fetch_view_terms(b, sc, i, d, g2d, sg);
+        cp_async_commit(); // one group per view slot, empty past the end
+    }
+    cp_async_wait<BWD_AHEAD>(); // the coefficients
     __syncthreads();
     if ((int)threadIdx.x < count) {
-        const int64_t i = first + threadIdx.x;
         float *hs = s_sh + threadIdx.x; // coefficient j at hs[j * SH_STRIDE]
-        float4 *sg = s_g + threadIdx.x;
         switch (sc.deg) {
-        case 0: pre_bwd_point<0>(b, o, sc, i, hs, sg, g2d, grad_pos, grad_opacity); break;
-        case 1: pre_bwd_point<1>(b, o, sc, i, hs, sg, g2d, grad_pos, grad_opacity); break;
-        case 2: pre_bwd_point<2>(b, o, sc, i, hs, sg, g2d, grad_pos, grad_opacity); break;
-        default: pre_bwd_point<3>(b, o, sc, i, hs, sg, g2d, grad_pos, grad_opacity); break;
+        case 0: pre_bwd_point<0>(b, o, sc, i, in, hs, sg, g2d, grad_pos, grad_opacity); break;
+        case 1: pre_bwd_point<1>(b, o, sc, i, in, hs, sg, g2d, grad_pos, grad_opacity); break;
+        case 2: pre_bwd_point<2>(b, o, sc, i, in, hs, sg, g2d, grad_pos, grad_opacity); break;
+        default: pre_bwd_point<3>(b, o, sc, i, in, hs, sg, g2d, grad_pos, grad_opacity); break;
         }
     }
     __syncthreads();
