@@ -308,19 +308,25 @@ int pbr::build_layout(const pbr_points *scenes, int32_t n_scenes, const int32_t 
 // the longest block's walk is a large share of the whole: with v the hits a
 // view's block visits (its list, or what saturates it: some 28 layers of
 // splats covering c of its 64 pixels), the batch is worth sum(v) / max(v)
-// equal blocks, and the line lies at 130000 / r of them forward and 45000 / r
-// backward, r the mean cutoff radius in pixels.  r comes from the pair count:
-// a point lists (1 + 2 r / tile_w)(1 + 2 r / tile_h) tiles, r = k f with f the
-// view's focal length in pixels, summed over the views and solved for k.
-// Measured, one pixel a lane / two (us; 16 x 16 tiles, streamed): 120k points,
-// 2 views of 500 x 400 (6.3k blocks, r 2.3): forward 47 / 52, backward 97 /
-// 107; 120k, 4 views of 800^2 (40k, 3.7): 91 / 89, 232 / 183; 45k large
-// points, 1024 x 768 (12.3k, 16): 34 / 33, 93 / 68; 125k, five views of
-// 104 x 141 to 647 x 549 (worth 2k): 217 / 311, 298 / 450; 808k, eight views
-// of 235 x 230 to 1737 x 835, persistent (worth 10k, 6.3): 398 / 534, 1038 /
-// 802.
+// equal blocks, and the line lies at c / r of them, r the mean cutoff radius
+// in pixels: forward c = 105000 streamed, 160000 with the stored list and
+// 250000 persistent, backward 60000; lower in proportion where a block's mean
+// walk is below 64 hits, since a warp's start then counts.  r comes from the
+// pair count: a point lists (1 + 2 r / tile_w)(1 + 2 r / tile_h) tiles, r = k
+// f with f the view's focal length in pixels, summed over the views and
+// solved for k.
+// Measured, half blocks / blocks (us, fwd and bwd; with worth times r, in
+// thousands): streamed, 16 x 16 tiles: 227k points, 7 views of 101 x 339 to
+// 1270 x 365 (16): 635 / 1039, 803 / 1259; 7k, 4 small views (71): 36 / 44,
+// 44 / 63; 16 views of 256^2 to 1920 x 1072 over four scenes (107): 876 / 769;
+// 500k, 4 views of 800^2 (149): 189 / 186, 429 / 364, stored 272 / 298, 565 /
+// 516; 272k, 33 views (179): 596 / 518, 958 / 714; one 1920 x 1080 view of 1M
+// (290): 167 / 151; one 1024 x 768 view of 45k, 18 hits a block (59): 37 / 22.
+// Persistent: 808k, 8 views of 235 x 230 to 1737 x 835 (64): 398 / 534, 1038 /
+// 802; 136k, 8 views (82): 172 / 262, 323 / 423; 136k, 43 views (216): 619 /
+// 680, 1448 / 1148.
 RasterLanes pbr::raster_lanes(const HostLayout &L, const DevOpts &o, int64_t n_vis,
-                              int64_t n_pairs)
+                              int64_t n_pairs, bool persistent, bool store)
 {
     RasterLanes r;
     if (L.n_pv <= 0 || n_vis <= 0) return r;
@@ -336,7 +342,7 @@ RasterLanes pbr::raster_lanes(const HostLayout &L, const DevOpts &o, int64_t n_v
         c += n;
     }
     const double k = c < 0.0 && a > 0.0 ? (-b + std::sqrt(b * b - 4.0 * a * c)) / (2.0 * a) : 0.0;
-    double most = 0.0, sum = 0.0, sum_r = 0.0;
+    double most = 0.0, sum = 0.0, sum_r = 0.0, sum_blocks = 0.0;
     for (const DevView &V : L.views) {
         const double blocks = (double)((V.W + 7) / 8) * ((V.H + 7) / 8);
         const double rc = std::max(k * focal(V), 0.5), w = 8.0 + 2.0 * rc;
@@ -344,13 +350,15 @@ RasterLanes pbr::raster_lanes(const HostLayout &L, const DevOpts &o, int64_t n_v
         const double v = std::min(share * (double)L.scenes[V.scene].n * (w * w / 64.0) / blocks,
                                   28.0 * 64.0 / cover);
         most = std::max(most, v);
+        sum_blocks += blocks;
         sum += blocks * v;
         sum_r += blocks * v * rc;
     }
     if (!(most > 0.0)) return r;
     const double worth = sum / most, mean_r = sum_r / sum;
-    r.fwd_two = worth * mean_r >= 130000.0;
-    r.bwd_two = worth * mean_r >= 45000.0;
+    const double line = std::min(1.0, sum / sum_blocks / 64.0);
+    r.fwd_two = worth * mean_r >= (persistent ? 250e3 : store ? 160e3 : 105e3) * line;
+    r.bwd_two = worth * mean_r >= 60e3 * line;
     return r;
 }
 
@@ -549,7 +557,8 @@ int pbr::forward_eager(pbr_ctx *c, pbr_state *st, float *out_rgb, cudaStream_t s
                           st->rec, out_rgb,
                           st->T_final, st->n_contrib,
                           st->opts.no_pair_stats ? nullptr : st->counters + 2, s,
-                          raster_lanes(L, o, st->n_vis, st->n_pairs).fwd_two, st->tile_order,
+                          raster_lanes(L, o, st->n_vis, st->n_pairs, persist, st->store_depth > 0).fwd_two,
+                          st->tile_order,
                           st->work, st->store());
     }
     PBR_CUDA(cudaGetLastError());
@@ -697,7 +706,9 @@ extern "C" int pbr_render_backward(pbr_ctx *c, pbr_state *st, const float *grad_
                           st->tile_vals, st->rec,
                           st->T_final, st->n_contrib, grad_rgb, g2d,
                           st->opts.no_pair_stats ? nullptr : st->counters + 2, s,
-                          raster_lanes(L, st->dopts, st->n_vis, st->n_pairs).bwd_two,
+                          raster_lanes(L, st->dopts, st->n_vis, st->n_pairs, st->work != nullptr,
+                                       st->store_depth > 0)
+                              .bwd_two,
                           st->tile_order, st->work, st->store());
     }
     {

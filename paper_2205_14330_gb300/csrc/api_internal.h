@@ -65,7 +65,8 @@ void zero_unviewed_grads(const HostLayout &L, float *grad_pos, float *grad_sh,
 struct RasterLanes {
     bool fwd_two = true, bwd_two = true;
 };
-RasterLanes raster_lanes(const HostLayout &L, const DevOpts &o, int64_t n_vis, int64_t n_pairs);
+RasterLanes raster_lanes(const HostLayout &L, const DevOpts &o, int64_t n_vis, int64_t n_pairs,
+                         bool persistent, bool store);
 int dalloc(void **p, size_t bytes, cudaStream_t s);
 void dfree(void *p, cudaStream_t s);
 void serve_shutdown(pbr_ctx *c);
