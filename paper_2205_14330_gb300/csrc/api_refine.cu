@@ -93,12 +93,11 @@ int pbr::make_params(TempBufs &tb, const float *pos, int64_t n, int cells, Searc
     S.fine.cells = cells;
     S.has_coarse = cells >= 16 && n > 0;
     if (n <= 0) return PBR_OK;
-    launch_grid_params(pos, n, cells, S.fine.gp, gtmp, s);
     if (S.has_coarse) {
         PBR_TRY(tb.alloc(&S.coarse.gp, sizeof(GridParams)));
         S.coarse.cells = (cells + 7) / 8;
-        launch_grid_params(pos, n, S.coarse.cells, S.coarse.gp, gtmp, s);
     }
+    launch_grid_params(pos, n, cells, S.fine.gp, S.coarse.cells, S.coarse.gp, gtmp, s);
     return PBR_OK;
 }
 

@@ -263,8 +263,10 @@ struct PointArraysOut {
     int nsh;
 };
 size_t grid_temp_bytes();
-void launch_grid_params(const float *pos, int64_t n, int n_cells, GridParams *gp, void *temp,
-                        cudaStream_t s);
+// Parameters of a grid of n_cells cells an axis over the cube of n points, and
+// (coarse not NULL) of one of n_coarse cells.
+void launch_grid_params(const float *pos, int64_t n, int n_cells, GridParams *gp, int n_coarse,
+                        GridParams *coarse, void *temp, cudaStream_t s);
 // keys = clamped cell ids, vals = 0..n-1
 void launch_cell_ids(const float *pos, int64_t n, const GridParams *gp, uint32_t *keys,
                      uint32_t *vals, cudaStream_t s);
