@@ -18,9 +18,9 @@
 //   5. tile_ranges      : [start, end) of every tile in the sorted list
 //
 // Scans are reduce-then-scan (three kernels, no inter-block waiting).  A
-// radix pass ranks keys stably inside a block with per-warp peer masks
-// (shared-memory OR) and shared atomics, and reorders them in shared memory
-// so that the scatter writes contiguous runs.  Short sorts run in one sweep
+// radix pass ranks keys stably inside a block with ballots and a counter per
+// warp and digit, and reorders them in shared memory so that the scatter writes
+// contiguous runs.  Short sorts run in one sweep
 // (one histogram of every digit, then a kernel per pass with look-back), long
 // ones with a histogram, a scan and a scatter per pass.
 #include <algorithm>
@@ -225,24 +225,6 @@ __device__ __forceinline__ uint32_t digit_of(uint32_t key, uint32_t key_lo, uint
     return ((k < key_max ? k : key_max) >> shift) & mask;
 }
 
-// Peers of each lane: lanes holding the same digit (digits < 2^10, the
-// out-of-range marker RBINS included), built from ballots.  full: no lane
-// holds the marker (warp-uniform), so its bit needs no ballot.
-__device__ __forceinline__ uint32_t peers_by_ballot(uint32_t d, bool full)
-{
-    uint32_t peers = 0xffffffffu;
-#pragma unroll
-    for (int bit = 0; bit < RB; ++bit) {
-        const uint32_t m = __ballot_sync(0xffffffffu, (d >> bit) & 1u);
-        peers &= ((d >> bit) & 1u) ? m : ~m;
-    }
-    if (!full) {
-        const uint32_t m = __ballot_sync(0xffffffffu, (d >> RB) & 1u);
-        peers &= ((d >> RB) & 1u) ? m : ~m;
-    }
-    return peers;
-}
-
 // Digit histograms of HIST_TILES consecutive scatter tiles (SORT_TILE keys
 // each) per block: shared-memory atomics into one counter per (tile,
 // digit), written out as hist[digit][tile].
@@ -280,157 +262,241 @@ radix_hist_kernel(const uint32_t *__restrict__ keys, const uint32_t *n_dev, int6
             hist[(int64_t)dd * nb + t0 + k] = s_h[k][dd];
 }
 
-constexpr size_t SCATTER_SMEM = sizeof(uint32_t) * (3 * SORT_TILE + SORT_WARPS * RBINS + 3 * RBINS +
-                                                    SORT_WARPS);
+// A warp's share of a tile: rows of 32 keys, row r's lane l holding key 32 r + l
+// of the share, cnt of them in range.
+template <int ITEMS>
+__device__ __forceinline__ int share_count(int64_t base, int64_t n)
+{
+    return (int)(n - base < 0 ? 0 : n - base < 32 * ITEMS ? n - base : 32 * ITEMS);
+}
 
-__global__ void __launch_bounds__(SORT_THREADS)
+// Stable rank of each of the warp's keys among the warp's keys of its digit,
+// with the digit above it (bits 16 and up); wh: the warp's digit counters
+// (zeros, counts afterwards).
+// Peers found by OR-ing lane bits into shared words, counted with shared
+// atomics, cost 39 shared-memory wavefronts per 32 keys and passed them one row
+// after another; with ballots, a plain read and write of the counter, values
+// that stay in registers and one bank of slots for keys and values it is 23,
+// and the shared memory of a block falls from 72 to 20 KB.  The five passes of
+// 64 views of 1M points: 2980 -> 2311 us, of 16 views of 1M 205 -> 178
+// (__match_any_sync for the ballots: about 20% slower; 64 registers for four
+// blocks a SM instead of three: 2434, by its spills).  Now bound by issue (the
+// ballots) and by the scattered writes' sectors.
+template <int ITEMS>
+__device__ __forceinline__ void rank_in_warp(const uint32_t (&key)[ITEMS], uint32_t (&rank)[ITEMS],
+                                             int cnt, int shift, int width, uint32_t *wh)
+{
+    const int lane = threadIdx.x & 31;
+    const uint32_t lt = lanemask_lt(), mask = (1u << width) - 1u;
+    // the lanes holding each lane's digit, from a ballot a bit: all rows' at
+    // once, so that none waits for another
+#pragma unroll
+    for (int r = 0; r < ITEMS; ++r) rank[r] = __ballot_sync(0xffffffffu, r * 32 + lane < cnt);
+    for (int b = 0; b < width; ++b) {
+        const uint32_t bit = 1u << (shift + b);
+#pragma unroll
+        for (int r = 0; r < ITEMS; ++r) {
+            const bool set = key[r] & bit;
+            const uint32_t m = __ballot_sync(0xffffffffu, set);
+            rank[r] &= m ^ ((uint32_t)set - 1u); // m, or its complement where the bit is clear
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < ITEMS; ++r) {
+        const uint32_t d = (key[r] >> shift) & mask;
+        const uint32_t peers = rank[r], before = (uint32_t)__popc(peers & lt);
+        const uint32_t old = wh[d];
+        __syncwarp(); // every lane has read the counter
+        if (before == 0 && r * 32 + lane < cnt) wh[d] = old + (uint32_t)__popc(peers);
+        __syncwarp(); // and the next round reads what its group's first lane wrote
+        rank[r] = (old + before) | d << 16;
+    }
+}
+
+// Turns the warps' digit counts (s_wh[warp][digit]) into each warp's first
+// slot of the digit in the tile's digit order.  tot, first: the tile's count
+// and first slot of digits 2 threadIdx.x and 2 threadIdx.x + 1.  publish(tot)
+// is called as soon as the counts are known.
+template <class Publish>
+__device__ __forceinline__ void digit_slots(uint32_t *s_wh, uint32_t *s_scan, uint32_t (&tot)[2],
+                                            uint32_t (&first)[2], Publish publish)
+{
+    static_assert(RBINS == 2 * SORT_THREADS, "two digits a thread");
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    uint2 x[SORT_WARPS];
+    tot[0] = tot[1] = 0;
+#pragma unroll
+    for (int j = 0; j < SORT_WARPS; ++j) {
+        x[j] = reinterpret_cast<uint2 *>(s_wh + j * RBINS)[threadIdx.x];
+        tot[0] += x[j].x;
+        tot[1] += x[j].y;
+    }
+    publish(tot);
+    const uint32_t sum = tot[0] + tot[1], inc = warp_incl_scan(sum);
+    if (lane == 31) s_scan[w] = inc;
+    __syncthreads();
+    first[0] = inc - sum;
+#pragma unroll
+    for (int j = 0; j < SORT_WARPS; ++j) first[0] += j < w ? s_scan[j] : 0u;
+    first[1] = first[0] + tot[0];
+    uint2 at{first[0], first[1]};
+#pragma unroll
+    for (int j = 0; j < SORT_WARPS; ++j) {
+        reinterpret_cast<uint2 *>(s_wh + j * RBINS)[threadIdx.x] = at;
+        at.x += x[j].x;
+        at.y += x[j].y;
+    }
+}
+
+// Shared memory of a pass over tiles of ITEMS keys a thread: the warps' digit
+// counters, then (in the same place) the tile's keys and after them its values
+// in digit order.
+template <int ITEMS>
+struct PassSmem {
+    static constexpr int TILE = SORT_THREADS * ITEMS, WH = SORT_WARPS * RBINS;
+    uint32_t wh_or_tile[TILE > WH ? TILE : WH];
+    uint32_t gbase[RBINS]; // output position of slot j of digit d: gbase[d] + j
+    uint32_t tot[RBINS];
+    uint32_t scan[SORT_WARPS];
+    uint32_t tile;
+};
+
+// Slots of a thread's keys in the tile's digit order, two to a register.
+template <int ITEMS>
+struct Slots {
+    uint32_t two[ITEMS / 2];
+    __device__ __forceinline__ uint32_t at(int r) const
+    {
+        return r & 1 ? two[r / 2] >> 16 : two[r / 2] & 0xffffu;
+    }
+};
+
+template <int ITEMS>
+__device__ __forceinline__ Slots<ITEMS> slots_of(const uint32_t (&rank)[ITEMS], const uint32_t *wh)
+{
+    static_assert(SORT_THREADS * ITEMS <= 1 << 16 && ITEMS % 2 == 0, "two slots a register");
+    Slots<ITEMS> s;
+#pragma unroll
+    for (int r = 0; r < ITEMS; r += 2)
+        s.two[r / 2] = ((rank[r] & 0xffffu) + wh[rank[r] >> 16]) |
+                       ((rank[r + 1] & 0xffffu) + wh[rank[r + 1] >> 16]) << 16;
+    return s;
+}
+
+// Places x in the tile's digit order.
+template <int ITEMS>
+__device__ __forceinline__ void place(const uint32_t (&x)[ITEMS], const Slots<ITEMS> &slot, int cnt,
+                                      uint32_t *s_t)
+{
+#pragma unroll
+    for (int r = 0; r < ITEMS; ++r)
+        if (r * 32 + (int)(threadIdx.x & 31) < cnt) s_t[slot.at(r)] = x[r];
+}
+
+// The share's words (0 where there are none): p is the share's first.
+template <int ITEMS>
+__device__ __forceinline__ void load_share(uint32_t (&x)[ITEMS], const uint32_t *__restrict__ p,
+                                           int cnt)
+{
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int r = 0; r < ITEMS; ++r) x[r] = r * 32 + lane < cnt ? p[r * 32 + lane] : 0u;
+}
+
+template <int ITEMS>
+__device__ __forceinline__ void load_vals(uint32_t (&v)[ITEMS], const uint32_t *__restrict__ vals,
+                                          int64_t base, int cnt, bool index_vals)
+{
+    if (index_vals) {
+#pragma unroll
+        for (int r = 0; r < ITEMS; ++r) v[r] = (uint32_t)base + r * 32 + (threadIdx.x & 31);
+    } else {
+        load_share(v, vals + base, cnt);
+    }
+}
+
+// Writes the placed keys, then the values: S.gbase is known and a barrier has
+// passed since the keys were placed.
+template <int ITEMS>
+__device__ __forceinline__ void write_tile(PassSmem<ITEMS> &S, const uint32_t (&val)[ITEMS],
+                                           const Slots<ITEMS> &slot, int cnt, int tile_cnt,
+                                           int shift, int width, uint32_t *__restrict__ keys_out,
+                                           uint32_t *__restrict__ vals_out)
+{
+    const uint32_t mask = (1u << width) - 1u;
+    uint32_t g[ITEMS];
+#pragma unroll
+    for (int q = 0; q < ITEMS; ++q) {
+        const int j = threadIdx.x + q * SORT_THREADS;
+        if (j < tile_cnt) {
+            const uint32_t k = S.wh_or_tile[j];
+            g[q] = S.gbase[(k >> shift) & mask] + (uint32_t)j;
+            keys_out[g[q]] = k;
+        }
+    }
+    __syncthreads();
+    place(val, slot, cnt, S.wh_or_tile);
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < ITEMS; ++q) {
+        const int j = threadIdx.x + q * SORT_THREADS;
+        if (j < tile_cnt) vals_out[g[q]] = S.wh_or_tile[j];
+    }
+}
+
+// key -> min(key - key_lo, key_max): keys above the range (the marker of an
+// invisible point-view) all take the largest value.  The passes sort, and
+// write, the reduced keys.
+template <int ITEMS>
+__device__ __forceinline__ void reduce_keys(uint32_t (&key)[ITEMS], uint32_t key_lo, uint32_t key_max)
+{
+#pragma unroll
+    for (int r = 0; r < ITEMS; ++r) key[r] = min(key[r] - key_lo, key_max);
+}
+
+__global__ void __launch_bounds__(SORT_THREADS, 3)
 radix_scatter_kernel(const uint32_t *__restrict__ keys_in, const uint32_t *__restrict__ vals_in,
                      uint32_t *__restrict__ keys_out, uint32_t *__restrict__ vals_out,
                      const uint32_t *n_dev, int64_t cap, uint32_t key_lo, uint32_t key_max,
                      int shift, int width, const uint32_t *__restrict__ hist, int64_t nb,
                      bool index_vals)
 {
-    extern __shared__ uint32_t s_mem[];
-    uint32_t *s_k = s_mem;                               // [SORT_TILE] keys, ranked order
-    uint32_t *s_v = s_k + SORT_TILE;                     // [SORT_TILE] values, ranked order
-    uint32_t *s_vin = s_v + SORT_TILE;                   // [SORT_TILE] values, input order
-    uint32_t(*s_wh)[RBINS] = (uint32_t(*)[RBINS])(s_vin + SORT_TILE); // [warps][RBINS]
-    uint32_t *s_tot = s_vin + SORT_TILE + SORT_WARPS * RBINS;
-    uint32_t *s_dbase = s_tot + RBINS;
-    uint32_t *s_gbase = s_dbase + RBINS;
-    uint32_t *s_scan = s_gbase + RBINS;
+    __shared__ __align__(16) PassSmem<SORT_ITEMS> S;
     const int64_t n = dev_count(n_dev, cap);
     const int64_t blk = (int64_t)blockIdx.x * SORT_TILE;
     if (blk >= n) return;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const uint32_t mask = (1u << width) - 1u;
     const int bins = 1 << width;
-    // the block's global digit bases, loaded now so that their latency
-    // hides behind the ranking (digits threadIdx.x + k SORT_THREADS)
-    constexpr int PER_T = RBINS / SORT_THREADS;
-    uint32_t gb[PER_T];
+    const int64_t base = blk + (int64_t)w * 32 * SORT_ITEMS;
+    const int cnt = share_count<SORT_ITEMS>(base, n);
+    uint32_t key[SORT_ITEMS], rank[SORT_ITEMS], val[SORT_ITEMS];
+    load_share(key, keys_in + base, cnt);
+    // the block's first output position of its digits, loaded now so that the
+    // latency hides behind the ranking
+    uint32_t gb[2];
 #pragma unroll
-    for (int k = 0; k < PER_T; ++k) {
-        const int dd = threadIdx.x + k * SORT_THREADS;
+    for (int k = 0; k < 2; ++k) {
+        const int dd = 2 * threadIdx.x + k;
         gb[k] = dd < bins ? hist[(int64_t)dd * nb + blockIdx.x] : 0u;
     }
-    for (int j = threadIdx.x; j < SORT_WARPS * RBINS; j += SORT_THREADS) (&s_wh[0][0])[j] = 0;
-    // the warps' peer masks (one word per digit) live in s_k, free until the
-    // placement below
-    uint32_t *s_pm = s_k + w * RBINS;
-    for (int j = threadIdx.x; j < SORT_TILE; j += SORT_THREADS) s_k[j] = 0;
-    const int64_t base = blk + (int64_t)w * 32 * SORT_ITEMS;
-    uint32_t key[SORT_ITEMS], rank[SORT_ITEMS];
-    const int lbase = w * 32 * SORT_ITEMS + lane; // local index of round 0
-#pragma unroll
-    for (int r = 0; r < SORT_ITEMS; ++r) {
-        const int64_t i = base + r * 32 + lane;
-        const bool ok = i < n;
-        key[r] = ok ? keys_in[i] : 0u;
-        s_vin[lbase + r * 32] = ok ? (index_vals ? (uint32_t)i : vals_in[i]) : 0u;
-    }
+    uint32_t *wh = S.wh_or_tile + w * RBINS; // the warp's own counters
+    for (int j = lane; j < RBINS; j += 32) wh[j] = 0;
+    __syncwarp();
+    reduce_keys(key, key_lo, key_max);
+    rank_in_warp(key, rank, cnt, shift, width, wh);
     __syncthreads();
-    const uint32_t lt = lanemask_lt();
-    const bool full = blk + SORT_TILE <= n; // every key of the block is in range
-    {
-        // stable rank inside the warp: the lanes holding the same digit (each
-        // lane ORs its bit into its digit's word of the warp's peer masks and
-        // reads the word back; with out-of-range keys, from ballots), the
-        // group leader's shared-memory atomic on the warp's digit counter
-        // (one warp's shared atomics execute in program order, so rounds stay
-        // ordered) and its reset of the peer word, then the broadcast of each
-        // group's base
-#pragma unroll
-        for (int r = 0; r < SORT_ITEMS; ++r) {
-            const bool ok = base + r * 32 + lane < n;
-            const uint32_t d = ok ? digit_of(key[r], key_lo, key_max, shift, mask) : (uint32_t)RBINS;
-            uint32_t peers;
-            if (full || __all_sync(0xffffffffu, ok)) {
-                atomicOr(&s_pm[d], 1u << lane);
-                __syncwarp();
-                peers = s_pm[d];
-                __syncwarp();
-            } else {
-                peers = peers_by_ballot(d, false);
-            }
-            uint32_t old = 0;
-            if (d < RBINS && (peers & lt) == 0) {
-                old = atomicAdd(&s_wh[w][d], (uint32_t)__popc(peers));
-                s_pm[d] = 0;
-            }
-            __syncwarp(); // peer words clear before the next round's ORs
-            rank[r] = (uint32_t)(__ffs(peers) - 1) | ((uint32_t)__popc(peers & lt) << 5) | (old << 10);
-        }
-#pragma unroll
-        for (int r = 0; r < SORT_ITEMS; ++r) {
-            const uint32_t packed = rank[r];
-            const uint32_t base_r = __shfl_sync(0xffffffffu, packed >> 10, packed & 31);
-            rank[r] = base_r + ((packed >> 5) & 31);
-        }
-    }
+    uint32_t tot[2], first[2];
+    digit_slots(S.wh_or_tile, S.scan, tot, first, [](const uint32_t (&)[2]) {});
+    S.gbase[2 * threadIdx.x] = gb[0] - first[0];
+    S.gbase[2 * threadIdx.x + 1] = gb[1] - first[1];
     __syncthreads();
-    // per digit: exclusive prefix over warps, digit total, global base
-#pragma unroll
-    for (int k = 0; k < PER_T; ++k) {
-        const int dd = threadIdx.x + k * SORT_THREADS;
-        uint32_t t = 0;
-        if (dd < bins) {
-#pragma unroll
-            for (int j = 0; j < SORT_WARPS; ++j) {
-                const uint32_t x = s_wh[j][dd];
-                s_wh[j][dd] = t;
-                t += x;
-            }
-            s_gbase[dd] = gb[k];
-        }
-        s_tot[dd] = t;
-    }
+    const auto slot = slots_of(rank, wh);
+    load_vals(val, vals_in, base, cnt, index_vals);
+    __syncthreads(); // the counters' place is the tile's from here
+    place(key, slot, cnt, S.wh_or_tile);
     __syncthreads();
-    // block exclusive scan of the digit totals (RBINS / SORT_THREADS per thread)
-    {
-        constexpr int PER = RBINS / SORT_THREADS;
-        uint32_t loc[PER], sum = 0;
-#pragma unroll
-        for (int q = 0; q < PER; ++q) {
-            loc[q] = s_tot[threadIdx.x * PER + q];
-            sum += loc[q];
-        }
-        const uint32_t inc = warp_incl_scan(sum);
-        if (lane == 31) s_scan[w] = inc;
-        __syncthreads();
-        uint32_t off = inc - sum;
-        for (int j = 0; j < w; ++j) off += s_scan[j];
-#pragma unroll
-        for (int q = 0; q < PER; ++q) {
-            s_dbase[threadIdx.x * PER + q] = off;
-            off += loc[q];
-        }
-    }
-    __syncthreads();
-    // output position of ranked slot j of digit d: s_gbase[d] + j - s_dbase[d]
-#pragma unroll
-    for (int k = 0; k < PER_T; ++k) {
-        const int dd = threadIdx.x + k * SORT_THREADS;
-        s_gbase[dd] -= s_dbase[dd];
-    }
-#pragma unroll
-    for (int r = 0; r < SORT_ITEMS; ++r) {
-        if (base + r * 32 + lane < n) {
-            const uint32_t d = digit_of(key[r], key_lo, key_max, shift, mask);
-            const uint32_t l = s_dbase[d] + s_wh[w][d] + rank[r];
-            s_k[l] = key[r];
-            s_v[l] = s_vin[lbase + r * 32];
-        }
-    }
-    __syncthreads();
-    const int cnt = (int)(n - blk < SORT_TILE ? n - blk : SORT_TILE);
-    for (int j = threadIdx.x; j < cnt; j += SORT_THREADS) {
-        const uint32_t k = s_k[j];
-        const uint32_t d = digit_of(k, key_lo, key_max, shift, mask);
-        const uint32_t g = s_gbase[d] + (uint32_t)j;
-        keys_out[g] = k;
-        vals_out[g] = s_v[j];
-    }
+    write_tile(S, val, slot, cnt, (int)(n - blk < SORT_TILE ? n - blk : SORT_TILE), shift, width, keys_out,
+               vals_out);
 }
 
 // ------------------------------------------------- one-sweep radix sort
@@ -574,161 +640,65 @@ __device__ uint32_t look_back(const uint32_t *state, uint32_t tile, uint32_t agg
 }
 
 template <int ITEMS>
-__host__ __device__ constexpr size_t sweep_smem()
-{
-    constexpr int TILE = SORT_THREADS * ITEMS;
-    constexpr int PM = SORT_WARPS * RBINS; // peer masks share the ranked keys' space
-    return sizeof(uint32_t) * ((TILE > PM ? TILE : PM) + 2 * TILE + SORT_WARPS * RBINS +
-                               3 * RBINS + SORT_WARPS + 1);
-}
-
-template <int ITEMS>
-__global__ void __launch_bounds__(SORT_THREADS)
+__global__ void __launch_bounds__(SORT_THREADS, 3)
 sweep_pass_kernel(const uint32_t *__restrict__ keys_in, const uint32_t *__restrict__ vals_in,
                   uint32_t *__restrict__ keys_out, uint32_t *__restrict__ vals_out,
                   const uint32_t *n_dev, int64_t cap, uint32_t key_lo, uint32_t key_max, int shift,
                   int width, int pass, uint32_t *head, bool index_vals, uint32_t *status)
 {
     constexpr int TILE = SORT_THREADS * ITEMS;
-    constexpr int PM = SORT_WARPS * RBINS;
-    extern __shared__ uint32_t s_mem[];
-    uint32_t *s_k = s_mem;                        // [TILE] keys, ranked order (peer masks first)
-    uint32_t *s_v = s_k + (TILE > PM ? TILE : PM); // [TILE] values, ranked order
-    uint32_t *s_vin = s_v + TILE;                 // [TILE] values, input order
-    uint32_t(*s_wh)[RBINS] = (uint32_t(*)[RBINS])(s_vin + TILE); // [warps][RBINS]
-    uint32_t *s_tot = s_vin + TILE + SORT_WARPS * RBINS;
-    uint32_t *s_dbase = s_tot + RBINS;
-    uint32_t *s_gbase = s_dbase + RBINS;
-    uint32_t *s_scan = s_gbase + RBINS;
-    uint32_t *s_tile = s_scan + SORT_WARPS;
+    __shared__ __align__(16) PassSmem<ITEMS> S;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int64_t n = dev_count(n_dev, cap);
-    if (threadIdx.x == 0) s_tile[0] = atomicAdd(head + SWEEP_PASSES * RBINS + pass, 1u);
-    for (int j = threadIdx.x; j < SORT_WARPS * RBINS; j += SORT_THREADS) {
-        (&s_wh[0][0])[j] = 0;
-        s_k[j] = 0;
-    }
+    if (threadIdx.x == 0) S.tile = atomicAdd(head + SWEEP_PASSES * RBINS + pass, 1u);
+    uint32_t *wh = S.wh_or_tile + w * RBINS; // the warp's own counters
+    for (int j = lane; j < RBINS; j += 32) wh[j] = 0;
     __syncthreads();
-    const uint32_t tile = s_tile[0];
+    const uint32_t tile = S.tile;
     const int64_t blk = (int64_t)tile * TILE;
     if (blk >= n) return;
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const uint32_t mask = (1u << width) - 1u;
     const int bins = 1 << width;
-    uint32_t *s_pm = s_k + w * RBINS; // this warp's peer masks
     const int64_t base = blk + (int64_t)w * 32 * ITEMS;
-    uint32_t key[ITEMS], rank[ITEMS];
-    const int lbase = w * 32 * ITEMS + lane; // local index of round 0
-#pragma unroll
-    for (int r = 0; r < ITEMS; ++r) {
-        const int64_t i = base + r * 32 + lane;
-        const bool ok = i < n;
-        key[r] = ok ? keys_in[i] : 0u;
-        s_vin[lbase + r * 32] = ok ? (index_vals ? (uint32_t)i : vals_in[i]) : 0u;
-    }
-    const uint32_t lt = lanemask_lt();
-    const bool full = blk + TILE <= n; // every key of the tile is in range
-    // stable rank inside the warp, as in radix_scatter_kernel
-#pragma unroll
-    for (int r = 0; r < ITEMS; ++r) {
-        const bool ok = base + r * 32 + lane < n;
-        const uint32_t d = ok ? digit_of(key[r], key_lo, key_max, shift, mask) : (uint32_t)RBINS;
-        uint32_t peers;
-        if (full || __all_sync(0xffffffffu, ok)) {
-            atomicOr(&s_pm[d], 1u << lane);
-            __syncwarp();
-            peers = s_pm[d];
-            __syncwarp();
-        } else {
-            peers = peers_by_ballot(d, false);
-        }
-        uint32_t old = 0;
-        if (d < RBINS && (peers & lt) == 0) {
-            old = atomicAdd(&s_wh[w][d], (uint32_t)__popc(peers));
-            s_pm[d] = 0;
-        }
-        __syncwarp(); // peer words clear before the next round's ORs
-        rank[r] = (uint32_t)(__ffs(peers) - 1) | ((uint32_t)__popc(peers & lt) << 5) | (old << 10);
-    }
-#pragma unroll
-    for (int r = 0; r < ITEMS; ++r) {
-        const uint32_t packed = rank[r];
-        const uint32_t base_r = __shfl_sync(0xffffffffu, packed >> 10, packed & 31);
-        rank[r] = base_r + ((packed >> 5) & 31);
-    }
+    const int cnt = share_count<ITEMS>(base, n);
+    uint32_t key[ITEMS], rank[ITEMS], val[ITEMS];
+    load_share(key, keys_in + base, cnt);
+    reduce_keys(key, key_lo, key_max);
+    rank_in_warp(key, rank, cnt, shift, width, wh);
     __syncthreads();
-    // per digit: exclusive prefix over warps, and the tile's count, published
-    constexpr int PER = RBINS / SORT_THREADS;
     uint32_t *states = head + SWEEP_HEAD;
     const uint32_t agg = 2u * (uint32_t)pass + 1u;
-    uint32_t mine[PER];
+    uint32_t tot[2], first[2];
+    digit_slots(S.wh_or_tile, S.scan, tot, first, [&](const uint32_t (&t)[2]) {
 #pragma unroll
-    for (int k = 0; k < PER; ++k) {
-        const int dd = threadIdx.x + k * SORT_THREADS;
-        uint32_t t = 0;
-        if (dd < bins) {
-#pragma unroll
-            for (int j = 0; j < SORT_WARPS; ++j) {
-                const uint32_t x = s_wh[j][dd];
-                s_wh[j][dd] = t;
-                t += x;
-            }
-            st_state(states + (size_t)tile * RBINS + dd, t | ((tile == 0 ? agg + 1u : agg) << 28));
+        for (int k = 0; k < 2; ++k) {
+            const int dd = 2 * threadIdx.x + k;
+            if (dd < bins)
+                st_state(states + (size_t)tile * RBINS + dd,
+                         t[k] | ((tile == 0 ? agg + 1u : agg) << 28));
         }
-        s_tot[dd] = t;
-        mine[k] = t;
+    });
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        S.tot[2 * threadIdx.x + k] = tot[k];
+        S.gbase[2 * threadIdx.x + k] = first[k];
     }
     __syncthreads();
-    // block exclusive scan of the digit totals
-    {
-        uint32_t loc[PER], sum = 0;
-#pragma unroll
-        for (int q = 0; q < PER; ++q) {
-            loc[q] = s_tot[threadIdx.x * PER + q];
-            sum += loc[q];
+    const auto slot = slots_of(rank, wh);
+    load_vals(val, vals_in, base, cnt, index_vals);
+    __syncthreads(); // the counters' place is the tile's from here
+    place(key, slot, cnt, S.wh_or_tile);
+    // add up the tiles before it
+    for (int dd = threadIdx.x; dd < bins; dd += SORT_THREADS) {
+        uint32_t before = 0;
+        if (tile > 0) {
+            before = look_back(states + dd, tile, agg, status);
+            st_state(states + (size_t)tile * RBINS + dd, (before + S.tot[dd]) | ((agg + 1u) << 28));
         }
-        const uint32_t inc = warp_incl_scan(sum);
-        if (lane == 31) s_scan[w] = inc;
-        __syncthreads();
-        uint32_t off = inc - sum;
-        for (int j = 0; j < w; ++j) off += s_scan[j];
-#pragma unroll
-        for (int q = 0; q < PER; ++q) {
-            s_dbase[threadIdx.x * PER + q] = off;
-            off += loc[q];
-        }
+        S.gbase[dd] = head[pass * RBINS + dd] + before - S.gbase[dd];
     }
     __syncthreads();
-    // place the tile in digit order, then add up the tiles before it
-#pragma unroll
-    for (int r = 0; r < ITEMS; ++r) {
-        if (base + r * 32 + lane < n) {
-            const uint32_t d = digit_of(key[r], key_lo, key_max, shift, mask);
-            const uint32_t l = s_dbase[d] + s_wh[w][d] + rank[r];
-            s_k[l] = key[r];
-            s_v[l] = s_vin[lbase + r * 32];
-        }
-    }
-#pragma unroll
-    for (int k = 0; k < PER; ++k) {
-        const int dd = threadIdx.x + k * SORT_THREADS;
-        if (dd < bins) {
-            uint32_t before = 0;
-            if (tile > 0) {
-                before = look_back(states + dd, tile, agg, status);
-                st_state(states + (size_t)tile * RBINS + dd, (before + mine[k]) | ((agg + 1u) << 28));
-            }
-            // output position of ranked slot j of digit d: s_gbase[d] + j
-            s_gbase[dd] = head[pass * RBINS + dd] + before - s_dbase[dd];
-        }
-    }
-    __syncthreads();
-    const int cnt = (int)(n - blk < TILE ? n - blk : TILE);
-    for (int j = threadIdx.x; j < cnt; j += SORT_THREADS) {
-        const uint32_t k = s_k[j];
-        const uint32_t g = s_gbase[digit_of(k, key_lo, key_max, shift, mask)] + (uint32_t)j;
-        keys_out[g] = k;
-        vals_out[g] = s_v[j];
-    }
+    write_tile(S, val, slot, cnt, (int)(n - blk < TILE ? n - blk : TILE), shift, width, keys_out,
+               vals_out);
 }
 
 // ------------------------------------------------------------ emission
@@ -990,13 +960,8 @@ void sweep_pass(const uint32_t *keys, const uint32_t *vals, uint32_t *keys_alt, 
                 const uint32_t *n_dev, int64_t cap, const SweepDigits &dg, int pass, uint32_t *head,
                 bool index_vals, uint32_t *status, cudaStream_t s)
 {
-    static const bool attr = cudaFuncSetAttribute(sweep_pass_kernel<ITEMS>,
-                                                  cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                  (int)sweep_smem<ITEMS>()) == cudaSuccess;
-    (void)attr;
     const int64_t tile = SORT_THREADS * ITEMS;
-    sweep_pass_kernel<ITEMS><<<(unsigned)((cap + tile - 1) / tile), SORT_THREADS,
-                               sweep_smem<ITEMS>(), s>>>(
+    sweep_pass_kernel<ITEMS><<<(unsigned)((cap + tile - 1) / tile), SORT_THREADS, 0, s>>>(
         keys, vals, keys_alt, vals_alt, n_dev, cap, dg.key_lo, dg.key_max, dg.shift[pass],
         dg.width[pass], pass, head, index_vals, status);
 }
@@ -1063,15 +1028,12 @@ void radix_sort_pairs(uint32_t *&keys, uint32_t *&vals, uint32_t *&keys_alt, uin
             auto f = sweep_items(cap) == 16 ? sweep_pass<16> : sweep_pass<4>;
             f(keys, vals, keys_alt, vals_alt, n_dev, cap, dg, p, head, index_vals && p == 0, status,
               s);
+            dg.key_lo = 0; // the keys written are the reduced ones
             swap();
         }
         count_launches(1 + passes);
         return;
     }
-    static const bool attr = cudaFuncSetAttribute(radix_scatter_kernel,
-                                                  cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                  (int)SCATTER_SMEM) == cudaSuccess;
-    (void)attr;
     const int64_t nb = (cap + SORT_TILE - 1) / SORT_TILE;
     uint32_t *hist = (uint32_t *)temp;
     void *scan_tmp = hist + nb * RBINS;
@@ -1080,10 +1042,11 @@ void radix_sort_pairs(uint32_t *&keys, uint32_t *&vals, uint32_t *&keys_alt, uin
         radix_hist_kernel<<<(unsigned)((nb + HIST_TILES - 1) / HIST_TILES), SORT_THREADS, 0, s>>>(
             keys, n_dev, cap, key_lo, key_max, shift, wd, hist, nb);
         run_scan(LoadU32{hist}, ActStore{hist}, nullptr, nb << wd, scan_tmp, nullptr, nullptr, s);
-        radix_scatter_kernel<<<(unsigned)nb, SORT_THREADS, SCATTER_SMEM, s>>>(
+        radix_scatter_kernel<<<(unsigned)nb, SORT_THREADS, 0, s>>>(
             keys, vals, keys_alt, vals_alt, n_dev, cap, key_lo, key_max, shift, wd, hist, nb,
             index_vals && shift == bit_lo);
         count_launches(2);
+        key_lo = 0; // the keys written are the reduced ones
         swap();
     }
 }
