@@ -56,7 +56,7 @@ struct Request {
     double t_arrival = 0, t_done = 0;
     int32_t status = PBR_OK;
     bool done = false;
-    size_t bytes = 0;
+    size_t bytes = 0, bound = 0; // reserved; admission_bytes
 };
 
 struct InFlight {
@@ -185,10 +185,16 @@ bool ServeState::launch_one()
             break;
         }
     if (slot < 0 || queue.empty()) return false;
+    // Requests share a batch while their host bounds fit the budget together
+    // (what the batch reserves may be less: reserve_bytes).  Going by the
+    // reservations alone, a budget of one bound and a half put one or two
+    // requests into a batch depending on whether the batch before had finished
+    // when its event was polled.
     std::vector<uint64_t> ids;
-    size_t bytes = 0;
+    size_t bytes = 0, bounds = 0;
     while (!queue.empty() && (int)ids.size() < max_views) {
         Request &r = reqs[queue.front()];
+        if (!ids.empty() && (r.bound > budget || bounds > budget - r.bound)) break;
         if (in_use + bytes + r.bytes > budget) {
             if (ids.empty() && inflight.empty()) { // can never fit: reject
                 r.done = true;
@@ -202,6 +208,7 @@ bool ServeState::launch_one()
             break; // wait for memory to free up
         }
         bytes += r.bytes;
+        bounds += r.bound;
         ids.push_back(queue.front());
         queue.pop_front();
     }
@@ -506,6 +513,7 @@ extern "C" int pbr_submit_request(pbr_ctx *c, int32_t scene_id, const pbr_camera
         r.out = out_rgb_device;
         r.t_arrival = arrival_time > 0.0 ? arrival_time : now_s();
         r.bytes = bytes;
+        r.bound = bound;
         S->reqs[r.id] = r;
         S->queue.push_back(r.id);
         ++S->submitted;
