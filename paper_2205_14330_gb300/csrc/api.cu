@@ -8,6 +8,7 @@
 #include <cstring>
 #include <mutex>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "pbr.h"
@@ -404,16 +405,105 @@ size_t pbr::store_bytes(int32_t store_depth, int64_t n_pix)
 
 void pbr_state::release()
 {
-    void **all[] = {(void **)&d_views, (void **)&d_scenes, (void **)&d_view_list, (void **)&rec,
-                    (void **)&ntiles, (void **)&counters, (void **)&tile_keys,
-                    (void **)&tile_vals, (void **)&ranges, (void **)&T_final,
-                    (void **)&n_contrib, (void **)&tile_order, (void **)&work,
-                    (void **)&T_store, (void **)&n_comp};
-    for (void **p : all) {
-        dfree(*p, stream);
-        *p = nullptr;
+    for (void *&p : mem) {
+        dfree(p, stream);
+        p = nullptr;
+    }
+    d_views = nullptr;
+    d_scenes = nullptr;
+    d_view_list = nullptr;
+    rec = nullptr;
+    ntiles = n_contrib = work = n_comp = tile_keys = tile_vals = nullptr;
+    counters = nullptr;
+    ranges = nullptr;
+    T_final = T_store = nullptr;
+    tile_order = nullptr;
+}
+
+namespace {
+
+// Buffers of one lifetime, laid out at 256-byte boundaries and allocated as
+// one: a forward pass needs some 25 buffers, and 25 stream-ordered allocations
+// and frees cost its host path more than its kernels take on small views
+// (one 640 x 480 view of 100k points: 151 -> 144 us a call).
+struct Arena {
+    size_t size = 0, bytes = 0; // allocated, asked for
+    std::vector<std::pair<void **, size_t>> parts;
+    template <class T> void add(T **p, size_t want)
+    {
+        want = std::max<size_t>(want, 16);
+        parts.emplace_back((void **)p, size);
+        bytes += want;
+        size += (want + 255) & ~(size_t)255;
+    }
+    void place(void *base)
+    {
+        for (auto &q : parts) *q.first = (char *)base + q.second;
+    }
+};
+
+// A forward pass's temporaries.
+struct ForwardTemps {
+    uint32_t *zbits = nullptr, *vk = nullptr, *vv = nullptr, *vk2 = nullptr, *vv2 = nullptr;
+    uint32_t *pk = nullptr, *pv = nullptr; // the pair lists' other buffers
+    uint4 *rect = nullptr;
+    uint8_t *nt8 = nullptr;
+    void *temp = nullptr;
+};
+
+// With most point-views visible, all of them are sorted by depth directly:
+// the invisible ones (key 0xffffffff, clamped to one above the deepest visible
+// key) land behind the visible ones, and no compaction pass is needed.
+// Otherwise the visible ones are compacted first.
+bool sort_all(int64_t n_vis, int64_t n_pv) { return n_vis > 0 && 4 * n_vis >= 3 * n_pv; }
+
+// Buffers of the per-point stage: the state's, the uploaded tables and the
+// counters leading, and temporaries.
+void plan_points(const HostLayout &L, pbr_state *st, ForwardTemps &t, Arena &kept, Arena &temps)
+{
+    const size_t npv = (size_t)L.n_pv;
+    kept.add(&st->counters, 128);
+    kept.add(&st->d_views, sizeof(DevView) * L.views.size());
+    kept.add(&st->d_scenes, sizeof(DevScene) * L.scenes.size());
+    kept.add(&st->d_view_list, sizeof(int32_t) * L.view_list.size());
+    kept.add(&st->rec, sizeof(float4) * 2 * npv);
+    kept.add(&st->ntiles, sizeof(uint32_t) * npv);
+    temps.add(&t.zbits, sizeof(uint32_t) * npv);
+    temps.add(&t.rect, sizeof(uint4) * npv);
+    temps.add(&t.nt8, npv);
+}
+
+// Buffers of the stages after it.
+void plan_lists(const HostLayout &L, int64_t n_vis, int64_t n_pairs, bool persist,
+                int32_t store_depth, pbr_state *st, ForwardTemps &t, Arena &kept, Arena &temps)
+{
+    const bool direct = sort_all(n_vis, L.n_pv);
+    const size_t n_sort = (size_t)(direct ? L.n_pv : n_vis), np = (size_t)n_pairs;
+    const int64_t cap_sort = std::max<int64_t>((int64_t)n_sort, n_pairs);
+    if (!direct) temps.add(&t.vk, sizeof(uint32_t) * n_sort);
+    temps.add(&t.vv, sizeof(uint32_t) * n_sort);
+    temps.add(&t.vk2, sizeof(uint32_t) * n_sort);
+    temps.add(&t.vv2, sizeof(uint32_t) * n_sort);
+    temps.add(&t.pk, sizeof(uint32_t) * np);
+    temps.add(&t.pv, sizeof(uint32_t) * np);
+    temps.add(&t.temp, std::max(std::max(scan_temp_bytes(L.n_pv), radix_temp_bytes(cap_sort)),
+                                emit_temp_bytes(n_vis)));
+    kept.add(&st->tile_keys, sizeof(uint32_t) * np);
+    kept.add(&st->tile_vals, sizeof(uint32_t) * np);
+    kept.add(&st->ranges, sizeof(uint2) * L.n_tiles);
+    kept.add(&st->T_final, sizeof(float) * L.n_pix);
+    kept.add(&st->n_contrib, sizeof(uint32_t) * L.n_pix);
+    if (persist) {
+        kept.add(&st->tile_order, sizeof(uint4) * L.n_tiles);
+        kept.add(&st->work, 64 * sizeof(uint32_t));
+    }
+    if (store_depth > 0) {
+        kept.add(&st->T_store, sizeof(float) * (size_t)store_depth * (size_t)L.n_pix);
+        kept.add(&st->n_comp, sizeof(uint32_t) * L.n_pix);
     }
 }
+
+} // namespace
 
 // Runs the forward chain into the state's buffers.  Exact-size workspaces:
 // one host synchronisation after the per-point stage reads the pair count.
@@ -421,30 +511,37 @@ int pbr::forward_eager(pbr_ctx *c, pbr_state *st, float *out_rgb, cudaStream_t s
 {
     HostLayout &L = st->layout;
     const DevOpts &o = st->dopts;
-    // tables
-    PBR_TRY(dalloc((void **)&st->d_views, sizeof(DevView) * L.views.size(), s));
-    PBR_TRY(dalloc((void **)&st->d_scenes, sizeof(DevScene) * L.scenes.size(), s));
-    PBR_TRY(dalloc((void **)&st->d_view_list, sizeof(int32_t) * L.view_list.size(), s));
-    PBR_CUDA(cudaMemcpyAsync(st->d_views, L.views.data(), sizeof(DevView) * L.views.size(),
-                             cudaMemcpyHostToDevice, s));
-    PBR_CUDA(cudaMemcpyAsync(st->d_scenes, L.scenes.data(), sizeof(DevScene) * L.scenes.size(),
-                             cudaMemcpyHostToDevice, s));
-    PBR_CUDA(cudaMemcpyAsync(st->d_view_list, L.view_list.data(),
-                             sizeof(int32_t) * L.view_list.size(), cudaMemcpyHostToDevice, s));
+    const bool persist = st->opts.persistent && st->batch_depth == 0;
+    TempBufs tmp(s);
+    ForwardTemps ft;
+    {
+        Arena kept, temps;
+        void *base = nullptr;
+        plan_points(L, st, ft, kept, temps);
+        PBR_TRY(tmp.alloc(&base, temps.size));
+        temps.place(base);
+        PBR_TRY(dalloc(&st->mem[0], kept.size, s));
+        kept.place(st->mem[0]);
+    }
+    // the counters' first values (the smallest depth bits: all ones) and the
+    // tables, in one copy
+    {
+        char *first = (char *)st->counters;
+        std::vector<char> up((char *)st->rec - first, 0);
+        std::memset(up.data() + 48, 0xff, 4);
+        auto put = [&](const void *dst, const void *src, size_t bytes) {
+            if (bytes) std::memcpy(up.data() + ((const char *)dst - first), src, bytes);
+        };
+        put(st->d_views, L.views.data(), sizeof(DevView) * L.views.size());
+        put(st->d_scenes, L.scenes.data(), sizeof(DevScene) * L.scenes.size());
+        put(st->d_view_list, L.view_list.data(), sizeof(int32_t) * L.view_list.size());
+        PBR_CUDA(cudaMemcpyAsync(first, up.data(), up.size(), cudaMemcpyHostToDevice, s));
+    }
     Batch b = st->batch();
     const int64_t npv = L.n_pv;
-    PBR_TRY(dalloc((void **)&st->rec, sizeof(float4) * 2 * npv, s));
-    PBR_TRY(dalloc((void **)&st->ntiles, sizeof(uint32_t) * npv, s));
-    PBR_TRY(dalloc((void **)&st->counters, 128, s));
-    TempBufs tmp(s);
-    uint32_t *zbits = nullptr;
-    uint4 *rect = nullptr;
-    uint8_t *nt8 = nullptr;
-    PBR_TRY(tmp.alloc(&zbits, sizeof(uint32_t) * npv));
-    PBR_TRY(tmp.alloc(&rect, sizeof(uint4) * npv));
-    PBR_TRY(tmp.alloc(&nt8, (size_t)npv));
-    PBR_CUDA(cudaMemsetAsync(st->counters, 0, 128, s));
-    PBR_CUDA(cudaMemsetAsync((char *)st->counters + 48, 0xff, 4, s)); // depth-bits minimum
+    uint32_t *zbits = ft.zbits;
+    uint4 *rect = ft.rect;
+    uint8_t *nt8 = ft.nt8;
     {
         StageScope t(c, STG_PREPROCESS_FWD, s);
         launch_preprocess_fwd(b, o, st->rec, zbits, st->ntiles, nt8, rect, st->counters, s);
@@ -459,39 +556,28 @@ int pbr::forward_eager(pbr_ctx *c, pbr_state *st, float *out_rgb, cudaStream_t s
     const uint64_t n_pairs = host[0], n_vis = host[1];
     const uint32_t zlo = ((const uint32_t *)host)[12];
     const uint32_t zhi = ((const uint32_t *)host)[13];
-    // With most point-views visible, all of them are sorted by depth
-    // directly: the invisible ones (key 0xffffffff, clamped to one above the
-    // deepest visible key) land behind the visible ones, and no compaction
-    // pass is needed.  Otherwise the visible ones are compacted first.
-    const bool direct = n_vis > 0 && 4 * n_vis >= 3 * (uint64_t)npv;
+    const bool direct = sort_all((int64_t)n_vis, npv);
     const uint32_t marker = n_vis > 0 ? zhi - zlo + 1 : 0u;
     const int depth_bits = direct ? 32 - __builtin_clz(marker)
                                   : (n_vis > 0 && zhi > zlo) ? 32 - __builtin_clz(zhi - zlo) : 0;
-    const int64_t n_sort = direct ? npv : (int64_t)n_vis;
     if (n_pairs >= UINT32_MAX) {
         return set_error(PBR_ERR_CAPACITY, "%llu (tile, point-view) pairs exceed 2^32-1",
                          (unsigned long long)n_pairs);
     }
     st->n_vis = (int64_t)n_vis;
     st->n_pairs = (int64_t)n_pairs;
-    uint32_t *vk = nullptr, *vv = nullptr, *vk2 = nullptr, *vv2 = nullptr;
-    uint32_t *pk2 = nullptr, *pv2 = nullptr;
-    void *temp = nullptr;
-    const int64_t cap_sort = std::max<int64_t>(n_sort, n_pairs);
-    const size_t temp_bytes = std::max(std::max(scan_temp_bytes(npv), radix_temp_bytes(cap_sort)),
-                                       emit_temp_bytes((int64_t)n_vis));
-    if (!direct) PBR_TRY(tmp.alloc(&vk, sizeof(uint32_t) * n_sort));
-    PBR_TRY(tmp.alloc(&vv, sizeof(uint32_t) * n_sort));
-    PBR_TRY(tmp.alloc(&vk2, sizeof(uint32_t) * n_sort));
-    PBR_TRY(tmp.alloc(&vv2, sizeof(uint32_t) * n_sort));
-    PBR_TRY(dalloc((void **)&st->tile_keys, sizeof(uint32_t) * n_pairs, s));
-    PBR_TRY(dalloc((void **)&st->tile_vals, sizeof(uint32_t) * n_pairs, s));
-    PBR_TRY(tmp.alloc(&pk2, sizeof(uint32_t) * n_pairs));
-    PBR_TRY(tmp.alloc(&pv2, sizeof(uint32_t) * n_pairs));
-    PBR_TRY(dalloc((void **)&st->ranges, sizeof(uint2) * L.n_tiles, s));
-    PBR_TRY(dalloc((void **)&st->T_final, sizeof(float) * L.n_pix, s));
-    PBR_TRY(dalloc((void **)&st->n_contrib, sizeof(uint32_t) * L.n_pix, s));
-    PBR_TRY(tmp.alloc(&temp, temp_bytes));
+    {
+        Arena kept, temps;
+        void *base = nullptr;
+        plan_lists(L, (int64_t)n_vis, (int64_t)n_pairs, persist, st->store_depth, st, ft, kept,
+                   temps);
+        PBR_TRY(tmp.alloc(&base, temps.size));
+        temps.place(base);
+        PBR_TRY(dalloc(&st->mem[1], kept.size, s));
+        kept.place(st->mem[1]);
+    }
+    uint32_t *vk = ft.vk, *vv = ft.vv, *vk2 = ft.vk2, *vv2 = ft.vv2;
+    void *temp = ft.temp;
     uint32_t *status = (uint32_t *)((char *)st->counters + 64);
     const uint32_t *n_vis_dev = (const uint32_t *)(st->counters + 1);  // low word (< 2^32)
     const uint32_t *n_pairs_dev = (const uint32_t *)(st->counters + 0); // low word (< 2^32)
@@ -511,7 +597,12 @@ int pbr::forward_eager(pbr_ctx *c, pbr_state *st, float *out_rgb, cudaStream_t s
                              zlo, 0xffffffffu, false, 0, status);
     }
     // 3. duplicate per covered tile, in depth order
-    uint32_t *tk = st->tile_keys, *tv = st->tile_vals;
+    // (each pass of the tile sort moves the list to the other buffers: it
+    // starts in those from which it ends in the state's)
+    const int tile_bits = key_bits_for(L.n_tiles);
+    const bool odd = radix_passes(tile_bits) & 1;
+    uint32_t *tk = odd ? ft.pk : st->tile_keys, *tv = odd ? ft.pv : st->tile_vals;
+    uint32_t *pk2 = odd ? st->tile_keys : ft.pk, *pv2 = odd ? st->tile_vals : ft.pv;
     {
         StageScope t(c, STG_EMIT, s);
         launch_emit_pairs(b, o, vv, n_vis_dev, (int64_t)n_vis, st->ntiles, nt8, rect, tk, tv,
@@ -520,18 +611,11 @@ int pbr::forward_eager(pbr_ctx *c, pbr_state *st, float *out_rgb, cudaStream_t s
     // 4. stable sort by tile id
     {
         StageScope t(c, STG_TILE_SORT, s);
-        radix_sort_pairs(tk, tv, pk2, pv2, n_pairs_dev, (int64_t)n_pairs,
-                         key_bits_for(L.n_tiles), temp, s, 0, 0xffffffffu, false,
-                         block_bits(o.tile_w, o.tile_h), status);
+        radix_sort_pairs(tk, tv, pk2, pv2, n_pairs_dev, (int64_t)n_pairs, tile_bits, temp, s, 0,
+                         0xffffffffu, false, block_bits(o.tile_w, o.tile_h), status);
     }
-    if (tk != st->tile_keys) { // result landed in the alternate buffers: swap ownership
-        for (void *&p : tmp.ptrs) {
-            if (p == (void *)tk) p = (void *)st->tile_keys;
-            else if (p == (void *)tv) p = (void *)st->tile_vals;
-        }
-        st->tile_keys = tk;
-        st->tile_vals = tv;
-    }
+    if (n_pairs > 0 && tk != st->tile_keys)
+        return set_error(PBR_ERR_CUDA, "the tile sort ended in the wrong buffers");
     // 5. per-tile ranges
     {
         StageScope t(c, STG_RANGES, s);
@@ -540,16 +624,6 @@ int pbr::forward_eager(pbr_ctx *c, pbr_state *st, float *out_rgb, cudaStream_t s
                            block_bits(o.tile_w, o.tile_h), s);
     }
     // 6. composite (optionally as one persistent launch over a longest-first tile order)
-    const bool persist = st->opts.persistent && st->batch_depth == 0;
-    if (persist) {
-        PBR_TRY(dalloc((void **)&st->tile_order, sizeof(uint4) * L.n_tiles, s));
-        PBR_TRY(dalloc((void **)&st->work, 64 * sizeof(uint32_t), s));
-    }
-    if (st->store_depth > 0) {
-        PBR_TRY(dalloc((void **)&st->T_store,
-                       sizeof(float) * (size_t)st->store_depth * (size_t)L.n_pix, s));
-        PBR_TRY(dalloc((void **)&st->n_comp, sizeof(uint32_t) * L.n_pix, s));
-    }
     {
         StageScope t(c, STG_RASTER_FWD, s);
         if (persist) launch_tile_order(b, st->ranges, L.n_tiles, st->tile_order, st->work, s);
@@ -565,32 +639,18 @@ int pbr::forward_eager(pbr_ctx *c, pbr_state *st, float *out_rgb, cudaStream_t s
     return PBR_OK;
 }
 
-// The bytes forward_eager allocates (each allocation at least 16 bytes), all
-// alive at its end: the state's buffers, the call's temporaries and, in store
-// mode, the transmittance list.
+// The bytes of forward_eager's buffers (before their rounding to 256), all
+// alive at its end: the state's, the call's temporaries and, in store mode,
+// the transmittance list.
 size_t pbr::forward_bytes(const HostLayout &L, int64_t n_vis, int64_t n_pairs,
                           const pbr_render_opts *o, int32_t store_depth)
 {
-    auto al = [](size_t b) { return b ? b : (size_t)16; };
-    const int64_t npv = L.n_pv;
-    const bool direct = n_vis > 0 && 4 * n_vis >= 3 * npv;
-    const int64_t n_sort = direct ? npv : n_vis;
-    const int64_t cap_sort = std::max<int64_t>(n_sort, n_pairs);
-    const size_t temp = std::max(std::max(scan_temp_bytes(npv), radix_temp_bytes(cap_sort)),
-                                 emit_temp_bytes(n_vis));
-    size_t b = al(sizeof(DevView) * L.views.size()) + al(sizeof(DevScene) * L.scenes.size()) +
-               al(sizeof(int32_t) * L.view_list.size());
-    b += al(32 * (size_t)npv) + al(4 * (size_t)npv) + 128;         // records, tile counts, counters
-    b += al(4 * (size_t)npv) + al(16 * (size_t)npv) + al((size_t)npv); // depth bits, rectangles,
-                                                                         // one-byte counts
-    b += (direct ? 0 : al(4 * (size_t)n_sort)) + 3 * al(4 * (size_t)n_sort); // depth sort
-    b += 4 * al(4 * (size_t)n_pairs);                              // pair lists, sort buffers
-    b += al(8 * (size_t)L.n_tiles) + 2 * al(4 * (size_t)L.n_pix);  // ranges, T_final, n_contrib
-    b += al(temp);
-    if (o->persistent && o->batch_depth == 0) b += al(16 * (size_t)L.n_tiles) + 256;
-    if (store_depth > 0)
-        b += al(4 * (size_t)store_depth * (size_t)L.n_pix) + al(4 * (size_t)L.n_pix);
-    return b;
+    pbr_state st;
+    ForwardTemps t;
+    Arena a;
+    plan_points(L, &st, t, a, a);
+    plan_lists(L, n_vis, n_pairs, o->persistent && o->batch_depth == 0, store_depth, &st, t, a, a);
+    return a.bytes;
 }
 
 extern "C" int pbr_forward_workspace_size(pbr_ctx *c, const pbr_points *scenes, int32_t n_scenes,

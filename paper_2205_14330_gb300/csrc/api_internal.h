@@ -80,7 +80,9 @@ struct pbr_state {
     int batch_depth = 256;
     pbr::HostLayout layout;
     int64_t n_vis = 0, n_pairs = 0;
-    // device buffers kept for the backward pass (all freed by release())
+    // device buffers kept for the backward pass, in two allocations (freed by
+    // release())
+    void *mem[2] = {nullptr, nullptr};
     pbr::DevView *d_views = nullptr;
     pbr::DevScene *d_scenes = nullptr;
     int32_t *d_view_list = nullptr;
