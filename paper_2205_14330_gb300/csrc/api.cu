@@ -591,10 +591,10 @@ int pbr::forward_eager(pbr_ctx *c, pbr_state *st, float *out_rgb, cudaStream_t s
         StageScope t(c, STG_DEPTH_SORT, s);
         if (direct)
             radix_sort_pairs(zbits, vv, vk2, vv2, nullptr, npv, depth_bits, temp, s, zlo, marker,
-                             true, 0, status);
+                             true);
         else
             radix_sort_pairs(vk, vv, vk2, vv2, n_vis_dev, (int64_t)n_vis, depth_bits, temp, s,
-                             zlo, 0xffffffffu, false, 0, status);
+                             zlo);
     }
     // 3. duplicate per covered tile, in depth order
     // (each pass of the tile sort moves the list to the other buffers: it
@@ -612,7 +612,7 @@ int pbr::forward_eager(pbr_ctx *c, pbr_state *st, float *out_rgb, cudaStream_t s
     {
         StageScope t(c, STG_TILE_SORT, s);
         radix_sort_pairs(tk, tv, pk2, pv2, n_pairs_dev, (int64_t)n_pairs, tile_bits, temp, s, 0,
-                         0xffffffffu, false, block_bits(o.tile_w, o.tile_h), status);
+                         0xffffffffu, false, block_bits(o.tile_w, o.tile_h));
     }
     if (n_pairs > 0 && tk != st->tile_keys)
         return set_error(PBR_ERR_CUDA, "the tile sort ended in the wrong buffers");
@@ -914,6 +914,28 @@ extern "C" int pbr_optimizer_step(int32_t kind, float *param, const float *grad,
         return set_error(PBR_ERR_INVALID_ARG, "pbr_optimizer_step: bad arguments");
     OptParams prm{kind, lr, beta1, beta2, eps, step};
     launch_optimizer(prm, nullptr, 0, param, grad, m, v, n, (cudaStream_t)stream);
+    PBR_CUDA(cudaGetLastError());
+    return PBR_OK;
+}
+
+// For the tests (not in the header): sorts (keys, vals) [n], in place, by the
+// low key_bits bits.  polls: see radix_sort_pairs.
+extern "C" int pbr_test_sort_pairs(uint32_t *keys, uint32_t *vals, int64_t n, int32_t key_bits,
+                                   int32_t polls, pbr_stream_t stream)
+{
+    cudaStream_t s = (cudaStream_t)stream;
+    TempBufs tb(s);
+    uint32_t *k = keys, *v = vals, *k2 = nullptr, *v2 = nullptr;
+    void *temp = nullptr;
+    PBR_TRY(tb.alloc(&k2, sizeof(uint32_t) * n));
+    PBR_TRY(tb.alloc(&v2, sizeof(uint32_t) * n));
+    PBR_TRY(tb.alloc(&temp, radix_temp_bytes(n)));
+    radix_sort_pairs(k, v, k2, v2, nullptr, n, key_bits, temp, s, 0, 0xffffffffu, false, 0, false,
+                     polls);
+    if (k != keys) {
+        PBR_CUDA(cudaMemcpyAsync(keys, k, sizeof(uint32_t) * n, cudaMemcpyDeviceToDevice, s));
+        PBR_CUDA(cudaMemcpyAsync(vals, v, sizeof(uint32_t) * n, cudaMemcpyDeviceToDevice, s));
+    }
     PBR_CUDA(cudaGetLastError());
     return PBR_OK;
 }

@@ -157,14 +157,14 @@ extern "C" int pbr_render_forward_noalloc(const pbr_points *scenes, int32_t n_sc
     const uint32_t *n_pairs_dev = (const uint32_t *)(counters + 0);
     launch_compact_visible(ntiles, zbits, npv, vk, vv, nullptr, temp, s);
     radix_sort_pairs(vk, vv, vk2, vv2, n_vis_dev, (int64_t)n_vis, 32, temp, s, 0, 0xffffffffu,
-                     false, 0, status, least);
+                     false, 0, least);
     launch_emit_pairs(b, o, vv, n_vis_dev, (int64_t)n_vis, ntiles, nt8, rect, tk, tv,
                       (int64_t)n_pairs, status, temp, s);
     int key_bits = 1;
     while (key_bits < 32 && ((L.n_tiles - 1) >> key_bits)) ++key_bits;
     const int sb = block_bits(o.tile_w, o.tile_h);
     radix_sort_pairs(tk, tv, pk2, pv2, n_pairs_dev, (int64_t)n_pairs, key_bits, temp, s, 0,
-                     0xffffffffu, false, sb, status, least);
+                     0xffffffffu, false, sb, least);
     PBR_CUDA(cudaMemsetAsync(ranges, 0, sizeof(uint2) * L.n_tiles, s));
     launch_tile_ranges(tk, n_pairs_dev, (int64_t)n_pairs, ranges, L.n_tiles, sb, s);
     launch_raster_fwd(b, o, opts->batch_depth, ranges, tk, tv, rec, out_rgb, T_final, n_contrib,

@@ -181,11 +181,11 @@ void enqueue_forward(pbr_graph *g, cudaStream_t s)
     if (g->direct_depth) {
         vk = g->zbits;
         radix_sort_pairs(vk, vv, vk2, vv2, nullptr, L.n_pv, g->depth_bits, g->temp, s,
-                         g->depth_lo, g->depth_marker, true, 0, status);
+                         g->depth_lo, g->depth_marker, true);
     } else {
         launch_compact_visible(g->ntiles, g->zbits, L.n_pv, g->vk, g->vv, nullptr, g->temp, s);
         radix_sort_pairs(vk, vv, vk2, vv2, n_vis_dev, g->cap_vis, g->depth_bits, g->temp, s,
-                         g->depth_lo, 0xffffffffu, false, 0, status);
+                         g->depth_lo);
     }
     uint32_t *tk = g->tk, *tv = g->tv, *tk2 = g->tk2, *tv2 = g->tv2;
     launch_emit_pairs(b, o, vv, n_vis_dev, g->cap_vis, g->ntiles, g->nt8, g->rect, tk, tv,
@@ -194,7 +194,7 @@ void enqueue_forward(pbr_graph *g, cudaStream_t s)
     if (key_bits < 1) key_bits = 1;
     const int sb = block_bits(o.tile_w, o.tile_h);
     radix_sort_pairs(tk, tv, tk2, tv2, n_pairs_dev, g->cap_pairs, key_bits, g->temp, s, 0,
-                     0xffffffffu, false, sb, status);
+                     0xffffffffu, false, sb);
     g->keys_final = tk;
     g->vals_final = tv;
     cudaMemsetAsync(g->ranges, 0, sizeof(uint2) * L.n_tiles, s);

@@ -21,7 +21,9 @@
 // radix pass ranks keys stably inside a block with ballots and a counter per
 // warp and digit, and reorders them in shared memory so that the scatter writes
 // contiguous runs.  Short sorts run in one sweep
-// (one histogram of every digit, then a kernel per pass with look-back), long
+// (one histogram of every digit, then a kernel per pass with look-back: the
+// method of Merrill and Garland, "Single-pass Parallel Prefix Scan with
+// Decoupled Look-back", 2016, and Adinets and Merrill, "Onesweep", 2022), long
 // ones with a histogram, a scan and a scatter per pass.
 #include <algorithm>
 
@@ -508,11 +510,11 @@ radix_scatter_kernel(const uint32_t *__restrict__ keys_in, const uint32_t *__res
 // it (28 bits) under a tag: 2 pass + 1 or 2 pass + 2; words of an earlier
 // pass carry smaller tags, so one clear serves all passes.  Tiles are taken
 // from a counter, so every tile before a block's own is running or done and
-// each wait ends; the waits are bounded all the same (SWEEP_SPINS polls, then
-// ST_SORT_STALL in *status and whatever order results).
+// each wait ends; the waits are bounded all the same: after SORT_POLLS polls a
+// thread counts its digit in the keys of a tile that has not reported, so that
+// no order of execution can change the result.
 constexpr int SWEEP_PASSES = 4;
 constexpr uint32_t SWEEP_COUNT = 0x0fffffffu; // counts a state word can hold
-constexpr int SWEEP_SPINS = 1 << 22;
 constexpr int64_t SWEEP_HIST_BLOCKS = 152 * 8;
 // Sorts of up to SWEEP_MOST entries run in one sweep, those below SWEEP_SMALL
 // with small tiles.  Depth and tile sort of one batch together (keys of 24 and
@@ -609,12 +611,13 @@ __device__ __forceinline__ void st_state(uint32_t *p, uint32_t v)
 }
 
 // Sum of the digit's counts over the tiles before `tile` (state: the digit's
-// column, one word per tile at a stride of RBINS).
-__device__ uint32_t look_back(const uint32_t *state, uint32_t tile, uint32_t agg_tag,
-                              uint32_t *status)
+// column, one word per tile at a stride of RBINS).  count(t): the digit's count
+// in tile t from its keys, for the tiles that `polls` polls found not ready.
+template <class Count>
+__device__ __forceinline__ uint32_t look_back(const uint32_t *state, uint32_t tile,
+                                              uint32_t agg_tag, int polls, Count count)
 {
     uint32_t sum = 0;
-    int spins = 0;
     for (int64_t t = (int64_t)tile - 1; t >= 0;) {
         // four predecessors at a time
         uint32_t v[4];
@@ -631,9 +634,9 @@ __device__ uint32_t look_back(const uint32_t *state, uint32_t tile, uint32_t agg
             ++used;
         }
         t -= used;
-        if (used == 0 && ++spins > SWEEP_SPINS) {
-            if (status) atomicOr(status, ST_SORT_STALL);
-            return sum;
+        if (used == 0) {
+            if (polls > 0) --polls;
+            else sum += count(t--); // waited long enough
         }
     }
     return sum;
@@ -644,7 +647,7 @@ __global__ void __launch_bounds__(SORT_THREADS, 3)
 sweep_pass_kernel(const uint32_t *__restrict__ keys_in, const uint32_t *__restrict__ vals_in,
                   uint32_t *__restrict__ keys_out, uint32_t *__restrict__ vals_out,
                   const uint32_t *n_dev, int64_t cap, uint32_t key_lo, uint32_t key_max, int shift,
-                  int width, int pass, uint32_t *head, bool index_vals, uint32_t *status)
+                  int width, int pass, uint32_t *head, bool index_vals, int polls)
 {
     constexpr int TILE = SORT_THREADS * ITEMS;
     __shared__ __align__(16) PassSmem<ITEMS> S;
@@ -691,7 +694,13 @@ sweep_pass_kernel(const uint32_t *__restrict__ keys_in, const uint32_t *__restri
     for (int dd = threadIdx.x; dd < bins; dd += SORT_THREADS) {
         uint32_t before = 0;
         if (tile > 0) {
-            before = look_back(states + dd, tile, agg, status);
+            before = look_back(states + dd, tile, agg, polls, [&](int64_t t) {
+                uint32_t c = 0; // tiles before another are full
+#pragma unroll 1
+                for (int64_t i = t * TILE; i < (t + 1) * TILE; ++i)
+                    c += digit_of(keys_in[i], key_lo, key_max, shift, (1u << width) - 1u) == (uint32_t)dd;
+                return c;
+            });
             st_state(states + (size_t)tile * RBINS + dd, (before + S.tot[dd]) | ((agg + 1u) << 28));
         }
         S.gbase[dd] = head[pass * RBINS + dd] + before - S.gbase[dd];
@@ -958,12 +967,12 @@ static_assert(SWEEP_MOST <= (int64_t)SWEEP_COUNT, "a state word holds the counts
 template <int ITEMS>
 void sweep_pass(const uint32_t *keys, const uint32_t *vals, uint32_t *keys_alt, uint32_t *vals_alt,
                 const uint32_t *n_dev, int64_t cap, const SweepDigits &dg, int pass, uint32_t *head,
-                bool index_vals, uint32_t *status, cudaStream_t s)
+                bool index_vals, int polls, cudaStream_t s)
 {
     const int64_t tile = SORT_THREADS * ITEMS;
     sweep_pass_kernel<ITEMS><<<(unsigned)((cap + tile - 1) / tile), SORT_THREADS, 0, s>>>(
         keys, vals, keys_alt, vals_alt, n_dev, cap, dg.key_lo, dg.key_max, dg.shift[pass],
-        dg.width[pass], pass, head, index_vals, status);
+        dg.width[pass], pass, head, index_vals, polls);
 }
 
 size_t three_kernel_temp_bytes(int64_t cap)
@@ -994,7 +1003,7 @@ int radix_passes(int key_bits)
 void radix_sort_pairs(uint32_t *&keys, uint32_t *&vals, uint32_t *&keys_alt, uint32_t *&vals_alt,
                       const uint32_t *n_dev, int64_t cap, int key_bits, void *temp,
                       cudaStream_t s, uint32_t key_lo, uint32_t key_max, bool index_vals,
-                      int bit_lo, uint32_t *status, bool least_temp)
+                      int bit_lo, bool least_temp, int polls)
 {
     if (cap <= 0) return;
     if (key_bits <= 0) {
@@ -1026,7 +1035,7 @@ void radix_sort_pairs(uint32_t *&keys, uint32_t *&vals, uint32_t *&keys_alt, uin
         sweep_hist_kernel<<<(unsigned)hb, SORT_THREADS, 0, s>>>(keys, n_dev, cap, dg, head);
         for (int p = 0; p < passes; ++p) {
             auto f = sweep_items(cap) == 16 ? sweep_pass<16> : sweep_pass<4>;
-            f(keys, vals, keys_alt, vals_alt, n_dev, cap, dg, p, head, index_vals && p == 0, status,
+            f(keys, vals, keys_alt, vals_alt, n_dev, cap, dg, p, head, index_vals && p == 0, polls,
               s);
             dg.key_lo = 0; // the keys written are the reduced ones
             swap();

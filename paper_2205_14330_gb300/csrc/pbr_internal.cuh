@@ -11,7 +11,6 @@ enum : uint32_t {
     ST_PAIR_OVERFLOW = 1u << 0,  // more (tile, point-view) pairs than capacity
     ST_COUNT_OVERFLOW = 1u << 1, // a 32-bit count or index would overflow
     ST_BAD_RANGE = 1u << 2,      // inconsistent tile range
-    ST_SORT_STALL = 1u << 4,     // a sort's wait ran out
 };
 
 // One view of the batch: camera of Sec. 3.1 Eq. 1 plus its place in the
@@ -220,16 +219,18 @@ void launch_exclusive_scan(const uint32_t *in, uint32_t *out, int64_t n,
 // passes.  index_vals: the input values are not read; value i is taken to
 // be i.  bit_lo > 0 needs key_lo = 0 and key_max = 0xffffffff.
 // temp: radix_temp_bytes(cap), or radix_temp_bytes_least(cap) with least_temp
-// (slower passes that need no more).  status: device status word (may be
-// NULL).
+// (slower passes that need no more).  polls: how often a block of the faster
+// passes looks for the counts of the blocks before it (a second or more) before
+// it counts their keys itself.
+constexpr int SORT_POLLS = 1 << 22;
 size_t radix_temp_bytes(int64_t cap);
 size_t radix_temp_bytes_least(int64_t cap);
 int radix_passes(int key_bits);
 void radix_sort_pairs(uint32_t *&keys, uint32_t *&vals, uint32_t *&keys_alt, uint32_t *&vals_alt,
                       const uint32_t *n_dev, int64_t cap, int key_bits, void *temp,
                       cudaStream_t s, uint32_t key_lo = 0, uint32_t key_max = 0xffffffffu,
-                      bool index_vals = false, int bit_lo = 0, uint32_t *status = nullptr,
-                      bool least_temp = false);
+                      bool index_vals = false, int bit_lo = 0, bool least_temp = false,
+                      int polls = SORT_POLLS);
 // Scratch of launch_emit_pairs (depth-ordered counts, offsets, scan).
 size_t emit_temp_bytes(int64_t cap_vis);
 // Emits (tile, pv) pairs in depth order: gathers the tile counts in depth
