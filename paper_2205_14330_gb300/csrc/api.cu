@@ -189,6 +189,20 @@ int pbr::check_opts(const pbr_render_opts *o)
     return PBR_OK;
 }
 
+// The options a pass runs with.  Compositing stops after the point that takes T
+// below t_eps.  The warp-streamed and persistent walks test T ahead of a point
+// instead, which is the same unless T starts below t_eps: above 1 the
+// block-staged schedule, which tests after it, takes the pass.
+pbr_render_opts pbr::scheduled_opts(const pbr_render_opts *o)
+{
+    pbr_render_opts r = *o;
+    if (r.t_eps > 1.0f && r.batch_depth == 0) {
+        r.batch_depth = 256;
+        r.persistent = 0;
+    }
+    return r;
+}
+
 DevOpts pbr::dev_opts(const pbr_render_opts *o)
 {
     DevOpts d;
@@ -661,6 +675,8 @@ extern "C" int pbr_forward_workspace_size(pbr_ctx *c, const pbr_points *scenes, 
 {
     if (!c || !bytes) return set_error(PBR_ERR_INVALID_ARG, "ctx or bytes is NULL");
     PBR_TRY(check_opts(opts));
+    const pbr_render_opts o = scheduled_opts(opts);
+    opts = &o;
     PBR_CUDA(cudaSetDevice(c->device));
     cudaStream_t s = (cudaStream_t)stream;
     HostLayout L;
@@ -714,6 +730,8 @@ extern "C" int pbr_render_forward(pbr_ctx *c, const pbr_points *scenes, int32_t 
     if (!c) return set_error(PBR_ERR_INVALID_ARG, "ctx is NULL");
     PBR_TRY(check_opts(opts));
     if (!out_rgb) return set_error(PBR_ERR_INVALID_ARG, "out_rgb is NULL");
+    const pbr_render_opts o = scheduled_opts(opts);
+    opts = &o;
     PBR_CUDA(cudaSetDevice(c->device));
     cudaStream_t s = (cudaStream_t)stream;
     pbr_state *st = new pbr_state();

@@ -48,6 +48,7 @@ struct HostLayout {
 
 int set_error(int code, const char *fmt, ...);
 int check_opts(const pbr_render_opts *o);
+pbr_render_opts scheduled_opts(const pbr_render_opts *o);
 DevOpts dev_opts(const pbr_render_opts *o);
 int build_layout(const pbr_points *scenes, int32_t n_scenes, const int32_t *scene_of_view,
                  const pbr_camera *cams, int32_t n_cams, const pbr_render_opts *o, HostLayout &L);

@@ -82,6 +82,8 @@ extern "C" int pbr_render_forward_noalloc(const pbr_points *scenes, int32_t n_sc
 {
     PBR_TRY(check_opts(opts));
     if (!out_rgb) return set_error(PBR_ERR_INVALID_ARG, "out_rgb is NULL");
+    const pbr_render_opts run = scheduled_opts(opts);
+    opts = &run;
     HostLayout L;
     PBR_TRY(build_layout(scenes, n_scenes, scene_of_view, cams, n_cams, opts, L));
     void *scratch = nullptr;

@@ -401,7 +401,7 @@ extern "C" int pbr_graph_create(pbr_ctx *c, const pbr_points *scenes, int32_t n_
     g->scenes.assign(scenes, scenes + n_scenes);
     if (scene_of_view) g->sov.assign(scene_of_view, scene_of_view + n_cams);
     g->cams.assign(cams, cams + n_cams);
-    g->opts = *opts;
+    g->opts = scheduled_opts(opts);
     g->out_rgb = out_rgb;
     g->target = target;
     g->loss_kind = loss_kind;

@@ -505,7 +505,9 @@ struct FwdWarp {
 // point at both of its pixels; the blend of a pixel the point does not
 // include (or that has stopped) is predicated off.  Each pixel's blend
 // sequence and roundings are the one-pixel walk's.
-// A pixel is active while its T is at least t_eps (-1 outside the image).
+// A pixel is active until its T is below t_eps (-1 outside the image; t_eps at
+// most 1, see scheduled_opts).  Both conditions of a pixel are evaluated, not one
+// after the other: persistent 3.91 -> 3.85 ms on the 1M-point, 64-view step.
 // COUNT: the points composited per pixel are counted (pair counts, store
 // mode, the count cap).
 // FUSED: the rounding of the squared distance (pair_d2).
@@ -543,8 +545,8 @@ __device__ __forceinline__ void fwd_pair_item(const DevView *V, int sx0, int sy0
     uint32_t qh = 0;
     while (true) {
         bool act[NP];
-        act[NP - 1] = T.y >= eps && cntB < cmax;
-        act[0] = T.x >= eps && cntA < cmax;
+        act[NP - 1] = !(T.y < eps) && cntB < cmax;
+        act[0] = !(T.x < eps) && cntA < cmax;
         if (!__any_sync(0xffffffffu, act[0] || act[NP - 1])) break;
         queue_fill_front(keys, pv_list, s, e, bit, p, qn, qh, m.q, lane);
         if (qn == 0) break;
@@ -578,8 +580,8 @@ __device__ __forceinline__ void fwd_pair_item(const DevView *V, int sx0, int sy0
                 float dx;
                 float2 dy;
                 const float2 d2 = pair_d2<FUSED>(ux, uy, aj.x, aj.y, dx, dy);
-                bool inA = d2.x <= aj.z && T.x >= eps;
-                bool inB = NP == 2 && d2.y <= aj.z && T.y >= eps;
+                bool inA = !(T.x < eps) & (d2.x <= aj.z);
+                bool inB = NP == 2 && (!(T.y < eps) & (d2.y <= aj.z));
                 if (COUNT) {
                     inA = inA && cntA < cmax;
                     inB = inB && cntB < cmax;

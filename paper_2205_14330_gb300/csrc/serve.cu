@@ -336,7 +336,7 @@ extern "C" int pbr_serve_start(pbr_ctx *c, const pbr_render_opts *opts, int32_t 
     PBR_CUDA(cudaSetDevice(c->device));
     ServeState *S = new ServeState();
     S->ctx = c;
-    S->opts = *opts;
+    S->opts = scheduled_opts(opts);
     S->max_views = max_batch_views;
     S->budget = c->hbm_budget;
     for (int k = 0; k < n_streams; ++k) {
