@@ -958,6 +958,24 @@ extern "C" int pbr_test_sort_pairs(uint32_t *keys, uint32_t *vals, int64_t n, in
     return PBR_OK;
 }
 
+// For the tests (not in the header; host only): whether the compositing warps of
+// a batch with these counts take whole blocks in the forward (two[0]) and the
+// backward (two[1]).  store: with the stored transmittance list.
+extern "C" int pbr_test_raster_lanes(const pbr_points *scenes, int32_t n_scenes,
+                                     const int32_t *scene_of_view, const pbr_camera *cams,
+                                     int32_t n_cams, const pbr_render_opts *opts, int32_t store,
+                                     int64_t n_vis, int64_t n_pairs, int32_t two[2])
+{
+    PBR_TRY(check_opts(opts));
+    HostLayout L;
+    PBR_TRY(build_layout(scenes, n_scenes, scene_of_view, cams, n_cams, opts, L));
+    const RasterLanes r = raster_lanes(L, dev_opts(opts), n_vis, n_pairs,
+                                       opts->persistent && opts->batch_depth == 0, store != 0);
+    two[0] = r.fwd_two;
+    two[1] = r.bwd_two;
+    return PBR_OK;
+}
+
 extern "C" int pbr_measure_alu_peaks(int device, double *fp32_flops, double *ex2_ops)
 {
     if (measure_alu_peaks(device, fp32_flops, ex2_ops) != 0)

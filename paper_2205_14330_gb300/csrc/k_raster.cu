@@ -1,7 +1,8 @@
 // Per-tile compositing of Sec. 3.2 and its adjoint.
 //
 // Per pixel centre u and listed point (records {px, py, rc^2, q'} {o, rgb}):
-//   d2 = (ux - px)^2 + (uy - py)^2            (fp32, round-to-nearest, no FMA)
+//   d2 = (ux - px)^2 + (uy - py)^2            (fp32, round-to-nearest; the persistent
+//                                             schedule fuses the second square)
 //   if d2 <= rc^2:                             (the cutoff of Sec. 3.2)
 //     alpha = min(alpha_max, o * 2^(q' d2))    (Eq. 5, q' = -log2(e)/(2 s^2))
 //     C += T alpha c ;  T *= (1 - alpha)       (Eqs. 6-7, front to back)
@@ -129,18 +130,22 @@ __device__ __forceinline__ PixelGeom pixel_geom(const Batch &b, uint32_t tile, i
 }
 
 // Culling test of one record against a rectangle of pixel centres: the
-// per-pixel cutoff test (the same fp32 round-to-nearest operations) applied
-// to the rectangle's pixel centre nearest the splat centre, floor(p) + 0.5
-// clamped into the rectangle per axis.  Rounding is monotone, so that
-// centre has the smallest fp32 squared distance of all the rectangle's
-// centres: the test keeps exactly the points some pixel of the rectangle
-// includes.
+// per-pixel cutoff test (the same fp32 operations, see pair_d2) applied to the
+// rectangle's pixel centre nearest the splat centre, floor(p) + 0.5 clamped
+// into the rectangle per axis.  Rounding is monotone, of products and sums as
+// of a fused multiply-add, so that centre has the smallest fp32 squared
+// distance of all the rectangle's centres: the test keeps exactly the points
+// some pixel of the rectangle includes.  Which points a pixel composites
+// therefore does not hang on the rectangle, and the forward and the backward
+// may cull with different ones.
+template <bool FUSED>
 __device__ __forceinline__ bool disc_meets_rect(const float4 a, const PixelGeom &g)
 {
     const float cx = fminf(fmaxf(floorf(a.x) + 0.5f, g.xl), g.xh);
     const float cy = fminf(fmaxf(floorf(a.y) + 0.5f, g.yl), g.yh);
     const float ex = __fsub_rn(cx, a.x), ey = __fsub_rn(cy, a.y);
-    return __fadd_rn(__fmul_rn(ex, ex), __fmul_rn(ey, ey)) <= a.z;
+    const float ex2 = __fmul_rn(ex, ex);
+    return (FUSED ? __fmaf_rn(ey, ey, ex2) : __fadd_rn(ex2, __fmul_rn(ey, ey))) <= a.z;
 }
 
 // The rectangle of the centres of the still active pixels of a warp that
@@ -560,7 +565,7 @@ __device__ __forceinline__ void fwd_pair_item(const DevView *V, int sx0, int sy0
         }
         // every lane takes part in the reductions, whatever its entry
         const PixelGeom ar = active_rect_rows<NP>(g, act);
-        const bool hit = valid && disc_meets_rect(a, ar);
+        const bool hit = valid && disc_meets_rect<FUSED>(a, ar);
         const uint32_t hm = __ballot_sync(0xffffffffu, hit);
         const int nh = __popc(hm);
         // the slots behind the hits are filled with points no pixel includes
@@ -880,7 +885,7 @@ __device__ __forceinline__ void bwd_pair_item(const DevView *V, int sx0, int sy0
         act[NP - 1] = p.LB > lowest;
         act[0] = p.LA > lowest;
         const PixelGeom ar = active_rect_rows<NP>(g, act);
-        const bool hit = lane < take && disc_meets_rect(ra, ar);
+        const bool hit = lane < take && disc_meets_rect<FUSED>(ra, ar);
         const uint32_t hm = __ballot_sync(0xffffffffu, hit);
         // amplitudes that may reach the clamp (a NaN counts as one)
         const bool clamp = __any_sync(0xffffffffu, hit && !(rc.x < o.alpha_max));
@@ -1141,7 +1146,7 @@ __device__ __forceinline__ int warp_cull(const float4 *s_a, int nb, const PixelG
     const uint32_t lt = lanemask_lt_r();
     for (int k0 = 0; k0 < nb; k0 += 32) {
         const int k = k0 + lane;
-        const bool hit = k < nb && disc_meets_rect(s_a[k], g);
+        const bool hit = k < nb && disc_meets_rect<false>(s_a[k], g);
         const uint32_t m = __ballot_sync(0xffffffffu, hit);
         if (hit) list[cnt + __popc(m & lt)] = (uint16_t)k;
         cnt += __popc(m);
