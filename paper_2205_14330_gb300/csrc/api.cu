@@ -538,10 +538,12 @@ int pbr::forward_eager(pbr_ctx *c, pbr_state *st, float *out_rgb, cudaStream_t s
         kept.place(st->mem[0]);
     }
     // the counters' first values (the smallest depth bits: all ones) and the
-    // tables, in one copy
+    // tables, in one copy (from memory that outlives it: a copy from pageable
+    // memory may run after the call)
+    std::vector<char> up;
     {
         char *first = (char *)st->counters;
-        std::vector<char> up((char *)st->rec - first, 0);
+        up.resize((size_t)((char *)st->rec - first), 0);
         std::memset(up.data() + 48, 0xff, 4);
         auto put = [&](const void *dst, const void *src, size_t bytes) {
             if (bytes) std::memcpy(up.data() + ((const char *)dst - first), src, bytes);
@@ -917,7 +919,7 @@ extern "C" int pbr_image_loss_tv(const pbr_camera *cams, int32_t n_cams, const f
     TempBufs tmp(s);
     DevView *d = nullptr;
     PBR_TRY(tmp.alloc(&d, sizeof(DevView) * n_cams));
-    PBR_CUDA(cudaMemcpyAsync(d, views.data(), sizeof(DevView) * n_cams, cudaMemcpyHostToDevice, s));
+    upload_small(d, views.data(), sizeof(DevView) * n_cams, s);
     launch_loss_tv(d, n_cams, max_pix, loss_kind, lambda_tv, pred, target, grad, loss_dev, s);
     PBR_CUDA(cudaGetLastError());
     return PBR_OK;

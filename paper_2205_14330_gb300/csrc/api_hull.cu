@@ -37,8 +37,7 @@ int upload_views(TempBufs &tb, const pbr_camera *cams, int32_t n_cams, float z_n
         base += (int64_t)c.width * c.height;
     }
     PBR_TRY(tb.alloc(d_views, sizeof(HullView) * n_cams));
-    PBR_CUDA(cudaMemcpyAsync(*d_views, v.data(), sizeof(HullView) * n_cams,
-                             cudaMemcpyHostToDevice, s));
+    upload_small(*d_views, v.data(), sizeof(HullView) * n_cams, s);
     return PBR_OK;
 }
 

@@ -1,5 +1,8 @@
 // Image loss of the training step (Sec. 3.3, Eq. 8 data term; L1 variant)
-// and the ALU microbenchmarks that give the raster kernels their roofline.
+// and the ALU microbenchmarks that give the raster kernels their roofline; small
+// uploads.
+#include <cstring>
+
 #include "pbr_internal.cuh"
 
 namespace pbr {
@@ -106,7 +109,33 @@ __global__ void ex2_peak_kernel(float *out, int iters)
     if (s == 1234.5f) out[0] = s;
 }
 
+// A piece of a host table in the launch's parameters, which the launch copies:
+// an asynchronous copy from pageable memory may read it after the call returns
+// (the GPU can reach the host's page tables), when its owner is gone.
+constexpr int UPLOAD_WORDS = 960;
+struct UploadPiece {
+    uint32_t w[UPLOAD_WORDS];
+};
+
+__global__ void __launch_bounds__(256)
+upload_kernel(uint32_t *__restrict__ dst, int n, const __grid_constant__ UploadPiece piece)
+{
+    for (int i = threadIdx.x; i < n; i += 256) dst[i] = piece.w[i];
+}
+
 } // namespace
+
+void upload_small(void *dst, const void *src, size_t bytes, cudaStream_t s)
+{
+    const size_t words = bytes / sizeof(uint32_t);
+    for (size_t at = 0; at < words; at += UPLOAD_WORDS) {
+        UploadPiece piece;
+        const int n = (int)(words - at < UPLOAD_WORDS ? words - at : UPLOAD_WORDS);
+        std::memcpy(piece.w, (const uint32_t *)src + at, sizeof(uint32_t) * n);
+        upload_kernel<<<1, 256, 0, s>>>((uint32_t *)dst + at, n, piece);
+        count_launches(1);
+    }
+}
 
 void launch_image_loss(int kind, const float *pred, const float *target, int64_t n, float *grad,
                        double *loss, cudaStream_t s)

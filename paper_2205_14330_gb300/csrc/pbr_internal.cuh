@@ -415,6 +415,9 @@ void launch_optimizer(const OptParams &prm, const OptState *dev, int group, floa
 void launch_step_counter(OptState *dev, cudaStream_t s);
 
 // ---- misc (k_misc.cu)
+// Copies a small host table (whole 32-bit words) to the device; the host memory
+// may be freed as soon as the call returns.
+void upload_small(void *dst, const void *src, size_t bytes, cudaStream_t s);
 void launch_image_loss(int kind, const float *pred, const float *target, int64_t n, float *grad,
                        double *loss, cudaStream_t s);
 int measure_alu_peaks(int device, double *fp32_flops, double *ex2_ops);
