@@ -441,13 +441,12 @@ namespace {
 // and frees cost its host path more than its kernels take on small views
 // (one 1024 x 768 view of 45k points: 151 -> 144 us a call).
 struct Arena {
-    size_t size = 0, bytes = 0; // allocated, asked for
+    size_t size = 0; // bytes of the one allocation
     std::vector<std::pair<void **, size_t>> parts;
     template <class T> void add(T **p, size_t want)
     {
         want = std::max<size_t>(want, 16);
         parts.emplace_back((void **)p, size);
-        bytes += want;
         size += (want + 255) & ~(size_t)255;
     }
     void place(void *base)
@@ -655,9 +654,8 @@ int pbr::forward_eager(pbr_ctx *c, pbr_state *st, float *out_rgb, cudaStream_t s
     return PBR_OK;
 }
 
-// The bytes of forward_eager's buffers (before their rounding to 256), all
-// alive at its end: the state's, the call's temporaries and, in store mode,
-// the transmittance list.
+// The bytes forward_eager allocates, all alive at its end: the state's
+// buffers, the call's temporaries and, in store mode, the transmittance list.
 size_t pbr::forward_bytes(const HostLayout &L, int64_t n_vis, int64_t n_pairs,
                           const pbr_render_opts *o, int32_t store_depth)
 {
@@ -666,7 +664,7 @@ size_t pbr::forward_bytes(const HostLayout &L, int64_t n_vis, int64_t n_pairs,
     Arena a;
     plan_points(L, &st, t, a, a);
     plan_lists(L, n_vis, n_pairs, o->persistent && o->batch_depth == 0, store_depth, &st, t, a, a);
-    return a.bytes;
+    return a.size;
 }
 
 extern "C" int pbr_forward_workspace_size(pbr_ctx *c, const pbr_points *scenes, int32_t n_scenes,
