@@ -56,7 +56,7 @@ struct Request {
     double t_arrival = 0, t_done = 0;
     int32_t status = PBR_OK;
     bool done = false;
-    size_t bytes = 0, bound = 0; // reserved; admission_bytes
+    size_t bytes = 0; // reserved
 };
 
 struct InFlight {
@@ -185,16 +185,10 @@ bool ServeState::launch_one()
             break;
         }
     if (slot < 0 || queue.empty()) return false;
-    // Requests share a batch while their host bounds fit the budget together
-    // (what the batch reserves may be less: reserve_bytes).  Going by the
-    // reservations alone, a budget of one bound and a half put one or two
-    // requests into a batch depending on whether the batch before had finished
-    // when its event was polled.
     std::vector<uint64_t> ids;
-    size_t bytes = 0, bounds = 0;
+    size_t bytes = 0;
     while (!queue.empty() && (int)ids.size() < max_views) {
         Request &r = reqs[queue.front()];
-        if (!ids.empty() && (r.bound > budget || bounds > budget - r.bound)) break;
         if (in_use + bytes + r.bytes > budget) {
             if (ids.empty() && inflight.empty()) { // can never fit: reject
                 r.done = true;
@@ -208,7 +202,6 @@ bool ServeState::launch_one()
             break; // wait for memory to free up
         }
         bytes += r.bytes;
-        bounds += r.bound;
         ids.push_back(queue.front());
         queue.pop_front();
     }
@@ -459,6 +452,10 @@ extern "C" int pbr_evict_scene(pbr_ctx *c, int32_t scene_id)
     return PBR_OK;
 }
 
+// Requests below this reserve their host bound whatever the budget, if it fits
+// at all: a counting pass costs a device round trip and would free less.
+constexpr size_t SMALL_REQUEST = (size_t)1 << 20;
+
 // The bytes a request reserves: the host bound of admission_bytes, or, when
 // that bound would take more than 1/64 of the budget (a camera close to or
 // inside the scene's bounding box makes it loose), the exact workspace of
@@ -469,7 +466,7 @@ static int reserve_bytes(pbr_ctx *c, ServeState *S, const pbr_points &pts, size_
                          size_t budget, const pbr_camera &cam, size_t *bytes)
 {
     *bytes = bound;
-    if (bound <= budget / 64) return PBR_OK;
+    if (bound <= std::max(budget / 64, std::min(budget, SMALL_REQUEST))) return PBR_OK;
     std::lock_guard<std::mutex> ga(S->admit_mu);
     size_t exact = 0;
     PBR_TRY(pbr_forward_workspace_size(c, &pts, 1, nullptr, &cam, 1, &S->opts, 0, &exact, nullptr,
@@ -513,7 +510,6 @@ extern "C" int pbr_submit_request(pbr_ctx *c, int32_t scene_id, const pbr_camera
         r.out = out_rgb_device;
         r.t_arrival = arrival_time > 0.0 ? arrival_time : now_s();
         r.bytes = bytes;
-        r.bound = bound;
         S->reqs[r.id] = r;
         S->queue.push_back(r.id);
         ++S->submitted;
