@@ -7,7 +7,10 @@
 // with the nearest points (from the exact neighbour search) held fixed.
 // The distances entering CD are taken in fp64 from the fp32 positions and
 // summed per block, one fp64 atomic per block; the second gradient term is
-// scattered with fp32 atomics.
+// scattered with fp32 atomics.  A point with no nearest one (nn -1: it is at no
+// finite distance to any) makes CD, and its own gradient, NaN.
+#include <cmath>
+
 #include "pbr_internal.cuh"
 
 namespace pbr {
@@ -39,7 +42,7 @@ chamfer_21_kernel(const float *__restrict__ p1, const float *__restrict__ p2, in
         const int64_t i = nn21[j];
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            const double d = (double)p2[3 * j + a] - (double)p1[3 * i + a];
+            const double d = i >= 0 ? (double)p2[3 * j + a] - (double)p1[3 * i + a] : (double)NAN;
             acc += d * d;
             if (grad2) grad2[3 * j + a] = (float)(2.0 * inv_n2 * d);
         }
@@ -57,6 +60,10 @@ chamfer_12_kernel(const float *__restrict__ p1, int64_t n1, const float *__restr
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n1;
          i += (int64_t)gridDim.x * blockDim.x) {
         const int64_t j = nn12[i];
+        if (j < 0) {
+            acc = (double)NAN;
+            continue;
+        }
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
             const double d = (double)p2[3 * j + a] - (double)p1[3 * i + a];

@@ -903,14 +903,18 @@ generate_kernel(const int32_t *__restrict__ nbr, int64_t n, int k, int keff, Par
 {
     const int lane = threadIdx.x & 31;
     const int nattr = 5 + in.nsh;
-    const float cnt = (float)keff;
     const int a0 = a_begin + lane, a1 = a0 + 32;
     for (int64_t q = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; q < n;
          q += ((int64_t)gridDim.x * blockDim.x) >> 5) {
         const int32_t *row = nbr + q * k;
         if (a0 >= nattr) continue;
+        // a point at no finite distance to enough others has fewer neighbours
+        // (rows end in -1): the mean of those there are, NaN without any
+        int have = keff;
+        while (have > 0 && __ldg(row + have - 1) < 0) --have;
+        const float cnt = (float)have;
         KahanSum s0, s1;
-        sum_points(in, [&](int m) { return (uint32_t)__ldg(row + m); }, keff, a0, a1, a1 < nattr, s0,
+        sum_points(in, [&](int m) { return (uint32_t)__ldg(row + m); }, have, a0, a1, a1 < nattr, s0,
                    s1);
         out.put(out_base + q, a0, __fdiv_rn(s0.s, cnt));
         if (a1 < nattr) out.put(out_base + q, a1, __fdiv_rn(s1.s, cnt));
