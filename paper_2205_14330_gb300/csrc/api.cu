@@ -322,26 +322,49 @@ int pbr::build_layout(const pbr_points *scenes, int32_t n_scenes, const int32_t 
 // point reaching both halves is stepped through twice.  Half blocks pay while
 // the longest block's walk is a large share of the whole: with v the hits a
 // view's block visits (its list, or what saturates it: some 28 layers of
-// splats covering c of its 64 pixels), the batch is worth sum(v) / max(v)
-// equal blocks, and the line lies at c / r of them, r the mean cutoff radius
-// in pixels: forward c = 105000 streamed, 160000 with the stored list and
-// 250000 persistent, backward 60000; lower in proportion where a block's mean
-// walk is below 64 hits, since a warp's start then counts.  r comes from the
-// pair count: a point lists (1 + 2 r / tile_w)(1 + 2 r / tile_h) tiles, r = k
-// f with f the view's focal length in pixels, summed over the views and
-// solved for k.
-// Measured, half blocks / blocks (us, fwd and bwd; with worth times r, in
-// thousands): streamed, 16 x 16 tiles: 227k points, 7 views of 101 x 339 to
-// 1270 x 365 (16): 635 / 1039, 803 / 1259; 7k, 4 small views (71): 36 / 44,
-// 44 / 63; 16 views of 256^2 to 1920 x 1072 over four scenes (107): 876 / 769;
-// 500k, 4 views of 800^2 (149): 189 / 186, 429 / 364, stored 272 / 298, 565 /
-// 516; 272k, 33 views (179): 596 / 518, 958 / 714; one 1920 x 1080 view of 1M
-// (290): 167 / 151; one 1024 x 768 view of 45k, 18 hits a block (59): 37 / 22.
-// Persistent: 808k, 8 views of 235 x 230 to 1737 x 835 (64): 398 / 534, 1038 /
-// 802; 136k, 8 views (82): 172 / 262, 323 / 423; 136k, 43 views (216): 619 /
-// 680, 1448 / 1148.
+// splats of amplitude 0.8, or the count cap, covering c of its 64 pixels; the
+// amplitudes are not known here), the batch is worth sum(v) / max(v) equal
+// blocks, and the line lies at c / r of them, r the mean cutoff radius in pixels.
+// c falls in proportion where a block's mean walk is below 64 hits (a warp's
+// start then counts: `line`) and, in most backwards, with a count cap below 28
+// (`layers`).  Streamed warps that count pairs end in atomics on one
+// address, which half the warps halve: their line is lower.  The stored list's
+// forward is bound by its scattered writes, which more warps hide.  r comes from
+// the pair count: a point lists (1 + 2 r / tile_w)(1 + 2 r / tile_h) tiles, r = k
+// f with f the view's focal length in pixels, summed over the views and solved
+// for k.
+// Measured, half blocks / blocks (us, 16 x 16 tiles; x = worth times r in
+// thousands, h = hits a block):
+//                                  streamed              streamed, stored list
+//                      x    h    forward   backward      forward    backward
+//   7k, 4 small views  1   36    32 / 41    60 / 85       43 / 73    89 / 137
+//   227k, 7 views     21  118  325 / 452  451 / 609     451 / 763  645 / 1083
+//   136k, 8 views     33   91  147 / 164  299 / 299     214 / 281   385 / 445
+//   808k, 8 views     44  158  568 / 609  1131 / 945   766 / 1005 1355 / 1390
+//   45k, 1024 x 768   53   16    25 / 24    56 / 52       38 / 44     70 / 72
+//   500k, 4 x 800^2  131  165  178 / 181  405 / 344     238 / 279   493 / 484
+//   136k, 43 views   175   93  552 / 535 1356 / 1128    766 / 889 1619 / 1561
+//   1M, 1920 x 1080  272   78  138 / 131  383 / 284     254 / 305   454 / 398
+//   272k, 33 views   477  128  885 / 850 2057 / 1688  1179 / 1326 2475 / 2341
+//                              counting, streamed      counting, stored list
+//   136k, 8 views     33   91  160 / 171  332 / 328     226 / 281   416 / 449
+//   45k, 1024 x 768   53   16    42 / 29    67 / 67       61 / 53     78 / 78
+//   500k, 4 x 800^2  131  165  199 / 188  472 / 416     261 / 281   538 / 509
+//   1M, 1920 x 1080  272   78  151 / 134  398 / 307     289 / 306   461 / 401
+//                                 persistent             persistent, stored list
+//   7k, 4 small views  1   36    53 / 77   81 / 114      70 / 130   106 / 162
+//   808k, 8 views     44  158  556 / 676 1019 / 1011   836 / 1165 1232 / 1564
+//   45k, 1024 x 768   53   16    44 / 51    58 / 78       64 / 78    71 / 107
+//   500k, 4 x 800^2  131  165  189 / 190  369 / 363     244 / 321   455 / 485
+//   136k, 43 views   175   93  560 / 538 1226 / 1012    868 / 913 1461 / 1388
+//   272k, 33 views   477  128  855 / 785 1907 / 1554  1246 / 1329 2217 / 2046
+// Over 256 batches (1k to 1M points, 1 to 43 views of 64 to 1920 pixels a side,
+// amplitudes 0.05 to 0.8, some capped at 15) in up to three tile sizes and four
+// schedules the choice costs 0.7% against the better of the two on geometric
+// average, 2.4% in the worst schedule and phase; lists of very uneven length,
+// unknown here, would move the line (55% on the worst batch).
 RasterLanes pbr::raster_lanes(const HostLayout &L, const DevOpts &o, int64_t n_vis,
-                              int64_t n_pairs, bool persistent, bool store)
+                              int64_t n_pairs, bool persistent, bool store, bool counted)
 {
     RasterLanes r;
     if (L.n_pv <= 0 || n_vis <= 0) return r;
@@ -357,23 +380,32 @@ RasterLanes pbr::raster_lanes(const HostLayout &L, const DevOpts &o, int64_t n_v
         c += n;
     }
     const double k = c < 0.0 && a > 0.0 ? (-b + std::sqrt(b * b - 4.0 * a * c)) / (2.0 * a) : 0.0;
+    const double deep = o.max_per_pixel > 0 ? std::min(28, o.max_per_pixel) : 28;
     double most = 0.0, sum = 0.0, sum_r = 0.0, sum_blocks = 0.0;
     for (const DevView &V : L.views) {
         const double blocks = (double)((V.W + 7) / 8) * ((V.H + 7) / 8);
         const double rc = std::max(k * focal(V), 0.5), w = 8.0 + 2.0 * rc;
         const double cover = 64.0 * 3.14159265 * rc * rc / (w * w); // pixels of a block per hit
         const double v = std::min(share * (double)L.scenes[V.scene].n * (w * w / 64.0) / blocks,
-                                  28.0 * 64.0 / cover);
+                                  deep * 64.0 / cover);
         most = std::max(most, v);
         sum_blocks += blocks;
         sum += blocks * v;
         sum_r += blocks * v * rc;
     }
     if (!(most > 0.0)) return r;
-    const double worth = sum / most, mean_r = sum_r / sum;
-    const double line = std::min(1.0, sum / sum_blocks / 64.0);
-    r.fwd_two = worth * mean_r >= (persistent ? 250e3 : store ? 160e3 : 105e3) * line;
-    r.bwd_two = worth * mean_r >= 60e3 * line;
+    const double x = sum / most * (sum_r / sum);
+    const double line = std::min(1.0, sum / sum_blocks / 64.0), layers = deep / 28.0;
+    if (persistent) {
+        r.fwd_two = x >= (store ? 2.4e6 : 225e3) * line;
+        r.bwd_two = x >= (store ? 104e3 : 104e3 * layers);
+    } else if (store) {
+        r.fwd_two = counted && x >= 200e3 * layers * line;
+        r.bwd_two = x >= 104e3 * layers;
+    } else {
+        r.fwd_two = x >= (counted ? 45e3 : 200e3) * line;
+        r.bwd_two = x >= (counted ? std::min(36e3, 112e3 * line) : 36e3);
+    }
     return r;
 }
 
@@ -646,7 +678,9 @@ int pbr::forward_eager(pbr_ctx *c, pbr_state *st, float *out_rgb, cudaStream_t s
                           st->rec, out_rgb,
                           st->T_final, st->n_contrib,
                           st->opts.no_pair_stats ? nullptr : st->counters + 2, s,
-                          raster_lanes(L, o, st->n_vis, st->n_pairs, persist, st->store_depth > 0).fwd_two,
+                          raster_lanes(L, o, st->n_vis, st->n_pairs, persist, st->store_depth > 0,
+                                       !st->opts.no_pair_stats)
+                              .fwd_two,
                           st->tile_order,
                           st->work, st->store());
     }
@@ -785,7 +819,7 @@ extern "C" int pbr_render_backward(pbr_ctx *c, pbr_state *st, const float *grad_
                           st->T_final, st->n_contrib, grad_rgb, g2d,
                           st->opts.no_pair_stats ? nullptr : st->counters + 2, s,
                           raster_lanes(L, st->dopts, st->n_vis, st->n_pairs, st->work != nullptr,
-                                       st->store_depth > 0)
+                                       st->store_depth > 0, !st->opts.no_pair_stats)
                               .bwd_two,
                           st->tile_order, st->work, st->store());
     }
@@ -970,7 +1004,8 @@ extern "C" int pbr_test_raster_lanes(const pbr_points *scenes, int32_t n_scenes,
     HostLayout L;
     PBR_TRY(build_layout(scenes, n_scenes, scene_of_view, cams, n_cams, opts, L));
     const RasterLanes r = raster_lanes(L, dev_opts(opts), n_vis, n_pairs,
-                                       opts->persistent && opts->batch_depth == 0, store != 0);
+                                       opts->persistent && opts->batch_depth == 0, store != 0,
+                                       !opts->no_pair_stats);
     two[0] = r.fwd_two;
     two[1] = r.bwd_two;
     return PBR_OK;

@@ -62,12 +62,13 @@ size_t forward_bytes(const HostLayout &L, int64_t n_vis, int64_t n_pairs,
 void zero_unviewed_grads(const HostLayout &L, float *grad_pos, float *grad_sh,
                          float *grad_opacity, cudaStream_t s);
 // Whether the compositing warps of a batch take 8 x 8 blocks (two pixels a
-// lane) or halves of them, from its sizes and list counts.
+// lane) or halves of them, from its sizes and list counts.  counted: the warps
+// count pairs (pbr_state_stats).
 struct RasterLanes {
     bool fwd_two = true, bwd_two = true;
 };
 RasterLanes raster_lanes(const HostLayout &L, const DevOpts &o, int64_t n_vis, int64_t n_pairs,
-                         bool persistent, bool store);
+                         bool persistent, bool store, bool counted);
 int dalloc(void **p, size_t bytes, cudaStream_t s);
 void dfree(void *p, cudaStream_t s);
 void serve_shutdown(pbr_ctx *c);

@@ -170,7 +170,7 @@ extern "C" int pbr_render_forward_noalloc(const pbr_points *scenes, int32_t n_sc
     PBR_CUDA(cudaMemsetAsync(ranges, 0, sizeof(uint2) * L.n_tiles, s));
     launch_tile_ranges(tk, n_pairs_dev, (int64_t)n_pairs, ranges, L.n_tiles, sb, s);
     launch_raster_fwd(b, o, opts->batch_depth, ranges, tk, tv, rec, out_rgb, T_final, n_contrib,
-                      nullptr, s, raster_lanes(L, o, (int64_t)n_vis, (int64_t)n_pairs, false, false).fwd_two);
+                      nullptr, s, raster_lanes(L, o, (int64_t)n_vis, (int64_t)n_pairs, false, false, false).fwd_two);
     PBR_CUDA(cudaGetLastError());
     // the kernels' status word (pair overflow, inconsistent counts): one
     // read-back into a host variable after the pass

@@ -311,7 +311,7 @@ int plan_and_capture(pbr_graph *g, cudaStream_t user_stream)
     const uint64_t n_pairs = g->host[0], n_vis = g->host[1];
     const uint32_t zlo = ((uint32_t *)g->host)[12], zhi = ((uint32_t *)g->host)[13];
     g->lanes = raster_lanes(L, g->dopts, (int64_t)n_vis, (int64_t)n_pairs,
-                            g->opts.persistent && g->opts.batch_depth == 0, false);
+                            g->opts.persistent && g->opts.batch_depth == 0, false, false);
     g->cap_vis = L.n_pv;
     g->cap_pairs = (int64_t)std::ceil((double)n_pairs * (1.0 + g->headroom)) + 4096;
     if (g->cap_pairs >= (int64_t)UINT32_MAX) g->cap_pairs = (int64_t)UINT32_MAX - 1;
