@@ -540,6 +540,7 @@ def measure_workload(args, pbr, torch, R, sc, desc, dist, world, local, headline
     # ---- schedule: autotuned over tile size x compositing schedule
     tune = None
     if args.autotune:
+        opts.bwd_mode = 1  # the backward that captured graphs run
         opts, table = pbr.autotune(R, scene_list, cams, opts, scene_of_view=sov, backward=True,
                                    reps=2)
         tune = {f"{t[0]}x{t[1]}/{'staged-' + str(d) if d else ('persistent' if p else 'streamed')}":

@@ -290,8 +290,11 @@ int pbr_graph_destroy(pbr_graph *graph);
  * {warp-streamed, persistent warp-streamed, block-staged 128 / 256 / 512})
  * on this batch -- forward only (mode 0) or forward + backward (mode 1),
  * `reps` timed runs each -- and writes the fastest into *opts (tile_w,
- * tile_h, batch_depth, persistent).  The choice is cached in the context
- * per shape class (views, log2 pixels, log2 point-views, SH degrees, mode);
+ * tile_h, batch_depth, persistent).  The backward timed is the one that
+ * opts->bwd_mode asks for: captured graphs always recompute, so a schedule
+ * for one is chosen with bwd_mode 1.  The choice is cached in the context
+ * per shape class (views, log2 pixels, log2 point-views, SH degrees, mode;
+ * choices made with bwd_mode 1 apart, as mode 2 in the file);
  * a cached class returns at once unless ms_out is given.  ms_out (nullable,
  * 15 entries) receives the mean milliseconds per candidate in the order
  * above, *n_candidates the number timed.  Synchronises. */

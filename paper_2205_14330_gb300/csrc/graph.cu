@@ -559,7 +559,10 @@ extern "C" int pbr_graph_destroy(pbr_graph *g)
 // block-staged with 128 / 256 / 512 points per batch}.  Each candidate runs
 // the eager forward (and backward, mode 1) `reps` times after one warm-up;
 // the fastest is written into *opts and cached in the context under the
-// batch's shape class.
+// batch's shape class.  The backward is the one that opts->bwd_mode asks for;
+// the stored list moves the schedules' order (64 views of 1M points, ms: 29.3
+// 16 x 16 streamed, 30.0 16 x 32 persistent with it, 20.4 and 20.0 without), so a
+// choice made with recomputation, as captured graphs run, is a class of its own.
 extern "C" int pbr_autotune(pbr_ctx *c, const pbr_points *scenes, int32_t n_scenes,
                             const int32_t *scene_of_view, const pbr_camera *cams, int32_t n_cams,
                             pbr_render_opts *opts, int32_t mode, int32_t reps, double *ms_out,
@@ -569,11 +572,13 @@ extern "C" int pbr_autotune(pbr_ctx *c, const pbr_points *scenes, int32_t n_scen
     PBR_TRY(check_opts(opts));
     HostLayout L;
     PBR_TRY(build_layout(scenes, n_scenes, scene_of_view, cams, n_cams, opts, L));
-    // shape class: views, log2 pixels, log2 point-views, degrees
+    // shape class: views, log2 pixels, log2 point-views, degrees, mode (2: mode 1
+    // with recomputation asked for)
     int64_t key_deg = 0;
     for (int s = 0; s < n_scenes; ++s) key_deg = key_deg * 4 + scenes[s].sh_degree;
     const auto key = std::make_tuple((int64_t)n_cams, (int64_t)std::log2((double)L.n_pix + 1),
-                                     (int64_t)std::log2((double)L.n_pv + 1), key_deg, (int64_t)mode);
+                                     (int64_t)std::log2((double)L.n_pv + 1), key_deg,
+                                     (int64_t)(mode == 1 && opts->bwd_mode == 1 ? 2 : mode));
     {
         auto it = c->tuned.find(key);
         if (it != c->tuned.end() && !ms_out) {
@@ -614,7 +619,7 @@ extern "C" int pbr_autotune(pbr_ctx *c, const pbr_points *scenes, int32_t n_scen
             o.tile_h = t[1];
             o.batch_depth = sc[0];
             o.persistent = sc[1];
-            o.no_pair_stats = 1; // time the kernels the captured graphs run
+            o.no_pair_stats = 1; // as in captured graphs
             float total = 0.f;
             for (int r = 0; r <= reps && rc == PBR_OK; ++r) {
                 cudaEventRecord(e0, s);
@@ -768,7 +773,7 @@ extern "C" int pbr_autotune_load(pbr_ctx *c, const char *path, int32_t *n_loaded
         o.batch_depth = (int32_t)v[7];
         o.persistent = (int32_t)v[8];
         if (v[5] != o.tile_w || v[6] != o.tile_h || v[7] != o.batch_depth ||
-            (v[8] != 0 && v[8] != 1) || (v[4] != 0 && v[4] != 1) || check_opts(&o) != PBR_OK)
+            (v[8] != 0 && v[8] != 1) || v[4] < 0 || v[4] > 2 || check_opts(&o) != PBR_OK)
             return set_error(PBR_ERR_INVALID_ARG, "%s: entry %zu holds an invalid schedule", path,
                              entries.size());
         entries.push_back({std::make_tuple(v[0], v[1], v[2], v[3], v[4]),
