@@ -41,29 +41,6 @@ int upload_views(TempBufs &tb, const pbr_camera *cams, int32_t n_cams, float z_n
     return PBR_OK;
 }
 
-// Candidates of the next batch, with `done` of the n_target points found among
-// `drawn` candidates.  A batch costs a host synchronisation,
-// candidates beyond the last one taken cost their draws.  n_target candidates are
-// needed whatever is accepted: the first batch draws those and shows the share;
-// the next ones allow for it and for three standard deviations of its estimate (no
-// share seen: the largest batch).  A first batch for one in 32 accepted drew what
-// it did not use where the masks take more: 500k points, every candidate accepted,
-// 16 views: 1647 us, of batches of 4 M 519.
-constexpr int64_t HULL_BATCH = 1ll << 24, HULL_LEAST = 1ll << 16;
-
-int64_t hull_batch(int64_t n_target, int64_t done, int64_t drawn)
-{
-    double want = (double)n_target;
-    if (drawn > 0) {
-        if (done == 0) return HULL_BATCH;
-        const double missing = (double)(n_target - done);
-        want = missing * (double)drawn / (double)done *
-               (1.0 + 3.0 / std::sqrt((double)std::min(done, n_target - done)));
-    }
-    const int64_t c = want < (double)HULL_BATCH ? (int64_t)want : HULL_BATCH;
-    return std::max(HULL_LEAST, (c + HULL_BLOCK - 1) / HULL_BLOCK * HULL_BLOCK);
-}
-
 int read_u64(const unsigned long long *dev, unsigned long long *out, cudaStream_t s)
 {
     PBR_CUDA(cudaMemcpyAsync(out, dev, sizeof(*out), cudaMemcpyDeviceToHost, s));
@@ -155,15 +132,24 @@ extern "C" int pbr_visual_hull_init(pbr_ctx *ctx, const float lo[3], const float
     TempBufs tb(s);
     HullView *views;
     PBR_TRY(upload_views(tb, cams, n_cams, z_near, &views, s));
-    // batches of candidates in counter order; the first n_target accepted
+    // Batches of candidates in counter order; the first n_target accepted.
+    // A batch costs a host synchronisation, candidates beyond the last one
+    // taken cost their draws: the first batch allows for one candidate in 32
+    // accepted, the next ones for the share seen so far and a little more.
+    constexpr int64_t BATCH = 1ll << 24, LEAST = 1ll << 16;
+    auto sized = [&](double want) {
+        const int64_t c = want < (double)BATCH ? (int64_t)want : BATCH;
+        return std::max(LEAST, (c + HULL_BLOCK - 1) / HULL_BLOCK * HULL_BLOCK);
+    };
+    int64_t size = sized(32.0 * (double)n_target);
     uint32_t *bits, *counts;
     unsigned long long *result;
-    PBR_TRY(tb.alloc(&bits, (size_t)(HULL_BATCH / 8)));
-    PBR_TRY(tb.alloc(&counts, sizeof(uint32_t) * (HULL_BATCH / HULL_BLOCK)));
+    PBR_TRY(tb.alloc(&bits, (size_t)(BATCH / 8)));
+    PBR_TRY(tb.alloc(&counts, sizeof(uint32_t) * (BATCH / HULL_BLOCK)));
     PBR_TRY(tb.alloc(&result, 2 * sizeof(unsigned long long)));
     int64_t done = 0, drawn = 0;
     while (done < n_target && drawn < max_candidates) {
-        const int64_t cnt = std::min(hull_batch(n_target, done, drawn), max_candidates - drawn);
+        const int64_t cnt = std::min<int64_t>(size, max_candidates - drawn);
         const uint32_t need = (uint32_t)(n_target - done);
         launch_hull_batch(seed, (uint64_t)drawn, cnt, lo, ext, views, n_cams, masks, z_near, bits,
                           counts, need, out_pos, done, result, s);
@@ -176,6 +162,8 @@ extern "C" int pbr_visual_hull_init(pbr_ctx *ctx, const float lo[3], const float
         } else {
             drawn += cnt;
             done += (int64_t)got[0];
+            size = done > 0 ? sized(1.05 * (double)(n_target - done) * (double)drawn / (double)done)
+                            : BATCH;
         }
     }
     // SH of the kept points: standard normals
@@ -188,10 +176,4 @@ extern "C" int pbr_visual_hull_init(pbr_ctx *ctx, const float lo[3], const float
     PBR_CUDA(cudaGetLastError());
     PBR_CUDA(cudaStreamSynchronize(s));
     return PBR_OK;
-}
-
-// For the tests (not in the header; host only): see hull_batch.
-extern "C" int64_t pbr_test_hull_batch(int64_t n_target, int64_t done, int64_t drawn)
-{
-    return hull_batch(n_target, done, drawn);
 }

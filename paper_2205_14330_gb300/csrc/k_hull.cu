@@ -80,7 +80,7 @@ __device__ __forceinline__ void candidate(const HullBox &b, uint64_t j, float p[
         p[a] = __fadd_rn(__fmul_rn(b.ex[a], uniform24(splitmix64(b.seed, 3 * j + a))), b.lo[a]);
 }
 
-// Acceptance of HB candidates per block, as a bit each (candidate i
+// Acceptance of HULL_BLOCK candidates per block, as a bit each (candidate i
 // of the batch in bit i & 31 of word i / 32) and a count per block.
 // A warp of candidates runs until its last one fails, so testing every view
 // at once keeps a warp for all views while a few lanes live (196 us for 4 M
@@ -89,27 +89,23 @@ __device__ __forceinline__ void candidate(const HullBox &b, uint64_t j, float p[
 // the next group runs with full warps; a survivor's position is drawn again
 // (kept in shared memory it cost occupancy: 95 -> 127 us for 6.4 M
 // candidates).  Bound by issue (three draws a candidate, two exact divisions
-// a test) and by the latency of the mask reads.  A batch of few blocks lasts as
-// long as one block: 1,024 candidates a block below HULL_FEW, 4,096 above, where
-// a queue's groups fill more warps (whole calls drawing 0.02, 0.26 and 8.6 M
-// candidates with 1,024 and 4,096 throughout: 203 / 343, 263 / 422, 322 / 307 us).
+// a test) and by the latency of the mask reads.
 constexpr int HULL_THREADS = 256;
 
-template <int HB>
 __global__ void __launch_bounds__(HULL_THREADS)
 hull_accept_kernel(HullBox box, uint64_t first, int64_t count, const HullView *__restrict__ views,
                    int nv, const uint8_t *__restrict__ masks, float z_near,
                    uint32_t *__restrict__ bits, uint32_t *__restrict__ counts)
 {
-    __shared__ uint16_t s_q[2][HB];
-    __shared__ uint32_t s_bits[HB / 32];
+    __shared__ uint16_t s_q[2][HULL_BLOCK];
+    __shared__ uint32_t s_bits[HULL_BLOCK / 32];
     __shared__ uint32_t s_n[2];
-    const int64_t base = (int64_t)blockIdx.x * HB;
+    const int64_t base = (int64_t)blockIdx.x * HULL_BLOCK;
     const int lane = threadIdx.x & 31;
-    for (int j = threadIdx.x; j < HB / 32; j += HULL_THREADS) s_bits[j] = 0;
+    for (int j = threadIdx.x; j < HULL_BLOCK / 32; j += HULL_THREADS) s_bits[j] = 0;
     if (threadIdx.x < 2) s_n[threadIdx.x] = 0;
     __syncthreads();
-    int n = (int)(count - base < HB ? count - base : HB);
+    int n = (int)(count - base < HULL_BLOCK ? count - base : HULL_BLOCK);
     int cur = 0;
     bool all = true; // the first group tests every candidate, without a queue
     for (int v0 = 0; v0 < nv && n > 0;) {
@@ -143,8 +139,8 @@ hull_accept_kernel(HullBox box, uint64_t first, int64_t count, const HullView *_
         atomicOr(&s_bits[i >> 5], 1u << (i & 31));
     }
     __syncthreads();
-    for (int j = threadIdx.x; j < HB / 32; j += HULL_THREADS)
-        bits[(int64_t)blockIdx.x * (HB / 32) + j] = s_bits[j];
+    for (int j = threadIdx.x; j < HULL_BLOCK / 32; j += HULL_THREADS)
+        bits[(int64_t)blockIdx.x * (HULL_BLOCK / 32) + j] = s_bits[j];
     if (threadIdx.x == 0) counts[blockIdx.x] = (uint32_t)n;
 }
 
@@ -183,13 +179,12 @@ hull_scan_kernel(uint32_t *counts, int nb, unsigned long long *out)
 
 // Accepted candidates of rank < need go to out[done + rank]; the candidate
 // of rank need - 1 reports its index.  One thread per word of bits.
-template <int HB>
-__global__ void __launch_bounds__(HB / 32)
+__global__ void __launch_bounds__(HULL_BLOCK / 32)
 hull_take_kernel(HullBox box, uint64_t first, const uint32_t *__restrict__ bits,
                  const uint32_t *__restrict__ offsets, uint32_t need, float *__restrict__ out,
                  int64_t done, unsigned long long *last)
 {
-    constexpr int WORDS = HB / 32;
+    constexpr int WORDS = HULL_BLOCK / 32;
     __shared__ uint32_t s_w[WORDS / 32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int64_t word = (int64_t)blockIdx.x * WORDS + threadIdx.x;
@@ -256,26 +251,6 @@ void launch_consistency(const float *pos, int64_t n, const HullView *views, int 
     count_launches(1);
 }
 
-namespace {
-
-constexpr int64_t HULL_FEW = 1ll << 21;
-
-template <int HB>
-void run_batch(const HullBox &box, uint64_t first, int64_t count, const HullView *views, int nv,
-               const uint8_t *masks, float z_near, uint32_t *bits, uint32_t *counts, uint32_t need,
-               float *out, int64_t done, unsigned long long *result, cudaStream_t s)
-{
-    const unsigned nb = (unsigned)((count + HB - 1) / HB);
-    hull_accept_kernel<HB><<<nb, HULL_THREADS, 0, s>>>(box, first, count, views, nv, masks, z_near,
-                                                       bits, counts);
-    hull_scan_kernel<<<1, 1024, 0, s>>>(counts, (int)nb, result);
-    hull_take_kernel<HB><<<nb, HB / 32, 0, s>>>(box, first, bits, counts, need, out, done,
-                                                result + 1);
-    count_launches(3);
-}
-
-} // namespace
-
 void launch_hull_batch(uint64_t seed, uint64_t first, int64_t count, const float lo[3],
                        const float ext[3], const HullView *views, int nv, const uint8_t *masks,
                        float z_near, uint32_t *bits, uint32_t *counts, uint32_t need, float *out,
@@ -288,12 +263,13 @@ void launch_hull_batch(uint64_t seed, uint64_t first, int64_t count, const float
         box.lo[a] = lo[a];
         box.ex[a] = ext[a];
     }
-    if (count < HULL_FEW)
-        run_batch<HULL_BLOCK / 4>(box, first, count, views, nv, masks, z_near, bits, counts, need,
-                                  out, done, result, s);
-    else
-        run_batch<HULL_BLOCK>(box, first, count, views, nv, masks, z_near, bits, counts, need, out,
-                              done, result, s);
+    const unsigned nb = (unsigned)((count + HULL_BLOCK - 1) / HULL_BLOCK);
+    hull_accept_kernel<<<nb, HULL_THREADS, 0, s>>>(box, first, count, views, nv, masks, z_near,
+                                                   bits, counts);
+    hull_scan_kernel<<<1, 1024, 0, s>>>(counts, (int)nb, result);
+    hull_take_kernel<<<nb, HULL_BLOCK / 32, 0, s>>>(box, first, bits, counts, need, out, done,
+                                                    result + 1);
+    count_launches(3);
 }
 
 void launch_sh_normals(uint64_t seed, int64_t count, float *out, cudaStream_t s)
