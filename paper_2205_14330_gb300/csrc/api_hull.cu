@@ -2,6 +2,7 @@
 // check (Sec. 3.1 and the appendix).
 #include <algorithm>
 #include <cmath>
+#include <cstring>
 #include <vector>
 
 #include "api_internal.h"
@@ -12,13 +13,16 @@ namespace {
 
 constexpr uint64_t SH_STREAM = 0x5DEECE66Dull; // SH draws: stream seed ^ this
 
-// Views of the check on the device; validates cameras and z_near.
+// Views of the check on the device, `zeros` words of 0 behind them; validates
+// cameras and z_near.
 int upload_views(TempBufs &tb, const pbr_camera *cams, int32_t n_cams, float z_near,
-                 HullView **d_views, cudaStream_t s)
+                 HullView **d_views, cudaStream_t s, int zeros = 0)
 {
     if (!cams || n_cams < 1 || !(z_near >= 0.0f) || !std::isfinite(z_near))
         return set_error(PBR_ERR_INVALID_ARG, "consistency check: bad cameras or z_near");
-    std::vector<HullView> v(n_cams);
+    const size_t bytes = sizeof(HullView) * n_cams + sizeof(uint32_t) * zeros;
+    std::vector<HullView> v((bytes + sizeof(HullView) - 1) / sizeof(HullView));
+    std::memset(v.data(), 0, sizeof(HullView) * v.size());
     int64_t base = 0;
     for (int i = 0; i < n_cams; ++i) {
         const pbr_camera &c = cams[i];
@@ -36,8 +40,8 @@ int upload_views(TempBufs &tb, const pbr_camera *cams, int32_t n_cams, float z_n
         h.pix_base = base;
         base += (int64_t)c.width * c.height;
     }
-    PBR_TRY(tb.alloc(d_views, sizeof(HullView) * n_cams));
-    upload_small(*d_views, v.data(), sizeof(HullView) * n_cams, s);
+    PBR_TRY(tb.alloc(d_views, bytes));
+    upload_small(*d_views, v.data(), bytes, s);
     return PBR_OK;
 }
 
@@ -131,28 +135,29 @@ extern "C" int pbr_visual_hull_init(pbr_ctx *ctx, const float lo[3], const float
     PBR_CUDA(cudaSetDevice(ctx->device));
     TempBufs tb(s);
     HullView *views;
-    PBR_TRY(upload_views(tb, cams, n_cams, z_near, &views, s));
+    PBR_TRY(upload_views(tb, cams, n_cams, z_near, &views, s, HULL_CHUNKS));
     // Batches of candidates in counter order; the first n_target accepted.
     // A batch costs a host synchronisation, candidates beyond the last one
-    // taken cost their draws: the first batch allows for one candidate in 32
-    // accepted, the next ones for the share seen so far and a little more.
-    constexpr int64_t BATCH = 1ll << 24, LEAST = 1ll << 16;
+    // taken cost their draws, but for those the kernel sees to be beyond it: the
+    // first batch allows for one candidate in 32 accepted, the next ones for the
+    // share seen so far and a little more.
+    constexpr int64_t BATCH = HULL_BATCH, LEAST = 1ll << 16;
     auto sized = [&](double want) {
         const int64_t c = want < (double)BATCH ? (int64_t)want : BATCH;
-        return std::max(LEAST, (c + HULL_BLOCK - 1) / HULL_BLOCK * HULL_BLOCK);
+        return std::max(LEAST, (c + 4 * HULL_BLOCK - 1) / (4 * HULL_BLOCK) * (4 * HULL_BLOCK));
     };
     int64_t size = sized(32.0 * (double)n_target);
-    uint32_t *bits, *counts;
-    unsigned long long *result;
-    PBR_TRY(tb.alloc(&bits, (size_t)(BATCH / 8)));
-    PBR_TRY(tb.alloc(&counts, sizeof(uint32_t) * (BATCH / HULL_BLOCK)));
-    PBR_TRY(tb.alloc(&result, 2 * sizeof(unsigned long long)));
+    unsigned long long *result; // and counts, bits: one allocation
+    PBR_TRY(tb.alloc(&result, 2 * sizeof(unsigned long long) +
+                                  sizeof(uint32_t) * (BATCH / HULL_BLOCK) + BATCH / 8));
+    uint32_t *counts = (uint32_t *)(result + 2), *bits = counts + BATCH / HULL_BLOCK,
+             *found = (uint32_t *)(views + n_cams);
     int64_t done = 0, drawn = 0;
     while (done < n_target && drawn < max_candidates) {
         const int64_t cnt = std::min<int64_t>(size, max_candidates - drawn);
         const uint32_t need = (uint32_t)(n_target - done);
         launch_hull_batch(seed, (uint64_t)drawn, cnt, lo, ext, views, n_cams, masks, z_near, bits,
-                          counts, need, out_pos, done, result, s);
+                          counts, found, need, out_pos, done, result, s);
         unsigned long long got[2] = {0, 0};
         PBR_CUDA(cudaMemcpyAsync(got, result, sizeof got, cudaMemcpyDeviceToHost, s));
         PBR_CUDA(cudaStreamSynchronize(s));

@@ -80,7 +80,7 @@ __device__ __forceinline__ void candidate(const HullBox &b, uint64_t j, float p[
         p[a] = __fadd_rn(__fmul_rn(b.ex[a], uniform24(splitmix64(b.seed, 3 * j + a))), b.lo[a]);
 }
 
-// Acceptance of HULL_BLOCK candidates per block, as a bit each (candidate i
+// Acceptance of HB candidates per block, as a bit each (candidate i
 // of the batch in bit i & 31 of word i / 32) and a count per block.
 // A warp of candidates runs until its last one fails, so testing every view
 // at once keeps a warp for all views while a few lanes live (196 us for 4 M
@@ -90,22 +90,43 @@ __device__ __forceinline__ void candidate(const HullBox &b, uint64_t j, float p[
 // (kept in shared memory it cost occupancy: 95 -> 127 us for 6.4 M
 // candidates).  Bound by issue (three draws a candidate, two exact divisions
 // a test) and by the latency of the mask reads.
+// The batch allows for few accepted; where the masks take more, the blocks that
+// start after `need` have been found among lower candidates test none: found[c]
+// adds up what the blocks of chunk c accepted, and a block looks at the chunks
+// below its own.  The blocks that start at once stay: 2,048 candidates a block keep
+// them few (4,096: 307 us a call as 2,048 on 8.6 M candidates of which one in 54 is
+// accepted), 1,024 in batches below HULL_FEW, which last as long as one block.
+// 500k points, every candidate accepted, 16 views, a first batch of 16 M: 1647 ->
+// 489 us.
 constexpr int HULL_THREADS = 256;
 
+template <int HB>
 __global__ void __launch_bounds__(HULL_THREADS)
 hull_accept_kernel(HullBox box, uint64_t first, int64_t count, const HullView *__restrict__ views,
                    int nv, const uint8_t *__restrict__ masks, float z_near,
-                   uint32_t *__restrict__ bits, uint32_t *__restrict__ counts)
+                   uint32_t need, uint32_t *__restrict__ bits, uint32_t *__restrict__ counts,
+                   uint32_t *found)
 {
-    __shared__ uint16_t s_q[2][HULL_BLOCK];
-    __shared__ uint32_t s_bits[HULL_BLOCK / 32];
+    __shared__ uint16_t s_q[2][HB];
+    __shared__ uint32_t s_bits[HB / 32];
     __shared__ uint32_t s_n[2];
-    const int64_t base = (int64_t)blockIdx.x * HULL_BLOCK;
+    __shared__ bool s_enough;
+    const int64_t base = (int64_t)blockIdx.x * HB;
     const int lane = threadIdx.x & 31;
-    for (int j = threadIdx.x; j < HULL_BLOCK / 32; j += HULL_THREADS) s_bits[j] = 0;
+    for (int j = threadIdx.x; j < HB / 32; j += HULL_THREADS) s_bits[j] = 0;
     if (threadIdx.x < 2) s_n[threadIdx.x] = 0;
+    const uint32_t chunk = blockIdx.x / HULL_CHUNK;
+    if (threadIdx.x < 32) {
+        const uint32_t below = __reduce_add_sync(
+            0xffffffffu, (uint32_t)lane < chunk ? __ldcg(found + lane) : 0u);
+        if (lane == 0) s_enough = below >= need;
+    }
     __syncthreads();
-    int n = (int)(count - base < HULL_BLOCK ? count - base : HULL_BLOCK);
+    if (s_enough) { // its candidates' ranks are all beyond `need`
+        if (threadIdx.x == 0) counts[blockIdx.x] = 0;
+        return;
+    }
+    int n = (int)(count - base < HB ? count - base : HB);
     int cur = 0;
     bool all = true; // the first group tests every candidate, without a queue
     for (int v0 = 0; v0 < nv && n > 0;) {
@@ -139,14 +160,18 @@ hull_accept_kernel(HullBox box, uint64_t first, int64_t count, const HullView *_
         atomicOr(&s_bits[i >> 5], 1u << (i & 31));
     }
     __syncthreads();
-    for (int j = threadIdx.x; j < HULL_BLOCK / 32; j += HULL_THREADS)
-        bits[(int64_t)blockIdx.x * (HULL_BLOCK / 32) + j] = s_bits[j];
-    if (threadIdx.x == 0) counts[blockIdx.x] = (uint32_t)n;
+    for (int j = threadIdx.x; j < HB / 32; j += HULL_THREADS)
+        bits[(int64_t)blockIdx.x * (HB / 32) + j] = s_bits[j];
+    if (threadIdx.x == 0) {
+        counts[blockIdx.x] = (uint32_t)n;
+        if (n) atomicAdd(found + chunk, (uint32_t)n);
+    }
 }
 
-// One block: exclusive scan of the nb block counts in place, out[0] = total.
+// One block: exclusive scan of the nb block counts in place, out[0] = total; found
+// is 0 again.
 __global__ void __launch_bounds__(1024)
-hull_scan_kernel(uint32_t *counts, int nb, unsigned long long *out)
+hull_scan_kernel(uint32_t *counts, int nb, uint32_t *found, unsigned long long *out)
 {
     __shared__ uint32_t s_w[32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -175,17 +200,20 @@ hull_scan_kernel(uint32_t *counts, int nb, unsigned long long *out)
         __syncthreads();
     }
     if (threadIdx.x == 0) out[0] = run;
+    if (threadIdx.x < HULL_CHUNKS) found[threadIdx.x] = 0;
 }
 
 // Accepted candidates of rank < need go to out[done + rank]; the candidate
 // of rank need - 1 reports its index.  One thread per word of bits.
-__global__ void __launch_bounds__(HULL_BLOCK / 32)
+template <int HB>
+__global__ void __launch_bounds__(HB / 32)
 hull_take_kernel(HullBox box, uint64_t first, const uint32_t *__restrict__ bits,
                  const uint32_t *__restrict__ offsets, uint32_t need, float *__restrict__ out,
                  int64_t done, unsigned long long *last)
 {
-    constexpr int WORDS = HULL_BLOCK / 32;
+    constexpr int WORDS = HB / 32;
     __shared__ uint32_t s_w[WORDS / 32];
+    if (offsets[blockIdx.x] >= need) return; // whole block (untested ones among them)
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int64_t word = (int64_t)blockIdx.x * WORDS + threadIdx.x;
     uint32_t m = bits[word];
@@ -251,10 +279,35 @@ void launch_consistency(const float *pos, int64_t n, const HullView *views, int 
     count_launches(1);
 }
 
+namespace {
+
+constexpr int64_t HULL_FEW = 1ll << 21;
+static_assert(HULL_BATCH / (2 * HULL_BLOCK) <= HULL_CHUNK * HULL_CHUNKS &&
+                  HULL_FEW / HULL_BLOCK <= HULL_CHUNK * HULL_CHUNKS && HULL_CHUNKS <= 32,
+              "a lane per chunk");
+
+template <int HB>
+void run_batch(const HullBox &box, uint64_t first, int64_t count, const HullView *views, int nv,
+               const uint8_t *masks, float z_near, uint32_t *bits, uint32_t *counts,
+               uint32_t *found, uint32_t need, float *out, int64_t done,
+               unsigned long long *result, cudaStream_t s)
+{
+    const unsigned nb = (unsigned)((count + HB - 1) / HB);
+    hull_accept_kernel<HB><<<nb, HULL_THREADS, 0, s>>>(box, first, count, views, nv, masks, z_near,
+                                                       need, bits, counts, found);
+    hull_scan_kernel<<<1, 1024, 0, s>>>(counts, (int)nb, found, result);
+    hull_take_kernel<HB><<<nb, HB / 32, 0, s>>>(box, first, bits, counts, need, out, done,
+                                                result + 1);
+    count_launches(3);
+}
+
+} // namespace
+
 void launch_hull_batch(uint64_t seed, uint64_t first, int64_t count, const float lo[3],
                        const float ext[3], const HullView *views, int nv, const uint8_t *masks,
-                       float z_near, uint32_t *bits, uint32_t *counts, uint32_t need, float *out,
-                       int64_t done, unsigned long long *result, cudaStream_t s)
+                       float z_near, uint32_t *bits, uint32_t *counts, uint32_t *found,
+                       uint32_t need, float *out, int64_t done, unsigned long long *result,
+                       cudaStream_t s)
 {
     if (count <= 0 || need == 0) return;
     HullBox box;
@@ -263,13 +316,12 @@ void launch_hull_batch(uint64_t seed, uint64_t first, int64_t count, const float
         box.lo[a] = lo[a];
         box.ex[a] = ext[a];
     }
-    const unsigned nb = (unsigned)((count + HULL_BLOCK - 1) / HULL_BLOCK);
-    hull_accept_kernel<<<nb, HULL_THREADS, 0, s>>>(box, first, count, views, nv, masks, z_near,
-                                                   bits, counts);
-    hull_scan_kernel<<<1, 1024, 0, s>>>(counts, (int)nb, result);
-    hull_take_kernel<<<nb, HULL_BLOCK / 32, 0, s>>>(box, first, bits, counts, need, out, done,
-                                                    result + 1);
-    count_launches(3);
+    if (count < HULL_FEW)
+        run_batch<HULL_BLOCK>(box, first, count, views, nv, masks, z_near, bits, counts, found, need,
+                              out, done, result, s);
+    else
+        run_batch<2 * HULL_BLOCK>(box, first, count, views, nv, masks, z_near, bits, counts, found,
+                                  need, out, done, result, s);
 }
 
 void launch_sh_normals(uint64_t seed, int64_t count, float *out, cudaStream_t s)

@@ -344,15 +344,20 @@ void launch_consistency(const float *pos, int64_t n, const HullView *views, int 
                         const uint8_t *masks, float z_near, uint8_t *flags8, uint32_t *flags32,
                         cudaStream_t s);
 // Candidates first .. first + count - 1 of stream `seed` in the box lo + [0,
-// ext): the first `need` accepted ones go to out[done ..].  result[0] (device)
-// receives the number accepted, result[1] the batch index of the need-th one
-// when there is one.  Scratch: a bit per candidate (count rounded up to
-// HULL_BLOCK) and a count per HULL_BLOCK candidates.
-constexpr int HULL_BLOCK = 4096;
+// ext), at most HULL_BATCH: the first `need` accepted ones go to out[done ..].
+// result[0] (device) receives the number accepted (of those tested: blocks that
+// start when `need` have been found below them test none), result[1] the batch
+// index of the need-th one when there is one.  Scratch: a bit per candidate
+// (count rounded up to 2 HULL_BLOCK), a count per HULL_BLOCK candidates, and
+// HULL_CHUNKS words that are 0 between batches.
+constexpr int HULL_BLOCK = 1024; // the smaller of two block sizes
+constexpr int64_t HULL_BATCH = 1ll << 24;
+constexpr int HULL_CHUNK = 256, HULL_CHUNKS = 32; // blocks a chunk, chunks
 void launch_hull_batch(uint64_t seed, uint64_t first, int64_t count, const float lo[3],
                        const float ext[3], const HullView *views, int nv, const uint8_t *masks,
-                       float z_near, uint32_t *bits, uint32_t *counts, uint32_t need, float *out,
-                       int64_t done, unsigned long long *result, cudaStream_t s);
+                       float z_near, uint32_t *bits, uint32_t *counts, uint32_t *found,
+                       uint32_t need, float *out, int64_t done, unsigned long long *result,
+                       cudaStream_t s);
 // out[i] = standard normal number i of stream `seed` (Box-Muller).
 void launch_sh_normals(uint64_t seed, int64_t count, float *out, cudaStream_t s);
 
