@@ -369,6 +369,9 @@ int plan_and_capture(pbr_graph *g, cudaStream_t user_stream)
                         cudaMemcpyHostToDevice));
     PBR_CUDA(cudaMemcpy(g->d_view_list, L.view_list.data(), sizeof(int32_t) * L.view_list.size(),
                         cudaMemcpyHostToDevice));
+    // (a copy from pageable memory may return before it has reached the device,
+    // and replays run on streams that do not wait for the legacy one)
+    PBR_CUDA(cudaStreamSynchronize(nullptr));
     // 3. capture: forward, backward (from the caller's dL/dimage), training step
     PBR_TRY(capture(g, 0, g->cap_stream));
     if (want_bwd && (g->grad_rgb || g->target)) PBR_TRY(capture(g, 1, g->cap_stream));
@@ -464,6 +467,7 @@ extern "C" int pbr_graph_set_optimizer(pbr_graph *g, const pbr_optimizer_cfg *cf
     g->opt_allocs.push_back(g->d_opt);
     OptState st{{cfg->lr_pos, cfg->lr_sh, cfg->lr_opacity}, 0};
     PBR_CUDA(cudaMemcpy(g->d_opt, &st, sizeof st, cudaMemcpyHostToDevice));
+    PBR_CUDA(cudaStreamSynchronize(nullptr)); // as in plan_and_capture; the moments' zeroing
     g->opt = *cfg;
     g->has_opt = true;
     if (g->exec[3]) {
@@ -478,6 +482,7 @@ extern "C" int pbr_graph_set_lr(pbr_graph *g, float lr_pos, float lr_sh, float l
     if (!g || !g->d_opt) return set_error(PBR_ERR_INVALID_ARG, "no optimiser on this graph");
     const float lr[3] = {lr_pos, lr_sh, lr_opacity};
     PBR_CUDA(cudaMemcpy(g->d_opt, lr, sizeof lr, cudaMemcpyHostToDevice));
+    PBR_CUDA(cudaStreamSynchronize(nullptr)); // as in plan_and_capture
     return PBR_OK;
 }
 
