@@ -325,9 +325,9 @@ int pbr::build_layout(const pbr_points *scenes, int32_t n_scenes, const int32_t 
 // splats of amplitude 0.8, or the count cap, covering c of its 64 pixels; the
 // amplitudes are not known here), the batch is worth sum(v) / max(v) equal
 // blocks, and the line lies at c / r of them, r the mean cutoff radius in pixels.
-// c falls in proportion where a block's mean walk is below 64 hits (a warp's
-// start then counts: `line`) and, in most backwards, with a count cap below 28
-// (`layers`).  Streamed warps that count pairs end in atomics on one
+// c falls where a block's mean walk is below 64 hits (a warp's start then counts:
+// `line`) and with a count cap below 28 (`layers`), in the powers that fitted the
+// measurements.  Streamed warps that count pairs end in atomics on one
 // address, which half the warps halve: their line is lower.  The stored list's
 // forward is bound by its scattered writes, which more warps hide.  r comes from
 // the pair count: a point lists (1 + 2 r / tile_w)(1 + 2 r / tile_h) tiles, r = k
@@ -358,11 +358,12 @@ int pbr::build_layout(const pbr_points *scenes, int32_t n_scenes, const int32_t 
 //   500k, 4 x 800^2  131  165  189 / 190  369 / 363     244 / 321   455 / 485
 //   136k, 43 views   175   93  560 / 538 1226 / 1012    868 / 913 1461 / 1388
 //   272k, 33 views   477  128  855 / 785 1907 / 1554  1246 / 1329 2217 / 2046
-// Over 256 batches (1k to 1M points, 1 to 43 views of 64 to 1920 pixels a side,
-// amplitudes 0.05 to 0.8, some capped at 15) in up to three tile sizes and four
-// schedules the choice costs 0.7% against the better of the two on geometric
-// average, 2.4% in the worst schedule and phase; lists of very uneven length,
-// unknown here, would move the line (55% on the worst batch).
+// The lines were drawn over 716 batches (1k to 1M points, 1 to 144 views of 64 to
+// 1920 pixels a side, amplitudes 0.05 to 0.8, some capped at 15), in up to three
+// tile sizes and four schedules, 6,900 pairs of timings: the choice costs 0.7%
+// against the better of the two on geometric average and 1.3% at most in one
+// schedule and phase, single batches up to 44%: the lists' lengths, unknown here,
+// would tell them apart.
 RasterLanes pbr::raster_lanes(const HostLayout &L, const DevOpts &o, int64_t n_vis,
                               int64_t n_pairs, bool persistent, bool store, bool counted)
 {
@@ -397,14 +398,14 @@ RasterLanes pbr::raster_lanes(const HostLayout &L, const DevOpts &o, int64_t n_v
     const double x = sum / most * (sum_r / sum);
     const double line = std::min(1.0, sum / sum_blocks / 64.0), layers = deep / 28.0;
     if (persistent) {
-        r.fwd_two = x >= (store ? 2.4e6 : 225e3) * line;
-        r.bwd_two = x >= (store ? 104e3 : 104e3 * layers);
+        r.fwd_two = x >= (store ? 2.4e6 : 250e3) * line;
+        r.bwd_two = x >= (store ? 104e3 : 110e3 * layers);
     } else if (store) {
-        r.fwd_two = counted && x >= 200e3 * layers * line;
-        r.bwd_two = x >= 104e3 * layers;
+        r.fwd_two = counted && x >= 211e3 * layers * line;
+        r.bwd_two = x >= 100e3 * layers;
     } else {
-        r.fwd_two = x >= (counted ? 45e3 : 200e3) * line;
-        r.bwd_two = x >= (counted ? std::min(36e3, 112e3 * line) : 36e3);
+        r.fwd_two = x >= (counted ? 51e3 : 211e3) * layers * line;
+        r.bwd_two = x >= std::min(43e3, 150e3 * line);
     }
     return r;
 }
