@@ -120,7 +120,7 @@ typedef struct {
                               not faster: writing and reading the list costs
                               more than the reciprocal and multiply per
                               composited point it saves (on the 1M-point,
-                              64-view step, 34.0 against 24.3 ms), so callers
+                              64-view step, 27.8 against 20.4 ms), so callers
                               after speed set 1. */
     int32_t store_depth;   /* composited points per pixel whose T is kept in store
                               mode (0 = default 32; at most 255) */
@@ -549,6 +549,8 @@ int pbr_knn(pbr_ctx *ctx, const float *ref_pos, int64_t n_ref, const float *quer
  *   loss_dev: device double, overwritten with CD.
  *   grad2 [n2,3] (device, nullable): overwritten with dCD/dp2.
  *   nn12 [n1], nn21 [n2] (device int32, nullable): the nearest-point maps.
+ * A point at no finite distance to the other cloud (nn -1) makes CD and its own
+ * gradient NaN.
  * Errors: PBR_ERR_INVALID_ARG, PBR_ERR_OOM, PBR_ERR_CUDA.  Asynchronous. */
 int pbr_chamfer(pbr_ctx *ctx, const float *p1, int64_t n1, const float *p2, int64_t n2,
                 double *loss_dev, float *grad2, int32_t *nn12, int32_t *nn21,

@@ -473,7 +473,6 @@ __device__ __forceinline__ void add_stats(unsigned long long *stats, uint32_t a,
 // apart (A above B); their per-point arithmetic runs in packed fp32x2
 // operations (.x pixel A, .y pixel B), one instruction for both pixels.
 __device__ __forceinline__ float2 f2(float a) { return make_float2(a, a); }
-__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
 __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 

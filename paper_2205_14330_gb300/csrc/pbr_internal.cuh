@@ -362,7 +362,7 @@ void launch_hull_batch(uint64_t seed, uint64_t first, int64_t count, const float
 void launch_sh_normals(uint64_t seed, int64_t count, float *out, cudaStream_t s);
 
 // ---- raster (k_raster.cu)
-// Store mode (bwd_mode 2): T[k * n_pix + pix] = the transmittance pixel pix
+// Store mode (bwd_mode 2): T[pix * depth + k] = the transmittance pixel pix
 // had before its k-th composited point (k < depth), n[pix] = the points it
 // composited.  T == nullptr: recompute mode (the backward recovers T by
 // dividing by 1 - alpha back to front).
